@@ -200,6 +200,10 @@ __device__ __forceinline__ uint32_t hash_home(int32_t v, int lg) {
     return ((uint32_t)v * 0x9E3779B1u) >> (32 - lg);
 }
 
+// Path counts are held as 64-bit words: exact integers (C = unsigned long long)
+// until a count could reach 2^53, FP64 values (C = double) of the sample from
+// there on.  Every integer below 2^53 is an FP64 value, so the two give the same
+// sums, and the same choices, as long as no count reaches it.
 template <class C>
 __device__ __forceinline__ unsigned long long count_bits(C c) {
     if constexpr (std::is_floating_point<C>::value) return (unsigned long long)__double_as_longlong(c);
@@ -209,6 +213,19 @@ template <class C>
 __device__ __forceinline__ C count_of(unsigned long long b) {
     if constexpr (std::is_floating_point<C>::value) return __longlong_as_double((long long)b);
     else return b;
+}
+
+// Choices compare a running count with a real target in (0, total].  Integer
+// counts compare with its ceiling (the same outcome below 2^53): a warp-wide FP64
+// conversion or comparison holds the SM sub-partition's FP64 pipe for ~64 cycles.
+template <class C>
+__device__ __forceinline__ C reach_of(double target) {
+    if constexpr (std::is_floating_point<C>::value) return target;
+    else return __double2ull_ru(target);
+}
+
+__device__ __forceinline__ int ceil_log2(long long v) {  // v >= 1
+    return v > 1 ? 64 - __clzll(v - 1) : 0;
 }
 
 // one side's {word, count} of an entry: 16 aligned bytes, read in one request
@@ -264,9 +281,7 @@ __device__ __forceinline__ int64_t hash_find(const unsigned long long *tab, int 
     return -1;
 }
 
-// C = unsigned long long: exact counts (flagged at 2^53, products checked);
-// C = double: FP64 counts, the rerun of a phase whose counts passed 2^53.
-template <class C, bool HASH, int BT>
+template <bool HASH, int BT>
 __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / BT) k_bibfs(BiArgs a) {
     using W = Word<HASH>;
     // The heavy pass scans a meeting level against a Bloom filter of the other
@@ -282,7 +297,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
         h1 = (uint32_t)(m >> (64 - NBB));
         h2 = (uint32_t)(m >> 24) & ((1u << NBB) - 1u);
     };
-    constexpr bool FP = std::is_floating_point<C>::value;
+    using u64 = unsigned long long;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int nw = BT / 32;
     const int64_t n = a.n;
@@ -296,31 +311,44 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
     // claims of a level go to counter set it % 3; thread 0 clears set (it + 1) % 3
     // at the start of level it, two barriers after its last readers
     __shared__ int s_new[3], s_meet, s_full;
-    __shared__ C s_bkt[kMeetBuckets];
+    __shared__ u64 s_bkt[kMeetBuckets];
     __shared__ int s_sel;
-    __shared__ C s_base;
-    __shared__ unsigned long long s_off;  // the sample's path slot in the arena
-    __shared__ int32_t s_pick;            // a backtrack step's choice
+    __shared__ u64 s_base;
+    __shared__ u64 s_off;               // the sample's path slot in the arena
+    __shared__ u64 s_reach;             // the meeting choice's target
+    __shared__ int32_t s_pick;          // a backtrack step's choice: vertex, entry, count
     __shared__ long long s_pickp;
+    __shared__ u64 s_pickc;
+    // the two walks of a path (0 towards s, 1 towards t): vertex, entry, its count and
+    // level, next random step, next place in the path, and 1 = a long list to scan
+    // block-wide, 0 = at its end, -1 = no candidate
+    __shared__ int32_t s_ww[2], s_wk[2], s_wstate[2];
+    __shared__ uint32_t s_wl[2], s_wstep[2];
+    __shared__ long long s_wp[2];
+    __shared__ u64 s_wc[2];
+    __shared__ int s_ovf;                 // this block has raised the overflow flag
     __shared__ int s_tstar, s_tlast;      // segment of a long candidate list holding the choice
-    __shared__ C s_tpre;
+    __shared__ u64 s_tpre;
     __shared__ int32_t s_lv[2][kLvCap + 2];  // queue range of level L of a side: [s_lv[L], s_lv[L+1])
     __shared__ int32_t s_mj[kMeetCap];       // a reverse backtrack candidate's place in the list
     __shared__ int s_nc;
     __shared__ unsigned long long s_newcost[3];
     __shared__ int32_t s_mv[kMeetCap];
     __shared__ int32_t s_mp[kMeetCap];
-    __shared__ C s_mw[kMeetCap];
-    __shared__ C s_redc[nw];
+    __shared__ u64 s_mw[kMeetCap];
+    __shared__ u64 s_redc[nw];
     __shared__ unsigned long long s_best[nw];
     __shared__ int64_t s_fe[kFlat];  // first edge of each frontier vertex of a chunk
-    __shared__ C s_fs[kFlat];        // its path count
+    __shared__ u64 s_fs[kFlat];      // its path count
     __shared__ int64_t s_pre[kFlat + 1];  // prefix sums of the chunk's degrees
     __shared__ unsigned long long s_work[6];
     __shared__ long long s_wsum[nw];    // per-warp degree sums of a chunk
-    __shared__ double s_wcnt[nw];       // per-warp sums of a chunk's path counts
+    __shared__ int s_wbits[nw];         // per-warp largest count (bits)
     if (threadIdx.x < 6) s_work[threadIdx.x] = 0ull;
-    if (threadIdx.x == 0) s_tlast = -1;
+    if (threadIdx.x == 0) {
+        s_tlast = -1;
+        s_ovf = 0;
+    }
     unsigned long long n_add = 0ull;
     uint32_t ep_slot = HASH ? a.slot_epoch[slot] : 0u;
     const long long count = a.count_dev ? (long long)__ldcg(a.count_dev) : a.count;
@@ -390,8 +418,8 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
             pt = t;
         }
         if (threadIdx.x == 0) {
-            st_pair(&tab[4 * ps], W::make(s, ep, 0), count_bits(C(1)));
-            st_pair(&tab[4 * pt + 2], W::make(t, ep, 0), count_bits(C(1)));
+            st_pair(&tab[4 * ps], W::make(s, ep, 0), 1ull);
+            st_pair(&tab[4 * pt + 2], W::make(t, ep, 0), 1ull);
             queue0[0] = make_int2(s, (int)ps);
             queue1[0] = make_int2(t, (int)pt);
             s_new[0] = 0;
@@ -411,7 +439,11 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
         bool met = s != t, handed = false;
         // expected hits that try a level for its meeting layer first (lower where the
         // filter makes a scan that finds no member cheap)
-        double meet_hits = BT != kBiBlock ? kMeetOnlyHitsBloom : kMeetOnlyHits;
+        float meet_hits = BT != kBiBlock ? kMeetOnlyHitsBloom : kMeetOnlyHits;
+        // counts of the sides' frontiers are below 2^ub0, 2^ub1; fp: the sample's counts
+        // are FP64 values (block-uniform)
+        int ub0 = 1, ub1 = 1;
+        bool fp = false;
         int bloom_side = -1;                // the filter holds side bloom_side's first bloom_n vertices
         long long bloom_n = 0;
         if (met) {
@@ -496,6 +528,40 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                         tab = ntab;
                     }
                 }
+                // A new count is at most the sum of the frontier's counts, below 2^nb.
+                // Where that could pass 2^52 the frontier's largest count is looked up, and
+                // if it still could, the sample's counts become FP64 values here, before the
+                // level: integer counts never reach 2^53, so they need no check per addition
+                // (an FP64 sum over the frontier per level and FP64 comparisons kept that
+                // pipe 57% busy on Barabasi-Albert 30k), and a phase whose counts pass it is
+                // not run a second time in FP64 (estimate on a 300 x 300 grid 55.7 -> 28.5 ms,
+                // on Barabasi-Albert 200k with new states 3.90 -> 3.67 ms).
+                int nb = (x ? ub1 : ub0) + ceil_log2(hi - lo);
+                if (!fp && nb > 52) {
+                    const int2 *qf = x ? queue1 : queue0;
+                    const int fs = x ? 3 : 1;
+                    int mb = 0;
+                    for (long long q = lo + threadIdx.x; q < hi; q += BT)
+                        mb = max(mb, 64 - __clzll((long long)__ldcg(&tab[4ll * qf[q].y + fs])));
+                    mb = __reduce_max_sync(0xffffffffu, mb);
+                    if (lane == 0) s_wbits[warp] = mb;
+                    __syncthreads();
+                    for (int q = 0; q < nw; ++q) mb = max(mb, s_wbits[q]);
+                    nb = mb + ceil_log2(hi - lo);
+                    if (nb > 52) {
+                        fp = true;
+                        for (int z = 0; z < 2; ++z) {
+                            const int2 *qz = z ? queue1 : queue0;
+                            const long long qn = z ? qhi[1] : qhi[0];
+                            for (long long q = threadIdx.x; q < qn; q += BT) {
+                                u64 *c = &tab[4ll * qz[q].y + (z ? 3 : 1)];
+                                __stcg(c, count_bits<double>((double)__ldcg(c)));
+                            }
+                        }
+                    }
+                    __syncthreads();
+                }
+                const bool checked = fp && !s_ovf;  // (a hint: any thread's view serves)
                 const int cs = it % 3;
                 // a large level's claims leave the degrees to a pass after it (lazy_deg)
                 const bool lazy_deg = (x ? cost[1] : cost[0]) >= kLazyDegEdges;
@@ -538,7 +604,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                 // level.  A claim swaps the whole {word, count} pair, so it also sets the
                 // count to the claiming parent's and counts never need clearing: a count
                 // is read only where its word carries the sample's epoch.
-                auto resolve = [&](Pre &r, const C su, const bool checked, const bool meet_only) {
+                auto resolve = [&](Pre &r, const u64 su, const bool meet_only) {
                     if (HASH && s_full) return;  // the sample goes to the direct store
                     const int32_t v = r.v;
                     const unsigned long long want = W::make(v, ep, nl);
@@ -569,7 +635,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                             }
                             if (meet_only && !yc) break;  // not in the meeting layer: left to a full pass
                             unsigned long long pw, pc;
-                            cas_pair(&tab[4 * p + xs], ow, oc, want, count_bits(su), pw, pc);
+                            cas_pair(&tab[4 * p + xs], ow, oc, want, su, pw, pc);
                             if (pw == ow && pc == oc) {
                                 won = true;
                                 meet = yc;
@@ -609,12 +675,20 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     }
                     if (a.work && (at || won)) ++n_add;
                     if (at) {
-                        C *cp = reinterpret_cast<C *>(&tab[4 * p + xs + 1]);
-                        if (checked) {  // counts may pass 2^53: find the addition that does
-                            const C o = atomicAdd(cp, su);
-                            if ((double)(o + su) >= kTwo53) atomicOr(a.status, DEV_SIGMA_OVERFLOW);
-                        } else {
+                        u64 *cp = &tab[4 * p + xs + 1];
+                        if (!fp) {
                             atomicAdd(cp, su);  // (no result waited for)
+                        } else {
+                            double *dp = reinterpret_cast<double *>(cp);
+                            const double ds = count_of<double>(su);
+                            if (checked) {  // find the addition that passes 2^53, until one is flagged
+                                if (atomicAdd(dp, ds) + ds >= kTwo53) {
+                                    atomicOr(a.status, DEV_SIGMA_OVERFLOW);
+                                    s_ovf = 1;
+                                }
+                            } else {
+                                atomicAdd(dp, ds);
+                            }
                         }
                     }
                 };
@@ -625,8 +699,8 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                 // which is all a level that meets needs (nothing reads its other
                 // vertices).  If it holds none the level is scanned again in full.
                 bool meet_only = a.gid == nullptr &&
-                                 (double)(x ? cost[1] : cost[0]) * (double)(x ? qhi[0] : qhi[1]) >=
-                                     meet_hits * (double)a.n;
+                                 (float)(x ? cost[1] : cost[0]) * (float)(x ? qhi[0] : qhi[1]) >=
+                                     meet_hits * (float)a.n;
                 if (BLOOM && meet_only) {
                     // the other side's vertices into the filter (it only grows: a side's
                     // queue lists every vertex it reached, in order)
@@ -651,10 +725,6 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     }
                 }
                 for (;;) {
-                    // every count of the new level is at most the sum of the frontier's
-                    // counts loaded so far (fcnt, FP64): below 2^52 no count can reach 2^53,
-                    // so the count additions need not wait for their results
-                    double fcnt = 0.0;
                     // the level's edges spread evenly over the block, kFlat frontier vertices
                     // at a time (a hub's adjacency is not left to one warp): the block loads
                     // the chunk, a few vertices per thread with their loads in flight
@@ -666,7 +736,6 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                             constexpr int per = kFlat >= BT ? kFlat / BT : 1;
                             int64_t loc[per];
                             int64_t tot = 0;
-                            double csum = 0.0;  // the chunk's path counts
     #pragma unroll
                             for (int r = 0; r < per; ++r) {
                                 const int k = (int)threadIdx.x * per + r;
@@ -675,9 +744,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                     const int2 qe = qx[c0 + k];
                                     const int64_t e0 = px[qe.x];
                                     s_fe[k] = e0;
-                                    const C fs = count_of<C>(__ldcg(&tab[4ll * qe.y + xs + 1]));
-                                    s_fs[k] = fs;
-                                    csum += (double)fs;
+                                    s_fs[k] = __ldcg(&tab[4ll * qe.y + xs + 1]);
                                     dg = px[qe.x + 1] - e0;
                                 }
                                 loc[r] = tot;
@@ -690,13 +757,9 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 if (lane >= o) incl += t2;
                             }
                             if (lane == 31) s_wsum[warp] = incl;
-    #pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) csum += __shfl_xor_sync(0xffffffffu, csum, o);
-                            if (lane == 0) s_wcnt[warp] = csum;
                             __syncthreads();
                             int64_t first = incl - tot;
                             for (int q = 0; q < warp; ++q) first += s_wsum[q];
-                            for (int q = 0; q < nw; ++q) fcnt += s_wcnt[q];
     #pragma unroll
                             for (int r = 0; r < per; ++r) {
                                 const int k = (int)threadIdx.x * per + r;
@@ -750,7 +813,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 for (int b = 0; b < kMeetBatch; ++b) {
                                     if (vv[b] < 0) continue;
                                     Pre pr = prefetch(vv[b]);
-                                    resolve(pr, s_fs[kk[b]], fcnt >= 0x1p52, true);
+                                    resolve(pr, s_fs[kk[b]], true);
                                 }
                             }
                         } else {
@@ -769,7 +832,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                     if (vv[b] >= 0) pr[b] = prefetch(vv[b]);
     #pragma unroll
                                 for (int b = 0; b < EB; ++b)
-                                    if (vv[b] >= 0) resolve(pr[b], s_fs[kk[b]], fcnt >= 0x1p52, meet_only);
+                                    if (vv[b] >= 0) resolve(pr[b], s_fs[kk[b]], meet_only);
                             }
                         }
                         if (c0 + kFlat < hi) __syncthreads();  // the chunk's shared arrays are reused
@@ -778,7 +841,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     __syncthreads();
                     if (s_meet || (HASH && s_full)) break;  // (the same in every thread after the barrier)
                     meet_only = false;  // no member: the level in full (nothing was claimed)
-                    meet_hits *= 8.0;   // (targets are not uniform: on grids the balls meet late)
+                    meet_hits *= 8.0f;  // (targets are not uniform: on grids the balls meet late)
                     __syncthreads();    // the chunk's shared arrays are reloaded
                 }
                 if (a.work && ne) atomicAdd(&s_work[0], ne);
@@ -814,11 +877,13 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     qhi[1] = nh;
                     lev[1] = nl;
                     cost[1] = nc;
+                    ub1 = nb;
                 } else {
                     qlo[0] = hi;
                     qhi[0] = nh;
                     lev[0] = nl;
                     cost[0] = nc;
+                    ub0 = nb;
                 }
                 if (s_meet) {
                     met = true;
@@ -847,217 +912,310 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
         } else {
             // meeting layer: the members of the last level of side x (vertices the
             // other side holds), listed as they were claimed; weights sigma_s sigma_t,
-            // kept in shared memory when they fit
+            // kept in shared memory when they fit.  Integer weights where their sum
+            // stays below 2^53, else FP64 (flagged where one or the sum reaches it).
             const int nm = s_meet;
-            auto weight = [&](const int2 qe) -> C {
-                return count_of<C>(__ldcg(&tab[4ll * qe.y + 1])) * count_of<C>(__ldcg(&tab[4ll * qe.y + 3]));
-            };
-            C part = C(0);
-            for (int m = threadIdx.x; m < nm; m += BT) {
-                const int2 qe = memb[m];
-                const C a0 = count_of<C>(__ldcg(&tab[4ll * qe.y + 1]));
-                const C a1 = count_of<C>(__ldcg(&tab[4ll * qe.y + 3]));
-                const C p = a0 * a1;
-                if ((double)a0 * (double)a1 >= kTwo53) atomicOr(a.status, DEV_SIGMA_OVERFLOW);
-                part += p;
-                if (m < kMeetCap) {
-                    s_mv[m] = qe.x;
-                    s_mp[m] = qe.y;
-                    s_mw[m] = p;
-                }
-            }
-            const C sst = block_sum<BT>(part, s_redc);
-            if (threadIdx.x == 0 && (double)sst >= kTwo53) atomicOr(a.status, DEV_SIGMA_OVERFLOW);
-            const double target = __dmul_rn(uniform_at(a.seed, (uint64_t)i, a.tag, 0), (double)sst);
-            if (a.work && threadIdx.x == 0 && nm > kMeetCap) s_work[3] += 1ull << 32;  // large layers (high word)
-            int32_t vm;
-            int64_t pm;
-            if (nm <= kMeetCap) {
-                // member j qualifies when the weights of the members with ids <= its
-                // own reach the target; the meeting vertex is the smallest such id
-                unsigned long long best = ~0ull;  // vertex << 32 | entry
-                for (int j = threadIdx.x; j < nm; j += BT) {
-                    const int32_t vj = s_mv[j];
-                    C pre = C(0);
-                    for (int k2 = 0; k2 < nm; ++k2)
-                        if (s_mv[k2] <= vj) pre += s_mw[k2];
-                    if ((double)pre >= target)
-                        best = min(best, ((unsigned long long)(uint32_t)vj << 32) | (uint32_t)s_mp[j]);
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
-                __syncthreads();
-                if (lane == 0) s_best[warp] = best;
-                __syncthreads();
-                unsigned long long bk = s_best[0];
-                for (int q = 1; q < nw; ++q) bk = min(bk, s_best[q]);
-                if (bk == ~0ull) {  // (FP64 counts) no member reaches the target: the last one takes it
-                    unsigned long long lk = 0ull;
-                    for (int j = 0; j < nm; ++j)
-                        lk = max(lk, ((unsigned long long)(uint32_t)s_mv[j] << 32) | (uint32_t)s_mp[j]);
-                    bk = lk;
-                }
-                vm = (int32_t)(bk >> 32);
-                pm = (int64_t)(uint32_t)bk;
-            } else {
-                // a large layer: the first id whose prefix sum (members in id order)
-                // reaches the target, narrowed in rounds of kMeetBuckets id buckets: the
-                // members' weights are summed per bucket in shared memory, the first
-                // bucket whose running total reaches the target holds the answer, and
-                // the next round splits that bucket (exact integer sums, so the same id
-                // as a sequential scan; three rounds for 2^30 ids)
-                int64_t lo_id = 0, span = n;
-                C base = C(0);  // weight of the members below lo_id
-                while (span > 1) {
-                    const int64_t wb = (span + kMeetBuckets - 1) / kMeetBuckets;
-                    for (int b = threadIdx.x; b < kMeetBuckets; b += BT) s_bkt[b] = C(0);
-                    __syncthreads();
-                    for (int m = threadIdx.x; m < nm; m += BT) {
-                        const int2 qe = memb[m];
-                        if (qe.x >= lo_id && qe.x < lo_id + span) atomicAdd(&s_bkt[(qe.x - lo_id) / wb], weight(qe));
+            int32_t vm = 0;
+            int64_t pm = 0;
+            auto choose_meeting = [&](auto zero) {
+                using C = decltype(zero);
+                constexpr bool FP = std::is_floating_point<C>::value;
+                auto side_count = [&](u64 b) -> C {
+                    if constexpr (FP) return fp ? count_of<double>(b) : (double)b;
+                    else return b;
+                };
+                auto weight = [&](const int2 qe) -> C {
+                    return side_count(__ldcg(&tab[4ll * qe.y + 1])) * side_count(__ldcg(&tab[4ll * qe.y + 3]));
+                };
+                C *const mw = reinterpret_cast<C *>(s_mw), *const redc = reinterpret_cast<C *>(s_redc);
+                C part = C(0);
+                for (int m = threadIdx.x; m < nm; m += BT) {
+                    const int2 qe = memb[m];
+                    const C p = weight(qe);
+                    if constexpr (FP) {
+                        if (p >= kTwo53) atomicOr(a.status, DEV_SIGMA_OVERFLOW);
                     }
-                    __syncthreads();
-                    if (warp == 0) {
-                        constexpr int per = kMeetBuckets / 32;
-                        C lsum = C(0);
-                        for (int j = 0; j < per; ++j) lsum += s_bkt[lane * per + j];
-                        C incl = lsum;
+                    part += p;
+                    if (m < kMeetCap) {
+                        s_mv[m] = qe.x;
+                        s_mp[m] = qe.y;
+                        mw[m] = p;
+                    }
+                }
+                const C sst = block_sum<BT>(part, redc);
+                if (threadIdx.x == 0) {
+                    if constexpr (FP) {
+                        if (sst >= kTwo53) atomicOr(a.status, DEV_SIGMA_OVERFLOW);
+                    }
+                    s_reach = count_bits<C>(
+                        reach_of<C>(__dmul_rn(uniform_at(a.seed, (uint64_t)i, a.tag, 0), (double)sst)));
+                    if (a.work && nm > kMeetCap) s_work[3] += 1ull << 32;  // large layers (high word)
+                }
+                __syncthreads();
+                const C target = count_of<C>(s_reach);
+                if (nm <= kMeetCap) {
+                    // member j qualifies when the weights of the members with ids <= its
+                    // own reach the target; the meeting vertex is the smallest such id
+                    u64 best = ~0ull;  // vertex << 32 | entry
+                    for (int j = threadIdx.x; j < nm; j += BT) {
+                        const int32_t vj = s_mv[j];
+                        C pre = C(0);
+                        for (int k2 = 0; k2 < nm; ++k2)
+                            if (s_mv[k2] <= vj) pre += mw[k2];
+                        if (pre >= target) best = min(best, ((u64)(uint32_t)vj << 32) | (uint32_t)s_mp[j]);
+                    }
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const C t2 = __shfl_up_sync(0xffffffffu, incl, o);
-                            if (lane >= o) incl += t2;
+                    for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
+                    if (lane == 0) s_best[warp] = best;
+                    __syncthreads();
+                    u64 bk = s_best[0];
+                    for (int q = 1; q < nw; ++q) bk = min(bk, s_best[q]);
+                    if (bk == ~0ull) {  // (FP64 counts) no member reaches the target: the last one takes it
+                        u64 lk = 0ull;
+                        for (int j = 0; j < nm; ++j)
+                            lk = max(lk, ((u64)(uint32_t)s_mv[j] << 32) | (uint32_t)s_mp[j]);
+                        bk = lk;
+                    }
+                    vm = (int32_t)(bk >> 32);
+                    pm = (int64_t)(uint32_t)bk;
+                } else {
+                    // a large layer: the first id whose prefix sum (members in id order)
+                    // reaches the target, narrowed in rounds of kMeetBuckets id buckets: the
+                    // members' weights are summed per bucket in shared memory, the first
+                    // bucket whose running total reaches the target holds the answer, and
+                    // the next round splits that bucket (exact integer sums, so the same id
+                    // as a sequential scan; three rounds for 2^30 ids)
+                    C *const bkt = reinterpret_cast<C *>(s_bkt);
+                    int64_t lo_id = 0, span = n;
+                    C base = C(0);  // weight of the members below lo_id
+                    while (span > 1) {
+                        const int64_t wb = (span + kMeetBuckets - 1) / kMeetBuckets;
+                        for (int b = threadIdx.x; b < kMeetBuckets; b += BT) bkt[b] = C(0);
+                        __syncthreads();
+                        for (int m = threadIdx.x; m < nm; m += BT) {
+                            const int2 qe = memb[m];
+                            if (qe.x >= lo_id && qe.x < lo_id + span) atomicAdd(&bkt[(qe.x - lo_id) / wb], weight(qe));
                         }
-                        const unsigned hit = __ballot_sync(0xffffffffu, (double)(base + incl) >= target);
-                        const unsigned nz = __ballot_sync(0xffffffffu, lsum > C(0));
-                        // FP64 counts past 2^53 may leave every total just below the target:
-                        // the last bucket with weight then takes the remainder
-                        const int L0 = hit ? __ffs(hit) - 1 : (nz ? 31 - __clz(nz) : 0);
-                        if (lane == L0) {  // the bucket within this lane's range, and the total below it
-                            C run = base + (incl - lsum), below = run;
-                            int bsel = 0;
-                            for (int j = 0; j < per; ++j) {
-                                const C bw = s_bkt[L0 * per + j];
-                                if (bw == C(0)) continue;
-                                bsel = j;
-                                below = run;
-                                run += bw;
-                                if (hit && (double)run >= target) break;
+                        __syncthreads();
+                        if (warp == 0) {
+                            constexpr int per = kMeetBuckets / 32;
+                            C lsum = C(0);
+                            for (int j = 0; j < per; ++j) lsum += bkt[lane * per + j];
+                            C incl = lsum;
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const C t2 = __shfl_up_sync(0xffffffffu, incl, o);
+                                if (lane >= o) incl += t2;
                             }
-                            s_sel = L0 * per + bsel;
-                            s_base = below;
+                            const unsigned hit = __ballot_sync(0xffffffffu, base + incl >= target);
+                            const unsigned nz = __ballot_sync(0xffffffffu, lsum > C(0));
+                            // FP64 counts past 2^53 may leave every total just below the target:
+                            // the last bucket with weight then takes the remainder
+                            const int L0 = hit ? __ffs(hit) - 1 : (nz ? 31 - __clz(nz) : 0);
+                            if (lane == L0) {  // the bucket within this lane's range, and the total below it
+                                C run = base + (incl - lsum), below = run;
+                                int bsel = 0;
+                                for (int j = 0; j < per; ++j) {
+                                    const C bw = bkt[L0 * per + j];
+                                    if (bw == C(0)) continue;
+                                    bsel = j;
+                                    below = run;
+                                    run += bw;
+                                    if (hit && run >= target) break;
+                                }
+                                s_sel = L0 * per + bsel;
+                                s_base = count_bits<C>(below);
+                            }
                         }
+                        __syncthreads();
+                        const int64_t nlo = lo_id + (int64_t)s_sel * wb;
+                        span = min(wb, lo_id + span - nlo);
+                        lo_id = nlo;
+                        base = count_of<C>(s_base);
+                        __syncthreads();
                     }
-                    __syncthreads();
-                    const int64_t nlo = lo_id + (int64_t)s_sel * wb;
-                    span = min(wb, lo_id + span - nlo);
-                    lo_id = nlo;
-                    base = s_base;
-                    __syncthreads();
+                    vm = (int32_t)lo_id;
+                    if constexpr (HASH) pm = hash_find(tab, lg, vm, ep);
+                    else pm = vm;
                 }
-                vm = (int32_t)lo_id;
-                if constexpr (HASH) pm = hash_find(tab, lg, vm, ep);
-                else pm = vm;
-            }
+            };
+            if (fp || ub0 + ub1 + ceil_log2(nm) > 52) choose_meeting(0.0);
+            else choose_meeting(0ull);
             if (a.trace && threadIdx.x == 0) t_meet = globaltimer_ns();
             // the path: the meeting vertex, then the s side backtracked from it, then
             // the t side.  A backtrack step scans the candidates (in-neighbours towards
             // s, out-neighbours towards t) in adjacency order for the first one one level
-            // closer whose running count reaches u sigma(w): one warp for short lists; the
-            // whole block for long ones (hubs), in two passes -- every thread sums a
-            // contiguous segment, a block scan of the sums finds the segment where the
-            // running count reaches the target, one warp scans that segment.
-            {
-                const uint32_t la = W::level(__ldcg(&tab[4 * pm]));
-                const uint32_t lb = W::level(__ldcg(&tab[4 * pm + 2]));
+            // closer whose running count reaches u sigma(w).  The two walks are independent
+            // (the s side takes as many random steps as the meeting vertex's level), so
+            // warp 0 walks towards s and warp 1 towards t, without block barriers, until
+            // both end or wait at a long list (a hub), which the whole block scans.
+            auto backtrack = [&](auto zero) {
+                using C = decltype(zero);
+                constexpr bool FP = std::is_floating_point<C>::value;
+                u64 wa, ca, wb, cb;
+                ld_pair(&tab[4 * pm], wa, ca);
+                ld_pair(&tab[4 * pm + 2], wb, cb);
+                const uint32_t la = W::level(wa), lb = W::level(wb);
                 const int32_t len = (int32_t)(la + lb) - 1;
+                const int32_t k0 = (vm != s && vm != t) ? 1 : 0;
                 if (threadIdx.x == 0) {
-                    const unsigned long long o = atomicAdd(a.arena_top, (unsigned long long)len);
+                    const u64 o = atomicAdd(a.arena_top, (u64)len);
                     if ((int64_t)(o + len) > a.arena_cap) atomicOr(a.status, DEV_ARENA_OVERFLOW);
                     a.ilen[i] = len;
                     a.path_off[i] = (long long)o;
                     s_off = o;
-                    if (vm != s && vm != t) {
+                    if (k0) {
                         if ((int64_t)(o + len) <= a.arena_cap) a.arena[o] = vm;
                         atomicAdd(&a.cnt[vm], 1ull);
                     }
+                    for (int z = 0; z < 2; ++z) {
+                        s_ww[z] = vm;
+                        s_wp[z] = pm;
+                        s_wl[z] = z ? lb : la;
+                        s_wc[z] = z ? cb : ca;
+                        s_wstep[z] = z ? la + 1 : 1;
+                        s_wk[z] = k0 + (z && la > 0 ? (int32_t)la - 1 : 0);
+                    }
                 }
                 __syncthreads();
-                const unsigned long long off = s_off;
+                const u64 off = s_off;
                 const bool store = (int64_t)(off + len) <= a.arena_cap;
-                int32_t k = (vm != s && vm != t) ? 1 : 0;
-                uint32_t step = 1;
-                for (int z = 0; z < 2; ++z) {
-                    // towards s: predecessors over in-edges; towards t: successors over out-edges
-                    const int64_t *bp = z == 0 ? a.irp : a.rp;
-                    const int32_t *bc = z == 0 ? a.icol : a.col;
-                    const int zs = z ? 2 : 0;
-                    const int32_t endz = z == 0 ? s : t;
-                    int32_t w = vm;
-                    int64_t pw = pm;
-                    bool bad = false;
-                    while (w != endz) {  // (the same in every thread)
-                        const uint32_t lw = W::level(__ldcg(&tab[4 * pw + zs]));
-                        const double tg = __dmul_rn(uniform_at(a.seed, (uint64_t)i, a.tag, step),
-                                                    (double)count_of<C>(__ldcg(&tab[4 * pw + zs + 1])));
-                        const int64_t e0 = bp[w], e1 = bp[w + 1];
-                        // the count of candidate e if it lies one level closer, else 0
-                        auto cand = [&](int64_t e, int32_t &pv, int64_t &pp) -> C {
-                            pv = bc[e];
-                            if constexpr (HASH) pp = hash_find(tab, lg, pv, ep);
-                            else pp = pv;
-                            if (pp < 0) return C(0);
-                            unsigned long long lw2, lc2;
-                            ld_pair(&tab[4 * pp + zs], lw2, lc2);
-                            return (W::current(lw2, ep) && W::level(lw2) + 1 == lw) ? count_of<C>(lc2) : C(0);
-                        };
-                        // one warp scans [b0, b1) from running count c0: first lane whose running
-                        // count reaches tg, else (FP64 counts) the last candidate
-                        auto warp_scan = [&](int64_t b0, int64_t b1, C c0) {
-                            C carry = c0;
-                            int32_t pick = -1, last = -1;
-                            int64_t pickp = -1, lastp = -1;
-                            for (int64_t eb = b0; eb < b1 && pick < 0; eb += 32) {
-                                const int64_t e = eb + lane;
-                                int32_t pv = -1;
-                                int64_t pp = -1;
-                                const C val = e < b1 ? cand(e, pv, pp) : C(0);
-                                C cum = val;
+                // side z = 0, towards s: predecessors over in-edges; 1, towards t: successors over out-edges
+                auto row_of = [&](int z) { return z == 0 ? a.irp : a.rp; };
+                auto adj_of = [&](int z) { return z == 0 ? a.icol : a.col; };
+                // the count of candidate e of side z if it lies at level lw - 1, else 0
+                auto cand = [&](int z, uint32_t lw, int64_t e, int32_t &pv, int64_t &pp) -> C {
+                    pv = adj_of(z)[e];
+                    if constexpr (HASH) pp = hash_find(tab, lg, pv, ep);
+                    else pp = pv;
+                    if (pp < 0) return C(0);
+                    u64 lw2, lc2;
+                    ld_pair(&tab[4 * pp + (z ? 2 : 0)], lw2, lc2);
+                    return (W::current(lw2, ep) && W::level(lw2) + 1 == lw) ? count_of<C>(lc2) : C(0);
+                };
+                auto target_of = [&](uint32_t step, C cw) -> C {
+                    return reach_of<C>(__dmul_rn(uniform_at(a.seed, (uint64_t)i, a.tag, step), (double)cw));
+                };
+                // one warp scans [b0, b1) from running count c0 for the first candidate whose
+                // running count reaches tg, else (FP64 counts past 2^53 may round the running
+                // sum just below u sigma(w)) the last candidate: vertex (-1: none), entry, count
+                auto warp_scan = [&](int z, uint32_t lw, int64_t b0, int64_t b1, C c0, C tg, int32_t &pick,
+                                     int64_t &pickp, C &pickc) {
+                    C carry = c0;
+                    pick = -1;
+                    pickp = -1;
+                    pickc = C(0);
+                    int32_t last = -1;
+                    int64_t lastp = -1;
+                    C lastc = C(0);
+                    for (int64_t eb = b0; eb < b1 && pick < 0; eb += 32) {
+                        const int64_t e = eb + lane;
+                        int32_t pv = -1;
+                        int64_t pp = -1;
+                        const C val = e < b1 ? cand(z, lw, e, pv, pp) : C(0);
+                        const unsigned cm = __ballot_sync(0xffffffffu, val > C(0));
+                        if (!cm) continue;
+                        C cum = val;
 #pragma unroll
-                                for (int o = 1; o < 32; o <<= 1) {
-                                    const C t2 = __shfl_up_sync(0xffffffffu, cum, o);
-                                    if (lane >= o) cum += t2;
-                                }
-                                cum += carry;
-                                const unsigned hit = __ballot_sync(0xffffffffu, val > C(0) && (double)cum >= tg);
-                                if (hit) {
-                                    pick = __shfl_sync(0xffffffffu, pv, __ffs(hit) - 1);
-                                    pickp = __shfl_sync(0xffffffffu, pp, __ffs(hit) - 1);
-                                }
-                                const unsigned cm = __ballot_sync(0xffffffffu, val > C(0));
-                                if (cm) {
-                                    last = __shfl_sync(0xffffffffu, pv, 31 - __clz(cm));
-                                    lastp = __shfl_sync(0xffffffffu, pp, 31 - __clz(cm));
-                                }
-                                carry = __shfl_sync(0xffffffffu, cum, 31);
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const C t2 = __shfl_up_sync(0xffffffffu, cum, o);
+                            if (lane >= o) cum += t2;
+                        }
+                        cum += carry;
+                        const unsigned hit = __ballot_sync(0xffffffffu, val > C(0) && cum >= tg);
+                        const int src = hit ? __ffs(hit) - 1 : 31 - __clz(cm);
+                        const int32_t v1 = __shfl_sync(0xffffffffu, pv, src);
+                        const int64_t p1 = __shfl_sync(0xffffffffu, pp, src);
+                        const C c1 = __shfl_sync(0xffffffffu, val, src);
+                        if (hit) {
+                            pick = v1;
+                            pickp = p1;
+                            pickc = c1;
+                        } else if (FP) {
+                            last = v1;
+                            lastp = p1;
+                            lastc = c1;
+                        }
+                        carry = __shfl_sync(0xffffffffu, cum, 31);
+                    }
+                    if (FP && pick < 0) {
+                        pick = last;
+                        pickp = lastp;
+                        pickc = lastc;
+                    }
+                };
+                auto failed = [&](int z, uint32_t step, int64_t deg, int32_t w, uint32_t lw) {
+                    atomicOr(a.status, DEV_BAD_PATH);
+                    if (a.trace) {  // where the path ended without a candidate
+                        a.trace[8 * i + 6] = (deg <= kBackWarp ? 1ull : 2ull) | ((u64)z << 4) | ((u64)step << 8) |
+                                             ((u64)deg << 32);
+                        a.trace[8 * i + 7] = ((u64)(uint32_t)w << 32) | lw;
+                    }
+                };
+                for (;;) {
+                    if (warp < 2) {
+                        const int z = warp;
+                        const int32_t endz = z == 0 ? s : t;
+                        int32_t w = s_ww[z], k = s_wk[z], state = 0;
+                        int64_t pw = s_wp[z];
+                        uint32_t lw = s_wl[z], step = s_wstep[z];
+                        C cw = count_of<C>(s_wc[z]);
+                        while (w != endz) {
+                            const int64_t e0 = row_of(z)[w], e1 = row_of(z)[w + 1];
+                            if (e1 - e0 > kBackWarp) {
+                                state = 1;
+                                break;
                             }
-                            // FP64 counts past 2^53 may round the running sum just below u sigma(w):
-                            // the last candidate then takes the remainder
-                            if (pick < 0 && FP) {
-                                pick = last;
-                                pickp = lastp;
+                            int32_t pick;
+                            int64_t pickp;
+                            C pickc;
+                            warp_scan(z, lw, e0, e1, C(0), target_of(step, cw), pick, pickp, pickc);
+                            if (pick < 0) {
+                                if (lane == 0) failed(z, step, e1 - e0, w, lw);
+                                state = -1;
+                                break;
                             }
-                            if (lane == 0) {
-                                s_pick = pick;
-                                s_pickp = pickp;
+                            if (pick != endz) {
+                                if (lane == 0) {
+                                    if (store && k < len) a.arena[off + k] = pick;
+                                    atomicAdd(&a.cnt[pick], 1ull);
+                                }
+                                ++k;
                             }
-                        };
+                            w = pick;
+                            pw = pickp;
+                            cw = pickc;
+                            --lw;
+                            ++step;
+                        }
+                        __syncwarp();
+                        if (lane == 0) {
+                            s_ww[z] = w;
+                            s_wk[z] = k;
+                            s_wp[z] = pw;
+                            s_wl[z] = lw;
+                            s_wstep[z] = step;
+                            s_wc[z] = count_bits<C>(cw);
+                            s_wstate[z] = state;
+                        }
+                    }
+                    __syncthreads();
+                    if (s_wstate[0] != 1 && s_wstate[1] != 1) break;  // (the same in every thread)
+                    for (int z = 0; z < 2; ++z) {
+                        if (s_wstate[z] != 1) continue;
+                        // a long list, by the whole block
+                        const int32_t w = s_ww[z], endz = z == 0 ? s : t;
+                        const uint32_t lw = s_wl[z], step = s_wstep[z];
+                        const C tg = target_of(step, count_of<C>(s_wc[z]));
+                        const int64_t e0 = row_of(z)[w], e1 = row_of(z)[w + 1];
+                        const int32_t *bc = adj_of(z);
+                        const int zs = z ? 2 : 0;
                         // the previous level of side z, when its queue range is kept
                         const uint32_t Lp = lw - 1;
                         const long long lq0 = Lp + 1 <= (uint32_t)kLvCap ? s_lv[z][Lp] : 0;
                         const long long lq1 = Lp + 1 <= (uint32_t)kLvCap ? s_lv[z][Lp + 1] : 0;
-                        if (e1 - e0 <= kBackWarp) {
-                            if (warp == 0) warp_scan(e0, e1, C(0));
-                        } else if (a.sorted && Lp + 1 <= (uint32_t)kLvCap && lq1 - lq0 <= kMeetCap) {
+                        C *const mw = reinterpret_cast<C *>(s_mw);
+                        if (a.sorted && Lp + 1 <= (uint32_t)kLvCap && lq1 - lq0 <= kMeetCap) {
                             // a long list and a small previous level: the candidates are that
                             // level's vertices found in w's (sorted) list by bisection, their
                             // places in it give the scan order; the choice is the first, in
@@ -1077,21 +1235,21 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                     const int c = atomicAdd(&s_nc, 1);
                                     s_mv[c] = qe.x;
                                     s_mp[c] = qe.y;
-                                    s_mw[c] = count_of<C>(__ldcg(&tab[4ll * qe.y + zs + 1]));
+                                    mw[c] = count_of<C>(__ldcg(&tab[4ll * qe.y + zs + 1]));
                                     s_mj[c] = (int32_t)(blo - e0);
                                 }
                             }
                             __syncthreads();
                             const int nc = s_nc;
-                            unsigned long long best = ~0ull, lastc = 0ull;  // place << 32 | candidate
+                            u64 best = ~0ull, lastc = 0ull;  // place << 32 | candidate
                             for (int c = threadIdx.x; c < nc; c += BT) {
                                 const int32_t jc = s_mj[c];
                                 C pre = C(0);
                                 for (int c2 = 0; c2 < nc; ++c2)
-                                    if (s_mj[c2] <= jc) pre += s_mw[c2];
-                                const unsigned long long key = ((unsigned long long)(uint32_t)jc << 32) | (uint32_t)c;
-                                if (s_mw[c] > C(0)) {
-                                    if ((double)pre >= tg) best = min(best, key);
+                                    if (s_mj[c2] <= jc) pre += mw[c2];
+                                const u64 key = ((u64)(uint32_t)jc << 32) | (uint32_t)c;
+                                if (mw[c] > C(0)) {
+                                    if (pre >= tg) best = min(best, key);
                                     lastc = max(lastc, key + 1ull);
                                 }
                             }
@@ -1102,25 +1260,23 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                             }
                             if (lane == 0) {
                                 s_best[warp] = best;
-                                s_redc[warp] = C(0);
+                                s_redc[warp] = lastc;
                             }
                             __syncthreads();
-                            unsigned long long bk = s_best[0];
-                            for (int q = 1; q < nw; ++q) bk = min(bk, s_best[q]);
-                            __syncthreads();
-                            if (lane == 0) s_best[warp] = lastc;
-                            __syncthreads();
                             if (threadIdx.x == 0) {
+                                u64 bk = s_best[0];
+                                for (int q = 1; q < nw; ++q) bk = min(bk, s_best[q]);
                                 // FP64 counts past 2^53 may round the running sum just below u
                                 // sigma(w): the last candidate then takes the remainder
                                 if (bk == ~0ull && FP) {
-                                    unsigned long long lk = 0ull;
-                                    for (int q = 0; q < nw; ++q) lk = max(lk, s_best[q]);
+                                    u64 lk = 0ull;
+                                    for (int q = 0; q < nw; ++q) lk = max(lk, s_redc[q]);
                                     bk = lk ? lk - 1ull : ~0ull;
                                 }
                                 const int c = bk == ~0ull ? -1 : (int)(uint32_t)bk;
                                 s_pick = c < 0 ? -1 : s_mv[c];
                                 s_pickp = c < 0 ? -1 : s_mp[c];
+                                s_pickc = c < 0 ? 0ull : s_mw[c];
                             }
                         } else {
                             const int64_t seg = (e1 - e0 + BT - 1) / BT;
@@ -1132,15 +1288,16 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 int64_t pp[4];
                                 C v[4];
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) v[u] = cand(e + u, pv[u], pp[u]);
+                                for (int u = 0; u < 4; ++u) v[u] = cand(z, lw, e + u, pv[u], pp[u]);
                                 my += (v[0] + v[1]) + (v[2] + v[3]);
                             }
                             for (; e < se; ++e) {
                                 int32_t pv;
                                 int64_t pp;
-                                my += cand(e, pv, pp);
+                                my += cand(z, lw, e, pv, pp);
                             }
                             // exclusive block scan of the segment sums
+                            C *const redc = reinterpret_cast<C *>(s_redc);
                             C inc = my;
 #pragma unroll
                             for (int o = 1; o < 32; o <<= 1) {
@@ -1148,11 +1305,11 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 if (lane >= o) inc += t2;
                             }
                             if (threadIdx.x == 0) s_tstar = 0x7fffffff;
-                            if (lane == 31) s_redc[warp] = inc;
+                            if (lane == 31) redc[warp] = inc;
                             __syncthreads();
                             C pre = inc - my;
-                            for (int q = 0; q < warp; ++q) pre += s_redc[q];
-                            const bool reach = my > C(0) && (double)(pre + my) >= tg;
+                            for (int q = 0; q < warp; ++q) pre += redc[q];
+                            const bool reach = my > C(0) && pre + my >= tg;
                             const unsigned rb = __ballot_sync(0xffffffffu, reach);
                             if (rb && lane == __ffs(rb) - 1) atomicMin(&s_tstar, (int)threadIdx.x);
                             __syncthreads();
@@ -1163,50 +1320,51 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 __syncthreads();
                                 ts = s_tlast;
                             }
-                            if ((int)threadIdx.x == ts) s_tpre = pre;
+                            if ((int)threadIdx.x == ts) s_tpre = count_bits<C>(pre);
                             __syncthreads();
                             if (warp == 0) {
+                                int32_t pick = -1;
+                                int64_t pickp = -1;
+                                C pickc = C(0);
                                 if (ts >= 0 && ts < BT) {  // (no segment with a candidate: no choice)
                                     const int64_t tb = min(e1, e0 + (int64_t)ts * seg);
-                                    warp_scan(tb, min(e1, tb + seg), s_tpre);
-                                } else if (lane == 0) {
-                                    s_pick = -1;
-                                    s_pickp = -1;
+                                    warp_scan(z, lw, tb, min(e1, tb + seg), count_of<C>(s_tpre), tg, pick, pickp,
+                                              pickc);
+                                }
+                                if (lane == 0) {
+                                    s_pick = pick;
+                                    s_pickp = pickp;
+                                    s_pickc = count_bits<C>(pickc);
                                 }
                             }
                             if (threadIdx.x == 0) s_tlast = -1;
                         }
                         __syncthreads();
-                        const int32_t pick = s_pick;
-                        const int64_t pickp = s_pickp;
-                        __syncthreads();  // s_pick is written again by the next step
-                        if (pick < 0) {
-                            if (threadIdx.x == 0) {
-                                atomicOr(a.status, DEV_BAD_PATH);
-                                if (a.trace) {  // where the path ended without a candidate
-                                    a.trace[8 * i + 6] = (e1 - e0 <= BT ? 1ull : 2ull) | ((unsigned long long)z << 4) |
-                                                         ((unsigned long long)step << 8) |
-                                                         ((unsigned long long)(e1 - e0) << 32);
-                                    a.trace[8 * i + 7] = ((unsigned long long)(uint32_t)w << 32) | lw;
+                        if (threadIdx.x == 0) {
+                            const int32_t pick = s_pick;
+                            if (pick < 0) {
+                                failed(z, step, e1 - e0, w, lw);
+                                s_ww[z] = endz;  // (the walk ends here)
+                            } else {
+                                if (pick != endz) {
+                                    const int32_t k = s_wk[z];
+                                    if (store && k < len) a.arena[off + k] = pick;
+                                    atomicAdd(&a.cnt[pick], 1ull);
+                                    s_wk[z] = k + 1;
                                 }
+                                s_ww[z] = pick;
+                                s_wp[z] = s_pickp;
+                                s_wc[z] = s_pickc;
+                                s_wl[z] = lw - 1;
+                                s_wstep[z] = step + 1;
                             }
-                            bad = true;
-                            break;
                         }
-                        if (pick != endz) {
-                            if (threadIdx.x == 0) {
-                                if (store && k < len) a.arena[off + k] = pick;
-                                atomicAdd(&a.cnt[pick], 1ull);
-                            }
-                            ++k;
-                        }
-                        w = pick;
-                        pw = pickp;
-                        ++step;
+                        __syncthreads();
                     }
-                    if (bad) break;
                 }
-            }
+            };
+            if (fp) backtrack(0.0);
+            else backtrack(0ull);
         }
         __syncthreads();
         if (a.work && threadIdx.x == 0) {
@@ -1285,9 +1443,8 @@ int blocks_per_sm(int *cache) {
         int per_sm = 0;
         const int dyn = (int)(sizeof(uint32_t) * (BT == kBiBlock ? kBloomWordsFirst : kBloomWords));
         if (dyn > 48 * 1024)
-            cudaFuncSetAttribute(k_bibfs<unsigned long long, HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 dyn);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bibfs<unsigned long long, HASH, BT>, BT, dyn) !=
+            cudaFuncSetAttribute(k_bibfs<HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bibfs<HASH, BT>, BT, dyn) !=
                 cudaSuccess ||
             per_sm < 1) {
             cudaGetLastError();
@@ -1303,11 +1460,9 @@ void launch(percis_ctx *ctx, int grid, const BiArgs &a) {
     // the heavy pass's Bloom filter (dynamic shared memory)
     const int dyn = (int)(sizeof(uint32_t) * (BT == kBiBlock ? kBloomWordsFirst : kBloomWords));
     if (dyn > 48 * 1024) {
-        cudaFuncSetAttribute(k_bibfs<double, HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        cudaFuncSetAttribute(k_bibfs<unsigned long long, HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        cudaFuncSetAttribute(k_bibfs<HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     }
-    if (ctx->sigma_mode == 2) k_bibfs<double, HASH, BT><<<grid, BT, dyn, ctx->stream>>>(a);
-    else k_bibfs<unsigned long long, HASH, BT><<<grid, BT, dyn, ctx->stream>>>(a);
+    k_bibfs<HASH, BT><<<grid, BT, dyn, ctx->stream>>>(a);
 }
 
 BiArgs common_args(percis_ctx *ctx, uint64_t seed, uint32_t tag_path) {

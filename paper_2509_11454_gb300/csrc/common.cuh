@@ -84,9 +84,10 @@ __device__ __forceinline__ void uniforms2(uint64_t seed, uint64_t i, uint32_t ta
 }
 
 __device__ __forceinline__ double uniform_at(uint64_t seed, uint64_t i, uint32_t tag, uint32_t step) {
-    double a, b;
-    uniforms2(seed, i, tag, step >> 1, a, b);
-    return (step & 1) ? b : a;
+    uint32_t c0 = (uint32_t)i, c1 = (uint32_t)(i >> 32), c2 = tag, c3 = step >> 1;
+    philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
+    const uint64_t w = (step & 1) ? ((uint64_t)c3 << 32) | c2 : ((uint64_t)c1 << 32) | c0;
+    return __dmul_rn((double)((w >> 11) + 1), 0x1p-53);
 }
 
 // ------------------------------------------------------------ timers/atomics

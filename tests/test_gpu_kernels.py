@@ -1,0 +1,66 @@
+"""Kernel branches at the sizes where they can go wrong, against the CPU oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2509_11454_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def binding():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2509_11454_gb300 import binding as b
+
+    b.load_library()
+    return b
+
+
+def _engine(binding, g, x=None, **opts):
+    eng = binding.PercIS(0)
+    if opts:
+        eng.set_options(**opts)
+    eng.load_csr(g.row_ptr, g.col, directed=g.directed)
+    if x is not None:
+        eng.set_states(x)
+    return eng
+
+
+def _np(t):
+    return t.cpu().numpy()
+
+
+@pytest.mark.parametrize("side,table_log", [(30, 0), (74, 0), (74, 13), (74, -1)])
+def test_bidir_counts_pass_2_53_inside_a_phase(binding, side, table_log):
+    """Samples whose counts (or only whose products) pass 2^53 change to FP64
+    counts on their own: the others' paths equal the oracle's exactly, theirs
+    are shortest paths of the same length (FP64 sums past 2^53 round in the
+    order of the additions, so the choice itself may differ there)."""
+    g = synth.grid_2d(side, 0.0, 0)
+    og = oracle.from_synth(g)
+    x = synth.states_uniform(g.n, 1)
+    prep = oracle.prepare(x)
+    eng = _engine(binding, g, x, form="bidir", bi_table_log=table_log)
+    count = 240
+    ph = eng.run_phase(3, 1, count)
+    ptr, nodes = (_np(v) for v in eng.get_paths(count))
+    over = 0
+    for i in range(count):
+        ref = oracle.run_samples(og, prep, 3, 1, 3, i, 1, keep_paths=True, bidir=True)
+        assert int(ph["kind"][i]) == int(ref.kind[0]) and int(ph["ilen"][i]) == int(ref.ilen[0]), i
+        path = nodes[ptr[i]:ptr[i + 1]]
+        if not ref.overflow:
+            assert np.array_equal(path, ref.path_nodes), i
+            continue
+        over += 1
+        rows, cols = np.divmod(np.sort(path), side)  # a monotone staircase between the ends
+        s, t = divmod(int(ref.s[0]), side), divmod(int(ref.t[0]), side)
+        assert len(set(path.tolist())) == len(path) == abs(s[0] - t[0]) + abs(s[1] - t[1]) - 1, i
+        assert rows.min() >= min(s[0], t[0]) and rows.max() <= max(s[0], t[0]), i
+        assert cols.min() >= min(s[1], t[1]) and cols.max() <= max(s[1], t[1]), i
+    assert (over > 0) == (side > 60) and over < count
+    eng.close()
