@@ -64,3 +64,24 @@ def test_bidir_counts_pass_2_53_inside_a_phase(binding, side, table_log):
         assert cols.min() >= min(s[1], t[1]) and cols.max() <= max(s[1], t[1]), i
     assert (over > 0) == (side > 60) and over < count
     eng.close()
+
+
+@pytest.mark.parametrize("n,hub", [(2, 0), (65, 0), (300, 129), (513, 128), (700, 400)])
+def test_exact_centrality_items(binding, n, hub):
+    """Exact centrality where its work splits: one or several words of sources, a last
+    batch narrower than the first (n = 513, 700), rows at and above the length a whole
+    block shares (128).  Sums of at most n^2 non-negative terms of relative error
+    2^-52 each way: 4 n^2 2^-53 relative to the largest value."""
+    rng = np.random.default_rng(n)
+    src, dst = rng.integers(0, n, 3 * n), rng.integers(0, n, 3 * n)
+    src, dst = np.concatenate([src, np.zeros(hub), [0]]), np.concatenate([dst, np.arange(1, hub + 1), [1]])
+    g = synth.csr_from_edges(n, src, dst, directed=False)
+    x = synth.states_uniform(n, n)
+    if n == 2:
+        with pytest.raises(RuntimeError):  # C_v = 0: undefined
+            _engine(binding, g, x)
+        return
+    eng = _engine(binding, g, x)
+    ref = oracle.exact_pc(oracle.from_synth(g), x)
+    assert np.max(np.abs(_np(eng.exact()) - ref)) <= 4 * n * n * 2.0 ** -53 * ref.max()
+    eng.close()
