@@ -45,8 +45,11 @@ struct alignas(16) MsCtl {
 struct PlainCtl {
     uint32_t bar_count, bar_gen;
     uint32_t status;
-    int32_t qsize[3];  // queue sizes, level L in slot L % 3
+    int32_t qsize[3];  // queue sizes, level L in slot L % 3: rows of ordinary length,
+    int32_t hsize[3];  // long rows, and the level's vertices of long in-rows
+    int32_t nhub[3];
     int32_t level;
+    alignas(16) int4 solo[2];  // a stint of block 0 alone: next frontier, its long rows, level, target found
     int32_t found;
 };
 
@@ -78,7 +81,7 @@ struct percis_ctx {
     percis::DevBuf dscal;  // device scalars: [0] = c, [1] = dhat
 
     // plain BFS state
-    percis::DevBuf ep, lvl, sigma1, qa, qb, plain_ctl;
+    percis::DevBuf stamp, plain_hub, sigma1, qa, qb, plain_ctl;
     int32_t epoch = 0;
     int plain_grid = 0;  // cooperative grid of the plain BFS on this device (0 = not yet queried)
     int bi_per_sm = 0;   // resident blocks per SM of the bidirectional kernel (0 = not yet queried)

@@ -85,3 +85,30 @@ def test_exact_centrality_items(binding, n, hub):
     ref = oracle.exact_pc(oracle.from_synth(g), x)
     assert np.max(np.abs(_np(eng.exact()) - ref)) <= 4 * n * n * 2.0 ** -53 * ref.max()
     eng.close()
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("hub", [31, 1024, 1025, 9000])
+def test_plain_bfs_rows_and_levels(binding, directed, hub):
+    """The single-source BFS where its work splits: rows of one warp, of a whole
+    block's parts (above 1,024 edges, out and in), frontiers one block runs alone
+    (a 300-vertex tail, more than one stint) and ones the grid takes; from the hub,
+    from the tail's end and truncated at a target; VertexDiamUB."""
+    rng = np.random.default_rng(hub)
+    n = hub + 2 + 300 + 2000
+    a, b = np.arange(2, hub + 2), np.full(hub, 1)
+    src = [np.zeros(hub, int), a, np.arange(hub + 2, hub + 302)]
+    dst = [a, b, np.arange(hub + 3, hub + 303)]
+    src += [[1], rng.integers(hub + 302, n, 6000), [hub + 302]]  # hub 0 -> spokes -> 1 -> tail -> random part
+    dst += [[hub + 2], rng.integers(hub + 302, n, 6000), [n - 1]]
+    g = synth.csr_from_edges(n, np.concatenate(src), np.concatenate(dst), directed=directed)
+    og = oracle.from_synth(g)
+    eng = _engine(binding, g)
+    for s, t in ((0, -1), (hub + 150, -1), (n - 1, -1), (0, 1), (0, hub + 200), (5, 0), (0, n - 1), (n - 1, n - 2)):
+        dist, sigma = (_np(v) for v in eng.bfs(s, t))
+        _, rd, rs, _, _, _ = oracle.bfs(og, s, t)
+        m = rd >= 0 if t >= 0 else slice(None)  # truncated: the vertices the oracle settled
+        assert np.array_equal(dist[m], rd[m]) and np.array_equal(sigma[m], rs[m]), (s, t)
+    if not directed:
+        assert binding.percis_get_prep(eng.ctx)["vertex_diam"] == oracle.vertex_diam_ub(og)
+    eng.close()
