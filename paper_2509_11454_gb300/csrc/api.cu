@@ -397,7 +397,8 @@ void percis_destroy(percis_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->aux) cudaStreamSynchronize(ctx->aux);
     DevBuf *bufs[] = {&ctx->rp, &ctx->col, &ctx->irp, &ctx->icol, &ctx->x, &ctx->xs, &ctx->perm, &ctx->w, &ctx->ci,
-                      &ctx->r, &ctx->Cv, &ctx->lam, &ctx->grp_lo, &ctx->grp_hi, &ctx->dscal, &ctx->stamp, &ctx->plain_hub,
+                      &ctx->r, &ctx->Cv, &ctx->lam, &ctx->grp_lo, &ctx->grp_hi, &ctx->dscal, &ctx->stamp, &ctx->plain_hub, &ctx->ms_big, &ctx->ms_walks,
+                      &ctx->ms_need, &ctx->ms_list, &ctx->ms_levels,
                       &ctx->sigma1, &ctx->qa, &ctx->qb, &ctx->plain_ctl, &ctx->vis, &ctx->fhist, &ctx->sigmaW,
                       &ctx->ms_ctl, &ctx->remaining, &ctx->found, &ctx->pair_s, &ctx->pair_t, &ctx->kind,
                       &ctx->ilen, &ctx->path_off, &ctx->arena, &ctx->cnt, &ctx->arena_top, &ctx->src_count,

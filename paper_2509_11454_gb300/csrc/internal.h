@@ -73,6 +73,8 @@ struct percis_ctx {
     bool rows_sorted = false;  // every CSR row strictly increasing (no duplicate edges)
     percis::DevBuf vorder;  // vertices sorted by (highest-degree neighbour, id): lane order of sources
     bool vorder_ready = false;
+    percis::DevBuf ms_big, ms_walks;  // batched form: long in-rows {count, safe levels, walk maxima, ids}, scratch
+    bool ms_rows_ready = false, ms_walks_ready = false;
 
     // states and preprocessing
     bool have_states = false;
@@ -92,6 +94,7 @@ struct percis_ctx {
     int32_t levels_alloc = 0;
     int sigma_mode = 0;  // batched sigma storage: 0 = 32-bit, 1 = 64-bit integers, 2 = FP64
     percis::DevBuf fq0, fq1;  // frontier queues
+    percis::DevBuf ms_need, ms_list, ms_levels;  // needed lanes of every vertex, their lists, counts per level
     percis::DevBuf acc_ap, ap_tau, ap_stamp, ap_list;  // all-paths estimator
     percis::DevBuf plan_dev;                           // lane batches of a many-graph phase
     percis::DevBuf bi_info, bi_queue;                  // bidirectional form, direct store: per-slot scratch

@@ -8,7 +8,8 @@
 // (the sigma recurrence of the oracle, summed in any order: the values are
 // integers below 2^53, so every order gives the same exact result).  A lane
 // retires once every target of its samples is discovered (its level is then
-// complete) or its frontier is empty.  After the last level the same launch
+// complete) or its frontier is empty.  Where only samples are wanted the counts
+// come after the levels, for the vertices their paths can pass (ms_batch).  Then the same launch
 // backtracks every sample of the batch (one warp per sample) exactly as the
 // plain form does, reading the frontier history for the predecessor test.
 //
@@ -38,6 +39,11 @@ constexpr int kMsBlock = 256;
 #ifndef PERCIS_BLOCK_DEG
 #define PERCIS_BLOCK_DEG 256
 #endif
+constexpr int kGroupLanes = 8;      // lanes that share a vertex
+constexpr int64_t kMidRow = 64;     // rows above it: a whole warp
+constexpr int64_t kBigRow = 256;    // in-rows above it: a whole block (listed once per graph)
+constexpr int64_t kLightOut = 64;   // out-rows above it: a whole block
+constexpr int kQueueBuf = 96;       // queue entries a warp gathers before it appends them
 constexpr int64_t kBlockDeg = PERCIS_BLOCK_DEG;  // in-degree above which a whole block counts one (vertex, word)
 
 struct MsArgs {
@@ -83,6 +89,16 @@ struct MsArgs {
     const int32_t *col;
     int32_t *fq0;
     int32_t *fq1;
+    // long rows, needed vertices (see ms_batch); nlist holds ncap entries, ncnt and
+    // cont are per level: {light, heavy} counts twice over, lanes that go on
+    const int32_t *big;
+    const int32_t *big_count;
+    const int32_t *lsafe;
+    uint64_t *need;
+    int32_t *nlist;
+    int64_t ncap;
+    int32_t *ncnt;
+    uint64_t *cont;
     int32_t policy;                   // 0 = pull every level, 1 = push every level, 2 = by work estimate
     double push_alpha;                // policy 2: push while alpha * push work < pull work
     // instrumentation (INSTR variant only)
@@ -177,22 +193,181 @@ __device__ __forceinline__ void gather_chunk(const ST *sig, int W, int w, uint64
     }
 }
 
-// One batch of lanes: levels, counts and the backtrack of its samples.  The
-// batch covers lanes lane_base .. lane_base + nlanes - 1 and the vertex range
-// [vlo, vlo + n); rp / irp point at entry vlo.  Returns false when the launch
-// must stop (a bounded wait ran out, or the frontier history is too short).
+// Counts of level L for the listed vertices (nl from the front of lq, those of
+// in-degree > 32, nh, from the back of hq): of a vertex's level-L lanes, all
+// (every), or those of `cont` and need.
 template <int K, bool INSTR, int SM>
-__device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_base, const int32_t nlanes,
-                                         const int32_t vlo, const int64_t n, const int64_t *rp, const int64_t *irp,
-                                         const int32_t ap_epoch) {
+__device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo, const int64_t *irp, int L,
+                                         const int32_t *lq, int64_t nl, const int32_t *hq, int64_t nh, bool every,
+                                         const uint64_t *cont, bool *ovf_out, unsigned long long *work) {
     constexpr int W = 64 * K;
     constexpr bool FPSIG = SM == 2;
     using S = typename SigmaMode<SM>::S;
     using ST = typename SigmaMode<SM>::ST;
     constexpr unsigned long long kLimit = SigmaMode<SM>::limit;
+    __shared__ S s_red[kMsBlock / 32][64];  // per-warp partial sums of a block-wide gather
+    ST *sig = static_cast<ST *>(a.sigma);
+    const int lane = threadIdx.x & 31, warp_in_block = threadIdx.x >> 5;
+    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t nk = n * K;
+    const uint64_t *fl = a.fh + (int64_t)L * nk;
+    bool ovf = false;
+    unsigned long long n_sload = 0, n_swrite = 0;
+    auto bits = [&](int32_t v, int wd) -> uint64_t {
+        const int64_t q = (int64_t)v * K + wd;
+        const uint64_t f = __ldcg(&fl[q]);
+        if (every) return f;
+        return f & ((cont ? __ldcg(&cont[wd]) : 0ull) | __ldcg(&a.need[q]));
+    };
+    const uint64_t *fprev = a.fh + (int64_t)(L - 1) * nk;
+    if (!FPSIG) {
+        // in-degree > kBlockDeg: one block per (vertex, word), its warps
+        // splitting the edges; the partial sums meet in shared memory
+        // (integer sums, so the order does not matter)
+        for (int64_t hi = blockIdx.x; hi < nh * K; hi += gridDim.x) {
+            const int64_t h = hi / K;
+            const int wd = (int)(hi - h * K);
+            const int32_t v = __ldcg(&hq[-h]);
+            const int64_t e0 = irp[v], e1 = irp[v + 1];
+            if (e1 - e0 <= kBlockDeg) continue;  // a warp item below; the same for the whole block
+            const uint64_t nbw = bits(v, wd);
+            if (nbw == 0ull) continue;
+            S acc0 = S(0), acc1 = S(0);
+            for (int64_t base = e0 + warp_in_block * 32; base < e1; base += kMsBlock) {
+                const int64_t e = base + lane;
+                int32_t u = 0;
+                uint64_t fw = 0ull;
+                if (e < e1) {
+                    u = a.icol[e] - vlo;
+                    fw = __ldcg(&fprev[(int64_t)u * K + wd]) & nbw;
+                }
+                if (INSTR) n_sload += (unsigned long long)__popcll(fw);
+                gather_chunk<SM, ST, S>(sig, W, wd, fw, u, acc0, acc1, ovf);
+            }
+            s_red[warp_in_block][lane] = acc0;
+            s_red[warp_in_block][lane + 32] = acc1;
+            __syncthreads();
+            if (warp_in_block == 0) {
+                S t0 = S(0), t1 = S(0);
+#pragma unroll
+                for (int q = 0; q < kMsBlock / 32; ++q) {
+                    t0 += s_red[q][lane];
+                    t1 += s_red[q][lane + 32];
+                }
+                ovf |= (t0 >= (S)kLimit) | (t1 >= (S)kLimit);
+                ST *drow = sig + (int64_t)v * W + 64 * wd;
+                if ((nbw >> lane) & 1ull) drow[lane] = (ST)t0;
+                if ((nbw >> (lane + 32)) & 1ull) drow[lane + 32] = (ST)t1;
+                if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
+            }
+            __syncthreads();
+        }
+    }
+    for (int64_t it = gwarp; it < nl + nh * K; it += nwarps) {
+        if (it < nl) {
+            // in-degree <= 32: one warp per vertex, its parents and all their
+            // words loaded once; lane w < K holds the word's lanes to count
+            const int32_t v = __ldcg(&lq[it]);
+            uint64_t nbl = 0ull;
+            if (lane < K) nbl = bits(v, lane);
+            const unsigned wm = __ballot_sync(0xffffffffu, nbl != 0ull);
+            if (!wm) continue;
+            const int64_t e0 = irp[v], e1 = irp[v + 1];
+            ST *drow = sig + (int64_t)v * W;
+            const int64_t e = e0 + lane;
+            int32_t u = 0;
+            uint64_t f[K];
+            if (e < e1) {
+                u = a.icol[e] - vlo;
+                load_words<K>(fprev + (int64_t)u * K, f);
+            } else {
+#pragma unroll
+                for (int q = 0; q < K; ++q) f[q] = 0ull;
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                if (!((wm >> q) & 1u)) continue;
+                const uint64_t nbw = shfl64(nbl, q);
+                const uint64_t fw = f[q] & nbw;
+                if (INSTR) n_sload += (unsigned long long)__popcll(fw);
+                S acc0 = S(0), acc1 = S(0);
+                gather_chunk<SM, ST, S>(sig, W, q, fw, u, acc0, acc1, ovf);
+                if (FPSIG) ovf |= (acc0 >= (S)kLimit) | (acc1 >= (S)kLimit);
+                if ((nbw >> lane) & 1ull) drow[64 * q + lane] = (ST)acc0;
+                if ((nbw >> (lane + 32)) & 1ull) drow[64 * q + lane + 32] = (ST)acc1;
+                if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
+            }
+        } else {
+            // in-degree in (32, kBlockDeg] (any, for FP64 counts, whose
+            // additions keep the in-adjacency order): one warp per
+            // (vertex, word) over 32-edge chunks
+            const int64_t h = (it - nl) / K;
+            const int wd = (int)(it - nl - h * K);
+            const int32_t v = __ldcg(&hq[-h]);
+            const int64_t e0 = irp[v], e1 = irp[v + 1];
+            if (!FPSIG && e1 - e0 > kBlockDeg) continue;
+            const uint64_t nbw = bits(v, wd);
+            if (nbw == 0ull) continue;
+            S acc0 = S(0), acc1 = S(0);
+            for (int64_t base = e0; base < e1; base += 32) {
+                const int64_t e = base + lane;
+                int32_t u = 0;
+                uint64_t fw = 0ull;
+                if (e < e1) {
+                    u = a.icol[e] - vlo;
+                    fw = __ldcg(&fprev[(int64_t)u * K + wd]) & nbw;
+                }
+                if (INSTR) n_sload += (unsigned long long)__popcll(fw);
+                gather_chunk<SM, ST, S>(sig, W, wd, fw, u, acc0, acc1, ovf);
+            }
+            if (FPSIG) ovf |= (acc0 >= (S)kLimit) | (acc1 >= (S)kLimit);
+            ST *drow = sig + (int64_t)v * W + 64 * wd;
+            if ((nbw >> lane) & 1ull) drow[lane] = (ST)acc0;
+            if ((nbw >> (lane + 32)) & 1ull) drow[lane + 32] = (ST)acc1;
+            if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
+        }
+    }
+    if (ovf) *ovf_out = true;
+    if (INSTR) {
+        work[0] += n_sload;
+        work[1] += n_swrite;
+    }
+}
+
+// One batch of lanes: levels, counts and the backtrack of its samples.  The
+// batch covers lanes lane_base .. lane_base + nlanes - 1 and the vertex range
+// [vlo, vlo + n); rp / irp point at entry vlo.  Returns false when the launch
+// must stop (a bounded wait ran out, or the frontier history is too short).
+//
+// A full traversal counts every vertex.  A sampling batch needs the counts of a
+// target's ancestors alone (the backtrack reads predecessors of what it has
+// reached), a few hundred of the 100,000 vertices a lane reaches: after the
+// levels, one backward pass over the frontier history marks them (one bit per
+// lane: need), and a forward pass counts those.  This is only done where no count
+// anywhere can reach 2^53 (the number of walks of that length, *a.lsafe), so that
+// the overflow flag says the same; otherwise every vertex of a continuing lane is
+// counted, as in FP64 reruns.  Barabasi-Albert 100k, 512 lanes: 1.54 ms a batch
+// with counts everywhere (the gathers of the two largest levels), 0.70 ms.
+//
+// Eight lanes share a vertex, lane w mod K on its word w (8 / K edges side by side
+// for K < 8): an edge's K words are one coalesced access and the OR over a row
+// stays in registers.
+template <int K, bool INSTR, int SM>
+__device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_base, const int32_t nlanes,
+                                         const int32_t vlo, const int64_t n, const int64_t *rp, const int64_t *irp,
+                                         const int32_t ap_epoch) {
+    constexpr int W = 64 * K;
+    constexpr int SUB = kGroupLanes / K;     // edges a vertex's eight lanes take side by side
+    constexpr int GW = 32 / kGroupLanes;     // vertices a warp takes together
+    constexpr int EW = 32 / K;               // edges a whole warp takes side by side
+    constexpr int EB = kMsBlock / K;         // edges a whole block takes side by side
+    constexpr bool FPSIG = SM == 2;
+    using S = typename SigmaMode<SM>::S;
+    using ST = typename SigmaMode<SM>::ST;
     ST *sig = static_cast<ST *>(a.sigma);
     bool ovf = false;
-    unsigned long long n_sload = 0, n_swrite = 0, n_uv = 0, n_ue = 0;
+    unsigned long long n_s[2] = {0, 0}, n_uv = 0, n_ue = 0;  // sigma reads and writes; frontier vertices, edges
     MsCtl *ctl = a.ctl;
     GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
     uint32_t *status = &ctl->status;
@@ -205,14 +380,20 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
     const int64_t nk = n * K;
     const long long p0 = a.full ? 0 : a.lane_off[lane_base];
     const long long p1 = a.full ? 0 : a.lane_off[lane_base + nlanes];
+    const int w = lane % K;  // this lane's word wherever lanes share a vertex
+    const int nbig = (int)__ldg(a.big_count);
+    const unsigned gmask = ((kGroupLanes == 32 ? 0u : (1u << kGroupLanes)) - 1u) << (lane & ~(kGroupLanes - 1));
 
-    // ---- prologue: clear visited, frontiers 0 and 1, (push) sigma; reset lane state
+    // ---- prologue: clear visited, need, frontiers 0 and 1; reset lane state
     for (int64_t i = tid; i < nk; i += nthreads) {
         a.vis[i] = 0ull;
+        if (!a.full) a.need[i] = 0ull;
         a.fh[i] = 0ull;
         a.fh[nk + i] = 0ull;
     }
     for (long long p = p0 + tid; p < p1; p += nthreads) a.found[p] = -1;
+    if (!a.full)
+        for (int64_t i = tid; i < 4 * (int64_t)(a.Lcap + 2); i += nthreads) a.ncnt[i] = 0;
     if (INSTR)
         for (int64_t i = tid; i < (int64_t)W * (a.Lcap + 1); i += nthreads) a.levdeg[i] = 0ull;
     if (blockIdx.x == 0) {
@@ -227,7 +408,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         if (threadIdx.x == 0) {
             ctl->ticket = 0;
             ctl->level = 0;
-            ctl->qn[0] = nlanes;
+            ctl->qn[0] = 0;
             ctl->qn[1] = 0;
             ctl->qh[0] = 0;
             ctl->qh[1] = 0;
@@ -242,7 +423,8 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         atomicOr((unsigned long long *)&a.vis[(int64_t)v * K + (j >> 6)], (unsigned long long)bit);
         atomicOr((unsigned long long *)&a.fh[(int64_t)v * K + (j >> 6)], (unsigned long long)bit);
         sig[(int64_t)v * W + j] = ST(1);
-        a.fq0[j] = v;
+        if (rp[v + 1] - rp[v] > kLightOut) a.fq0[n - 1 - atomicAdd(&ctl->qh[0], 1)] = v;
+        else a.fq0[atomicAdd(&ctl->qn[0], 1)] = v;
         if (INSTR) a.levdeg[(int64_t)j * (a.Lcap + 1)] = (unsigned long long)(rp[v + 1] - rp[v]);
         if (!a.full) {
             const long long q0 = a.lane_off[lane_base + j], q1 = a.lane_off[lane_base + j + 1];
@@ -253,148 +435,215 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
 
     __shared__ unsigned long long s_nonempty[K];
     __shared__ unsigned long long s_act[K];
-    __shared__ unsigned long long s_cont[K];
-    __shared__ S s_red[kMsBlock / 32][64];  // per-warp partial sums of a block-wide gather
+    __shared__ unsigned long long s_or[K];
+    __shared__ int32_t s_q[kMsBlock / 32][kQueueBuf];
+    __shared__ int s_last;
+
+    // append the vertices of lanes with `any` (light from the front, heavy from the
+    // back); a warp's light ones go out in runs.  Every lane of the warp calls it.
+    int held = 0;  // (the same in every lane)
+    auto flush = [&](int32_t *q, int32_t *qn, int64_t cap) {
+        if (held == 0) return;
+        __syncwarp();
+        int pos = 0;
+        if (lane == 0) pos = atomicAdd(qn, held);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        for (int k = lane; k < held; k += 32)
+            if (pos + k < cap) q[pos + k] = s_q[warp_in_block][k];
+        __syncwarp();
+        held = 0;
+    };
+    auto append = [&](bool light, bool heavy, int32_t v, int32_t *q, int32_t *qn, int32_t *qh, int64_t cap,
+                      int64_t hoff) {
+        const unsigned am = __ballot_sync(0xffffffffu, light);
+        if (light) s_q[warp_in_block][held + __popc(am & ((1u << lane) - 1u))] = v;
+        held += __popc(am);
+        if (held > kQueueBuf - 32) flush(q, qn, cap);
+        if (heavy) {
+            const int64_t pos = hoff + atomicAdd(qh, 1);
+            if (pos < cap) q[cap - 1 - pos] = v;
+        }
+    };
+
     int L = 0;
     for (;;) {
-        bool any_act = false;
-#pragma unroll
-        for (int w = 0; w < K; ++w) any_act |= ld_relaxed_u64((const uint64_t *)&ctl->active[w]) != 0ull;
-        if (!any_act) break;
         if (threadIdx.x < K) {
             s_nonempty[threadIdx.x] = 0ull;
             s_act[threadIdx.x] = ld_relaxed_u64((const uint64_t *)&ctl->active[threadIdx.x]);
         }
         __syncthreads();
+        unsigned long long any_act = 0ull;
+#pragma unroll
+        for (int q = 0; q < K; ++q) any_act |= s_act[q];
+        if (!any_act) break;  // (the same in every block)
+        const uint64_t actw = s_act[w];
         const uint64_t *fcur = a.fh + (int64_t)L * nk;
         uint64_t *fnext = a.fh + (int64_t)(L + 1) * nk;
         const int32_t *qcur = (L & 1) ? a.fq1 : a.fq0;
         int32_t *qnext = (L & 1) ? a.fq0 : a.fq1;
-        int32_t *qn_next = &ctl->qn[(L + 1) & 1];
-        int32_t *qh_next = &ctl->qh[(L + 1) & 1];
         const bool push = ld_relaxed_u32((const uint32_t *)&ctl->push_next) != 0u;
+        const int64_t qn = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qn[L & 1]);
+        const int64_t qh = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qh[L & 1]);
 
-        // ---- phase A1: discover level L+1 (frontier bits only; counts follow in A2).
-        // One warp per vertex with all K lane words at once: lane w < K holds
-        // word w, edges are spread over the lanes and their K words are loaded
-        // together.
+        // ---- discover level L+1 (frontier bits only)
         if (push) {
-            const int64_t qn = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qn[L & 1]);
-            const int64_t qh = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qh[L & 1]);
-            // vertices of in-degree > 32 (the back of the queue) one block each,
-            // its warps splitting the edges; then one warp per light vertex
+            auto push_edges = [&](int64_t e, int64_t e1, int64_t stride, uint64_t fu) {
+                for (; e < e1; e += 4 * stride) {
+                    int32_t v[4];
+                    uint64_t m[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = e + q * stride < e1 ? a.col[e + q * stride] - vlo : -1;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) m[q] = v[q] >= 0 ? fu & ~__ldcg(&a.vis[(int64_t)v[q] * K + w]) : 0ull;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)  // fire-and-forget: collected after the barrier
+                        if (m[q]) atomicOr((unsigned long long *)&fnext[(int64_t)v[q] * K + w], (unsigned long long)m[q]);
+                }
+            };
+            // long rows one block each, then one warp per vertex
             for (int64_t r = blockIdx.x; r < qh; r += gridDim.x) {
                 const int32_t u = __ldcg(&qcur[n - 1 - r]);
-                uint64_t fl = 0ull;
-                if (lane < K) fl = __ldcg(&fcur[(int64_t)u * K + lane]) & s_act[lane];
-                if (!__ballot_sync(0xffffffffu, fl != 0ull)) continue;
-                uint64_t fu[K];
-#pragma unroll
-                for (int w = 0; w < K; ++w) fu[w] = shfl64(fl, w);
-                const int64_t e0 = rp[u], e1 = rp[u + 1];
-                for (int64_t e = e0 + warp_in_block * 32 + lane; e < e1; e += kMsBlock) {
-                    const int32_t v = a.col[e] - vlo;
-                    uint64_t vv[K];
-                    load_words<K>(a.vis + (int64_t)v * K, vv);
-#pragma unroll
-                    for (int w = 0; w < K; ++w) {
-                        const uint64_t m = fu[w] & ~vv[w];
-                        if (m) atomicOr((unsigned long long *)&fnext[(int64_t)v * K + w], (unsigned long long)m);
-                    }
-                }
+                push_edges(rp[u] + threadIdx.x / K, rp[u + 1], EB, __ldcg(&fcur[(int64_t)u * K + w]) & actw);
             }
             for (int64_t k = gwarp; k < qn; k += nwarps) {
                 const int32_t u = __ldcg(&qcur[k]);
-                uint64_t fl = 0ull;
-                if (lane < K) fl = __ldcg(&fcur[(int64_t)u * K + lane]) & s_act[lane];
-                if (!__ballot_sync(0xffffffffu, fl != 0ull)) continue;
-                uint64_t fu[K];
-#pragma unroll
-                for (int w = 0; w < K; ++w) fu[w] = shfl64(fl, w);
-                const int64_t e0 = rp[u], e1 = rp[u + 1];
-                for (int64_t e = e0 + lane; e < e1; e += 32) {
-                    const int32_t v = a.col[e] - vlo;
-                    uint64_t vv[K];
-                    load_words<K>(a.vis + (int64_t)v * K, vv);
-#pragma unroll
-                    for (int w = 0; w < K; ++w) {
-                        const uint64_t m = fu[w] & ~vv[w];
-                        // fire-and-forget: the new frontier is collected after the barrier
-                        if (m) atomicOr((unsigned long long *)&fnext[(int64_t)v * K + w], (unsigned long long)m);
-                    }
-                }
+                push_edges(rp[u] + lane / K, rp[u + 1], EW, __ldcg(&fcur[(int64_t)u * K + w]) & actw);
             }
         } else {
-            // every vertex with unvisited active lanes; the scan stops once each
+            // every vertex with unvisited active lanes; a row's scan stops once each
             // such lane has found a parent
-            for (int64_t v = gwarp; v < n; v += nwarps) {
-                uint64_t cl = 0ull;
-                if (lane < K) cl = s_act[lane] & ~__ldcg(&a.vis[v * K + lane]);
-                if (!__ballot_sync(0xffffffffu, cl != 0ull)) continue;
-                uint64_t nbl = 0ull;
-                const int64_t e0 = irp[v], e1 = irp[v + 1];
-                for (int64_t base = e0; base < e1; base += 32) {
-                    const int64_t e = base + lane;
-                    uint64_t f[K];
-                    if (e < e1) {
-                        load_words<K>(fcur + (int64_t)(a.icol[e] - vlo) * K, f);
-                    } else {
+            for (int b = blockIdx.x; b < nbig; b += gridDim.x) {  // rows above kBigRow: a block each
+                const int64_t v = (int64_t)a.big[b] - vlo;
+                if (v < 0 || v >= n) continue;  // (the same for the whole block)
+                const uint64_t c = actw & ~__ldcg(&a.vis[v * K + w]);
+                if (threadIdx.x < K) s_or[threadIdx.x] = 0ull;
+                if (!__syncthreads_or(c != 0ull)) continue;
+                uint64_t nb = 0ull;
+                const int64_t e1 = irp[v + 1];
+                for (int64_t e = irp[v] + threadIdx.x / K; e < e1 && (c & ~nb); e += 4 * EB) {
+                    int32_t u[4];
 #pragma unroll
-                        for (int w = 0; w < K; ++w) f[w] = 0ull;
-                    }
+                    for (int q = 0; q < 4; ++q) u[q] = e + q * EB < e1 ? a.icol[e + q * EB] - vlo : -1;
 #pragma unroll
-                    for (int w = 0; w < K; ++w) {
-                        const uint64_t r = warp_or64(f[w]);
-                        if (lane == w) nbl |= r & cl;
-                    }
-                    if (__all_sync(0xffffffffu, nbl == cl)) break;
+                    for (int q = 0; q < 4; ++q)
+                        if (u[q] >= 0) nb |= __ldcg(&fcur[(int64_t)u[q] * K + w]);
                 }
-                if (lane < K && nbl) fnext[v * K + lane] = nbl;
-                if (__ballot_sync(0xffffffffu, nbl != 0ull) && lane == 0) {
-                    if (e1 - e0 > 32) qnext[n - 1 - atomicAdd(qh_next, 1)] = (int32_t)v;
-                    else qnext[atomicAdd(qn_next, 1)] = (int32_t)v;
+                nb &= c;
+                if (nb) atomicOr(&s_or[w], (unsigned long long)nb);
+                __syncthreads();
+                if (threadIdx.x < K && s_or[threadIdx.x]) fnext[v * K + threadIdx.x] = s_or[threadIdx.x];
+                __syncthreads();
+            }
+            for (int64_t vb = gwarp * GW; vb < n; vb += nwarps * GW) {
+                const int64_t v = vb + lane / kGroupLanes;
+                uint64_t c = 0ull;
+                if (v < n) c = actw & ~__ldcg(&a.vis[v * K + w]);
+                const bool some = (__ballot_sync(0xffffffffu, c != 0ull) & gmask) != 0u;
+                int64_t e0 = 0, e1 = 0;
+                if (some) {
+                    e0 = irp[v];
+                    e1 = irp[v + 1];
+                    if (e1 - e0 > kBigRow) e1 = e0;  // above
+                }
+                const bool mid = e1 - e0 > kMidRow;
+                uint64_t nb = 0ull;
+                for (int64_t e = e0 + (lane % kGroupLanes) / K;; e += 4 * SUB) {
+                    const bool go = !mid && e < e1 && (SUB > 1 || (c & ~nb) != 0ull);
+                    if (!__any_sync(0xffffffffu, go)) break;
+                    int32_t u[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) u[q] = go && e + q * SUB < e1 ? a.icol[e + q * SUB] - vlo : -1;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (u[q] >= 0) nb |= __ldcg(&fcur[(int64_t)u[q] * K + w]);
+                }
+#pragma unroll
+                for (int o = K; o < kGroupLanes; o <<= 1) nb |= __shfl_xor_sync(0xffffffffu, nb, o);
+                nb &= c;
+                if (nb && lane % kGroupLanes < K) fnext[v * K + w] = nb;
+                for (unsigned mm = __ballot_sync(0xffffffffu, mid && lane % kGroupLanes == 0); mm; mm &= mm - 1) {
+                    const int src = __ffs(mm) - 1;  // a row of middle length, by the whole warp
+                    const int64_t f0 = __shfl_sync(0xffffffffu, e0, src), f1 = __shfl_sync(0xffffffffu, e1, src);
+                    const uint64_t cm = shfl64(c, src + w);
+                    uint64_t mb = 0ull;
+                    for (int64_t e = f0 + lane / K; __any_sync(0xffffffffu, e < f1 && (cm & ~mb)); e += 4 * EW) {
+                        int32_t u[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) u[q] = e + q * EW < f1 ? a.icol[e + q * EW] - vlo : -1;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (u[q] >= 0) mb |= __ldcg(&fcur[(int64_t)u[q] * K + w]);
+                    }
+#pragma unroll
+                    for (int o = K; o < 32; o <<= 1) mb |= __shfl_xor_sync(0xffffffffu, mb, o);
+                    mb &= cm;
+                    if (mb && lane < K) fnext[(vb + src / kGroupLanes) * K + w] = mb;
                 }
             }
         }
+        // full traversal: the counts of level L, whose frontier is settled, meanwhile
+        if (a.full && L > 0)
+            count_level<K, INSTR, SM>(a, n, vlo, irp, L, qcur, qn, qcur + (n - 1), qh, true, nullptr, &ovf, n_s);
         if (!grid_sync(bar, status, a.budget_ns)) return false;
         if (tid == 0 && L < 32) ctl->lvl_rec[L][4] = globaltimer_ns() - ctl->t_start;
 
-        if (push) {
-            // collect the vertices that gained frontier bits into the next queue
-            // (warp-aggregated appends; each vertex is looked at by one thread)
-            for (int64_t vb = gwarp * 32; vb < n; vb += nwarps * 32) {
-                const int64_t v = vb + lane;
-                bool any = false;
-                if (v < n) {
-                    if (K == 1) {
-                        any = __ldcg(&fnext[v]) != 0ull;
-                    } else {
-                        uint64_t f[K];
-                        load_words<K>(fnext + v * K, f);
-#pragma unroll
-                        for (int w = 0; w < K; ++w) any |= f[w] != 0ull;
+        // ---- settle the new frontier: visited bits, non-empty lanes, the queue of its
+        // vertices, the next level's work estimates; the frontier after it starts empty
+        {
+            uint64_t ne = 0ull;
+            unsigned long long fe = 0ull, ue = 0ull;
+            uint64_t *f2 = L + 2 <= a.Lcap ? a.fh + (int64_t)(L + 2) * nk : nullptr;
+            int32_t *qn_next = &ctl->qn[(L + 1) & 1], *qh_next = &ctl->qh[(L + 1) & 1];
+            for (int64_t ib = gwarp * 32; ib < nk; ib += nwarps * 32) {
+                const int64_t it = ib + lane, v = it / K;
+                uint64_t fn = 0ull, un = 0ull;
+                if (it < nk) {
+                    fn = __ldcg(&fnext[it]);
+                    const uint64_t vv = __ldcg(&a.vis[it]) | fn;
+                    if (fn) a.vis[it] = vv;
+                    if (f2) f2[it] = 0ull;
+                    un = actw & ~vv;
+                    ne |= fn;
+                }
+                const unsigned fm = __ballot_sync(0xffffffffu, fn != 0ull), um = __ballot_sync(0xffffffffu, un != 0ull);
+                const unsigned km = (K == 32 ? 0xffffffffu : ((1u << K) - 1u)) << (lane & ~(K - 1));
+                bool light = false, heavy = false;
+                if (w == 0 && (((fm | um) & km) != 0u)) {
+                    const int64_t din = irp[v + 1] - irp[v];
+                    ue += (unsigned long long)din * __popc(um & km);
+                    if (fm & km) {
+                        const int64_t dout = rp[v + 1] - rp[v];
+                        fe += (unsigned long long)dout * __popc(fm & km);
+                        heavy = din > 32 || dout > kLightOut;
+                        light = !heavy;
+                        if (INSTR) {
+                            n_uv += 1;
+                            n_ue += (unsigned long long)dout;
+                        }
                     }
                 }
-                const bool heavy = any && irp[v + 1] - irp[v] > 32;
-                const unsigned am = __ballot_sync(0xffffffffu, any && !heavy);
-                const unsigned hm = __ballot_sync(0xffffffffu, heavy);
-                if (am) {
-                    const int leader = __ffs(am) - 1;
-                    int pos = 0;
-                    if (lane == leader) pos = atomicAdd(qn_next, __popc(am));
-                    pos = __shfl_sync(0xffffffffu, pos, leader);
-                    if (any && !heavy) qnext[pos + __popc(am & ((1u << lane) - 1u))] = (int32_t)v;
-                }
-                if (hm) {
-                    const int leader = __ffs(hm) - 1;
-                    int pos = 0;
-                    if (lane == leader) pos = atomicAdd(qh_next, __popc(hm));
-                    pos = __shfl_sync(0xffffffffu, pos, leader);
-                    if (heavy) qnext[n - 1 - (pos + __popc(hm & ((1u << lane) - 1u)))] = (int32_t)v;
+                append(light, heavy, (int32_t)v, qnext, qn_next, qh_next, n, 0);
+                if (INSTR && fn) {
+                    const unsigned long long dg = (unsigned long long)(rp[v + 1] - rp[v]);
+                    uint64_t m2 = fn;
+                    while (m2) {
+                        const int b = __ffsll((long long)m2) - 1;
+                        m2 &= m2 - 1;
+                        atomicAdd(&a.levdeg[(int64_t)(64 * w + b) * (a.Lcap + 1) + L + 1], dg);
+                    }
                 }
             }
+            flush(qnext, qn_next, n);
+            if (ne) atomicOr(&s_nonempty[w], (unsigned long long)ne);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                fe += __shfl_xor_sync(0xffffffffu, fe, off);
+                ue += __shfl_xor_sync(0xffffffffu, ue, off);
+            }
+            if (lane == 0 && fe) atomicAdd(&ctl->fedges[(L + 1) & 1], fe);
+            if (lane == 0 && ue) atomicAdd(&ctl->uedges[(L + 1) & 1], ue);
         }
-        // mark settled targets
+        // settled targets
         if (!a.full) {
             for (long long p = p0 + tid; p < p1; p += nthreads) {
                 if (a.found[p] >= 0) continue;
@@ -403,256 +652,45 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 const int64_t q = (int64_t)t * K + (j >> 6);
                 if (((__ldcg(&a.vis[q]) | __ldcg(&fnext[q])) >> (j & 63)) & 1ull) {
                     a.found[p] = L + 1;
+                    atomicOr((unsigned long long *)&a.need[q], 1ull << (j & 63));
                     atomicSub(&a.remaining[j], 1);
                 }
             }
         }
-        if (!grid_sync(bar, status, a.budget_ns)) return false;
-        if (tid == 0 && L < 32) ctl->lvl_rec[L][5] = globaltimer_ns() - ctl->t_start;
-
-        // ---- phase A2: counts of level L+1.  A lane whose last targets were
-        // settled at this level retires after it, and of its level-(L+1)
-        // vertices only those targets are ever read (by the backtrack), so its
-        // counts are formed there alone.
-        if (a.full) {
-            if (threadIdx.x < K) s_cont[threadIdx.x] = s_act[threadIdx.x];
-        } else {
-            if (threadIdx.x < K) s_cont[threadIdx.x] = 0ull;
-            __syncthreads();
-            for (int j = threadIdx.x; j < W; j += blockDim.x) {
-                const bool c = ((s_act[j >> 6] >> (j & 63)) & 1ull) && __ldcg(&a.remaining[j]) > 0;
-                const unsigned bm = __ballot_sync(0xffffffffu, c);
-                if (lane == 0 && bm) atomicOr(&s_cont[j >> 6], (unsigned long long)bm << (j & 32));
-            }
-        }
-        __syncthreads();
-        const int64_t qn1 = (int64_t)ld_relaxed_u32((const uint32_t *)qn_next);
-        const int64_t qh1 = (int64_t)ld_relaxed_u32((const uint32_t *)qh_next);
-        if (!FPSIG) {
-            // in-degree > kBlockDeg: one block per (vertex, word), its warps
-            // splitting the edges; the partial sums meet in shared memory
-            // (integer sums, so the order does not matter)
-            for (int64_t hi = blockIdx.x; hi < qh1 * K; hi += gridDim.x) {
-                const int64_t h = hi / K;
-                const int w = (int)(hi - h * K);
-                const int32_t v = __ldcg(&qnext[n - 1 - h]);
-                const int64_t e0 = irp[v], e1 = irp[v + 1];
-                if (e1 - e0 <= kBlockDeg) continue;  // a warp item below; the same for the whole block
-                const uint64_t nbw = __ldcg(&fnext[(int64_t)v * K + w]) & s_cont[w];
-                if (nbw == 0ull) continue;
-                S acc0 = S(0), acc1 = S(0);
-                for (int64_t base = e0 + warp_in_block * 32; base < e1; base += kMsBlock) {
-                    const int64_t e = base + lane;
-                    int32_t u = 0;
-                    uint64_t fw = 0ull;
-                    if (e < e1) {
-                        u = a.icol[e] - vlo;
-                        fw = __ldcg(&fcur[(int64_t)u * K + w]) & nbw;
-                    }
-                    if (INSTR) n_sload += (unsigned long long)__popcll(fw);
-                    gather_chunk<SM, ST, S>(sig, W, w, fw, u, acc0, acc1, ovf);
-                }
-                s_red[warp_in_block][lane] = acc0;
-                s_red[warp_in_block][lane + 32] = acc1;
-                __syncthreads();
-                if (warp_in_block == 0) {
-                    S t0 = S(0), t1 = S(0);
-#pragma unroll
-                    for (int q = 0; q < kMsBlock / 32; ++q) {
-                        t0 += s_red[q][lane];
-                        t1 += s_red[q][lane + 32];
-                    }
-                    ovf |= (t0 >= (S)kLimit) | (t1 >= (S)kLimit);
-                    ST *drow = sig + (int64_t)v * W + 64 * w;
-                    if ((nbw >> lane) & 1ull) drow[lane] = (ST)t0;
-                    if ((nbw >> (lane + 32)) & 1ull) drow[lane + 32] = (ST)t1;
-                    if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
-                }
-                __syncthreads();
-            }
-        }
-        for (int64_t it = gwarp; it < qn1 + qh1 * K; it += nwarps) {
-            if (it < qn1) {
-                // in-degree <= 32: one warp per new vertex, its parents and all
-                // their words loaded once; lane w < K holds the word's lanes to count
-                const int32_t v = __ldcg(&qnext[it]);
-                uint64_t nbl = 0ull;
-                if (lane < K) nbl = __ldcg(&fnext[(int64_t)v * K + lane]) & s_cont[lane];
-                const unsigned wm = __ballot_sync(0xffffffffu, nbl != 0ull);
-                if (!wm) continue;
-                const int64_t e0 = irp[v], e1 = irp[v + 1];
-                ST *drow = sig + (int64_t)v * W;
-                const int64_t e = e0 + lane;
-                int32_t u = 0;
-                uint64_t f[K];
-                if (e < e1) {
-                    u = a.icol[e] - vlo;
-                    load_words<K>(fcur + (int64_t)u * K, f);
-                } else {
-#pragma unroll
-                    for (int w = 0; w < K; ++w) f[w] = 0ull;
-                }
-#pragma unroll
-                for (int w = 0; w < K; ++w) {
-                    if (!((wm >> w) & 1u)) continue;
-                    const uint64_t nbw = shfl64(nbl, w);
-                    const uint64_t fw = f[w] & nbw;
-                    if (INSTR) n_sload += (unsigned long long)__popcll(fw);
-                    S acc0 = S(0), acc1 = S(0);
-                    gather_chunk<SM, ST, S>(sig, W, w, fw, u, acc0, acc1, ovf);
-                    if (FPSIG) ovf |= (acc0 >= (S)kLimit) | (acc1 >= (S)kLimit);
-                    if ((nbw >> lane) & 1ull) drow[64 * w + lane] = (ST)acc0;
-                    if ((nbw >> (lane + 32)) & 1ull) drow[64 * w + lane + 32] = (ST)acc1;
-                    if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
-                }
-            } else {
-                // in-degree in (32, kBlockDeg] (any, for FP64 counts, whose
-                // additions keep the in-adjacency order): one warp per
-                // (vertex, word) over 32-edge chunks
-                const int64_t h = (it - qn1) / K;
-                const int w = (int)(it - qn1 - h * K);
-                const int32_t v = __ldcg(&qnext[n - 1 - h]);
-                const int64_t e0 = irp[v], e1 = irp[v + 1];
-                if (!FPSIG && e1 - e0 > kBlockDeg) continue;
-                const uint64_t nbw = __ldcg(&fnext[(int64_t)v * K + w]) & s_cont[w];
-                if (nbw == 0ull) continue;
-                S acc0 = S(0), acc1 = S(0);
-                for (int64_t base = e0; base < e1; base += 32) {
-                    const int64_t e = base + lane;
-                    int32_t u = 0;
-                    uint64_t fw = 0ull;
-                    if (e < e1) {
-                        u = a.icol[e] - vlo;
-                        fw = __ldcg(&fcur[(int64_t)u * K + w]) & nbw;
-                    }
-                    if (INSTR) n_sload += (unsigned long long)__popcll(fw);
-                    gather_chunk<SM, ST, S>(sig, W, w, fw, u, acc0, acc1, ovf);
-                }
-                if (FPSIG) ovf |= (acc0 >= (S)kLimit) | (acc1 >= (S)kLimit);
-                ST *drow = sig + (int64_t)v * W + 64 * w;
-                if ((nbw >> lane) & 1ull) drow[lane] = (ST)acc0;
-                if ((nbw >> (lane + 32)) & 1ull) drow[lane + 32] = (ST)acc1;
-                if (INSTR) n_swrite += lane == 0 ? (unsigned long long)__popcll(nbw) : 0ull;
-            }
-        }
-        if (!a.full) {
-            // targets of the retiring lanes: one warp per sample settled at L+1
-            for (long long p = p0 + gwarp; p < p1; p += nwarps) {
-                if (__ldcg(&a.found[p]) != L + 1) continue;
-                const int32_t j = a.samp_lane[p] - lane_base;
-                const int w = j >> 6;
-                const uint64_t bj = 1ull << (j & 63);
-                if (s_cont[w] & bj) continue;
-                const int32_t t = a.samp_t[p] - vlo;
-                const int64_t e0 = irp[t], e1 = irp[t + 1];
-                S acc = S(0);
-                if (FPSIG) {
-                    // in-adjacency order
-                    if (lane == 0)
-                        for (int64_t e = e0; e < e1; ++e) {
-                            const int32_t u = a.icol[e] - vlo;
-                            if (__ldcg(&fcur[(int64_t)u * K + w]) & bj) acc += (S)__ldcg(&sig[(int64_t)u * W + j]);
-                        }
-                } else {
-                    for (int64_t e = e0 + lane; e < e1; e += 32) {
-                        const int32_t u = a.icol[e] - vlo;
-                        if (__ldcg(&fcur[(int64_t)u * K + w]) & bj) {
-                            acc += (S)__ldcg(&sig[(int64_t)u * W + j]);
-                            if (INSTR) ++n_sload;
-                        }
-                    }
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                }
-                if (lane == 0) {
-                    ovf |= acc >= (S)kLimit;
-                    sig[(int64_t)t * W + j] = (ST)acc;
-                    if (INSTR) ++n_swrite;
-                }
-            }
-        }
-
-        // ---- phase B(1): settle the new frontier: visited bits, nonempty lanes,
-        // next frontier's out-edges (no reader of these runs in this interval)
-        {
-            unsigned long long fe = 0ull;
-            for (int64_t it = tid; it < (qn1 + qh1) * K; it += nthreads) {
-                const int64_t k = it / K;
-                const int w = (int)(it - k * K);
-                const int32_t v = __ldcg(&qnext[k < qn1 ? k : n - 1 - (k - qn1)]);
-                const uint64_t nb = __ldcg(&fnext[(int64_t)v * K + w]);
-                if (!nb) continue;
-                a.vis[(int64_t)v * K + w] = __ldcg(&a.vis[(int64_t)v * K + w]) | nb;
-                atomicOr(&s_nonempty[w], (unsigned long long)nb);
-                fe += (unsigned long long)(rp[v + 1] - rp[v]);
-                if (INSTR && w == 0) {
-                    n_uv += 1;
-                    n_ue += (unsigned long long)(rp[v + 1] - rp[v]);
-                }
-                if (INSTR) {
-                    const unsigned long long dg = (unsigned long long)(rp[v + 1] - rp[v]);
-                    uint64_t m2 = nb;
-                    while (m2) {
-                        const int b = __ffsll((long long)m2) - 1;
-                        m2 &= m2 - 1;
-                        atomicAdd(&a.levdeg[(int64_t)(64 * w + b) * (a.Lcap + 1) + L + 1], dg);
-                    }
-                }
-            }
-            // frontier out-edges for the direction choice
-            for (int off = 16; off > 0; off >>= 1) fe += __shfl_xor_sync(0xffffffffu, fe, off);
-            if (lane == 0 && fe) atomicAdd(&ctl->fedges[(L + 1) & 1], fe);
-            if (L + 2 <= a.Lcap) {
-                uint64_t *f2 = a.fh + (int64_t)(L + 2) * nk;
-                for (int64_t i = tid; i < nk; i += nthreads) f2[i] = 0ull;
-            }
-            if (a.policy == 2) {
-                // pull work of the next level: in-edges of every (vertex, word) that
-                // still has an unvisited active lane
-                unsigned long long ue = 0ull;
-                for (int64_t it = tid; it < nk; it += nthreads) {
-                    const int64_t v = it / K;
-                    const int w = (int)(it - v * K);
-                    const uint64_t vw = __ldcg(&a.vis[it]) | __ldcg(&fnext[it]);
-                    if (s_act[w] & ~vw) ue += (unsigned long long)(irp[v + 1] - irp[v]);
-                }
-                for (int off = 16; off > 0; off >>= 1) ue += __shfl_xor_sync(0xffffffffu, ue, off);
-                if (lane == 0 && ue) atomicAdd(&ctl->uedges[(L + 1) & 1], ue);
-            }
-        }
-        if (__any_sync(0xffffffffu, ovf) && lane == 0) atomicOr(status, SigmaMode<SM>::flag);
-        ovf = false;
         __syncthreads();
         if (threadIdx.x < K && s_nonempty[threadIdx.x])
             atomicOr(&ctl->nonempty[L & 1][threadIdx.x], s_nonempty[threadIdx.x]);
         __syncthreads();
-        __shared__ int s_last;
         if (threadIdx.x == 0) {
             __threadfence();
             s_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
         }
         __syncthreads();
         if (s_last) {
+            // the last block: lanes that go on (a new frontier, and a target left)
             __threadfence();
-            if (threadIdx.x < K) {
-                const int w = threadIdx.x;
-                uint64_t nact = s_act[w] & ld_relaxed_u64((const uint64_t *)&ctl->nonempty[L & 1][w]);
-                if (!a.full) {
-                    uint64_t m = nact;
-                    while (m) {
-                        const int b = __ffsll((long long)m) - 1;
-                        m &= m - 1;
-                        if (atomicAdd(&a.remaining[w * 64 + b], 0) <= 0) nact &= ~(1ull << b);
-                    }
+            if (threadIdx.x < K) s_or[threadIdx.x] = a.full ? ~0ull : 0ull;
+            __syncthreads();
+            if (!a.full) {
+                for (int j = threadIdx.x; j < W; j += blockDim.x) {
+                    const unsigned bm = __ballot_sync(0xffffffffu, __ldcg(&a.remaining[j]) > 0);
+                    if (lane == 0 && bm) atomicOr(&s_or[j >> 6], (unsigned long long)bm << (j & 32));
                 }
-                ctl->active[w] = nact;
-                ctl->nonempty[L & 1][w] = 0ull;
+                __syncthreads();
+            }
+            if (threadIdx.x < K) {
+                const uint64_t nact = s_act[threadIdx.x] & s_or[threadIdx.x] &
+                                      ld_relaxed_u64((const uint64_t *)&ctl->nonempty[L & 1][threadIdx.x]);
+                ctl->active[threadIdx.x] = nact;
+                ctl->nonempty[L & 1][threadIdx.x] = 0ull;
+                // lanes whose counts of level L+1 every vertex would need (a target is left)
+                if (!a.full) a.cont[(int64_t)(L + 1) * K + threadIdx.x] = s_act[threadIdx.x] & s_or[threadIdx.x];
             }
             if (threadIdx.x == 0) {
                 ctl->ticket = 0;
                 ctl->level = L + 1;
                 if (L < 32) {
-                    ctl->lvl_rec[L][0] = globaltimer_ns() - ctl->t_start;
+                    ctl->lvl_rec[L][0] = ctl->lvl_rec[L][5] = globaltimer_ns() - ctl->t_start;
                     ctl->lvl_rec[L][1] = (push ? 1ull : 0ull) | (ctl->uedges[L & 1] << 1);
                     ctl->lvl_rec[L][2] = (unsigned long long)(ctl->qn[L & 1] + ctl->qh[L & 1]);
                     ctl->lvl_rec[L][3] = ctl->fedges[L & 1];
@@ -670,23 +708,123 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         ++L;
         bool more = false;
 #pragma unroll
-        for (int w = 0; w < K; ++w) more |= ld_relaxed_u64((const uint64_t *)&ctl->active[w]) != 0ull;
+        for (int q = 0; q < K; ++q) more |= ld_relaxed_u64((const uint64_t *)&ctl->active[q]) != 0ull;
         if (!more) break;
         if (L + 1 > a.Lcap) {
             if (tid == 0) atomicOr(status, DEV_NEED_LEVELS);
             return false;
         }
     }
+
+    if (!a.full && L > 0) {
+        // ---- the vertices whose counts the samples' paths can need
+        const bool cone = !FPSIG && L <= (int)__ldg(a.lsafe);
+        const int64_t cap = a.ncap;
+        int64_t nl = 0, nh = 0;  // entries listed so far (deepest level first)
+        for (int l = L; cone && l >= 1; --l) {
+            const uint64_t *fl = a.fh + (int64_t)l * nk, *fp = a.fh + (int64_t)(l - 1) * nk;
+            auto mark_parents = [&](int64_t e, int64_t e1, int64_t stride, uint64_t b) {
+                for (; e < e1; e += 4 * stride) {
+                    int32_t u[4];
+                    uint64_t m[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) u[q] = e + q * stride < e1 ? a.icol[e + q * stride] - vlo : -1;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) m[q] = u[q] >= 0 ? b & __ldcg(&fp[(int64_t)u[q] * K + w]) : 0ull;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (m[q]) atomicOr((unsigned long long *)&a.need[(int64_t)u[q] * K + w], (unsigned long long)m[q]);
+                }
+            };
+            for (int b = blockIdx.x; l > 1 && b < nbig; b += gridDim.x) {  // rows above kBigRow: a block each
+                const int64_t v = (int64_t)a.big[b] - vlo;
+                if (v < 0 || v >= n) continue;
+                const uint64_t bits = __ldcg(&a.need[v * K + w]) & __ldcg(&fl[v * K + w]);
+                mark_parents(irp[v] + threadIdx.x / K, bits ? irp[v + 1] : 0, EB, bits);
+            }
+            for (int64_t ib = gwarp * GW; ib < n; ib += nwarps * GW) {
+                const int64_t v = ib + lane / kGroupLanes;
+                uint64_t bits = 0ull;
+                if (v < n) {
+                    bits = __ldcg(&a.need[v * K + w]);
+                    if (bits) bits &= __ldcg(&fl[v * K + w]);
+                }
+                const unsigned bm = __ballot_sync(0xffffffffu, bits != 0ull);
+                if (!bm) continue;
+                int64_t e0 = 0, e1 = 0;
+                if (bm & gmask) {
+                    e0 = irp[v];
+                    e1 = irp[v + 1];
+                }
+                const bool rep = (bm & gmask) && lane % kGroupLanes == 0;
+                append(rep && e1 - e0 <= 32, rep && e1 - e0 > 32, (int32_t)v, a.nlist + nl, &a.ncnt[2 * l],
+                       &a.ncnt[2 * l + 1], cap - nl, nh);
+                if (l == 1) continue;
+                if (e1 - e0 > kBigRow) e1 = e0;  // above
+                const bool mid = e1 - e0 > kMidRow;
+                mark_parents(e0 + (lane % kGroupLanes) / K, mid ? e0 : e1, SUB, bits);
+                for (unsigned mm = __ballot_sync(0xffffffffu, mid && lane % kGroupLanes == 0); mm; mm &= mm - 1) {
+                    const int src = __ffs(mm) - 1;
+                    const int64_t f0 = __shfl_sync(0xffffffffu, e0, src), f1 = __shfl_sync(0xffffffffu, e1, src);
+                    mark_parents(f0 + lane / K, f1, EW, shfl64(bits, src + w));
+                    __syncwarp();
+                }
+            }
+            flush(a.nlist + nl, &a.ncnt[2 * l], cap - nl);
+            if (!grid_sync(bar, status, a.budget_ns)) return false;
+            nl += __ldcg(&a.ncnt[2 * l]);
+            nh += __ldcg(&a.ncnt[2 * l + 1]);
+        }
+        // ---- their counts, level by level
+        if (cone && nl + nh <= cap) {
+            for (int l = 1; l <= L; ++l) {
+                const int64_t cl = __ldcg(&a.ncnt[2 * l]), ch = __ldcg(&a.ncnt[2 * l + 1]);
+                nl -= cl;
+                nh -= ch;
+                count_level<K, INSTR, SM>(a, n, vlo, irp, l, a.nlist + nl, cl, a.nlist + (cap - 1 - nh), ch, false,
+                                          nullptr, &ovf, n_s);
+                if (!grid_sync(bar, status, a.budget_ns)) return false;
+            }
+        } else {
+            // every vertex of the lanes that go on, and what is needed of the others: the
+            // vertices of a level are listed while the level before is counted
+            int32_t *dcnt = a.ncnt + 2 * (a.Lcap + 2);
+            for (int l = 0; l <= L; ++l) {
+                if (l < L) {
+                    const uint64_t *fl = a.fh + (int64_t)(l + 1) * nk;
+                    const uint64_t cw = cone ? 0ull : __ldcg(&a.cont[(int64_t)(l + 1) * K + w]);
+                    int32_t *q = (l & 1) ? a.fq1 : a.fq0, *qc = dcnt + 2 * (l + 1);
+                    for (int64_t ib = gwarp * GW; ib < n; ib += nwarps * GW) {
+                        const int64_t v = ib + lane / kGroupLanes;
+                        uint64_t bits = 0ull;
+                        if (v < n) bits = __ldcg(&fl[v * K + w]) & (cw | __ldcg(&a.need[v * K + w]));
+                        const bool rep = (__ballot_sync(0xffffffffu, bits != 0ull) & gmask) && lane % kGroupLanes == 0;
+                        const int64_t din = rep ? irp[v + 1] - irp[v] : 0;
+                        append(rep && din <= 32, rep && din > 32, (int32_t)v, q, &qc[0], &qc[1], n, 0);
+                    }
+                    flush(q, &qc[0], n);
+                }
+                if (l > 0) {
+                    const int32_t *q = (l & 1) ? a.fq0 : a.fq1;  // listed one round ago
+                    count_level<K, INSTR, SM>(a, n, vlo, irp, l, q, (int64_t)__ldcg(&dcnt[2 * l]), q + (n - 1),
+                                              (int64_t)__ldcg(&dcnt[2 * l + 1]), false,
+                                              cone ? nullptr : a.cont + (int64_t)l * K, &ovf, n_s);
+                }
+                if (!grid_sync(bar, status, a.budget_ns)) return false;
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, ovf) && lane == 0) atomicOr(status, SigmaMode<SM>::flag);
     if (INSTR) {
         for (int off = 16; off > 0; off >>= 1) {
-            n_sload += __shfl_xor_sync(0xffffffffu, n_sload, off);
-            n_swrite += __shfl_xor_sync(0xffffffffu, n_swrite, off);
+            n_s[0] += __shfl_xor_sync(0xffffffffu, n_s[0], off);
+            n_s[1] += __shfl_xor_sync(0xffffffffu, n_s[1], off);
             n_uv += __shfl_xor_sync(0xffffffffu, n_uv, off);
             n_ue += __shfl_xor_sync(0xffffffffu, n_ue, off);
         }
         if (lane == 0) {
-            atomicAdd(&a.counters[0], n_sload);
-            atomicAdd(&a.counters[1], n_swrite);
+            atomicAdd(&a.counters[0], n_s[0]);
+            atomicAdd(&a.counters[1], n_s[1]);
             atomicAdd(&a.counters[2], n_uv);
             atomicAdd(&a.counters[3], n_ue);
         }
@@ -827,19 +965,29 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
             const int64_t e0 = irp[w], e1 = irp[w + 1];
             S carry = S(0);
             int32_t pick = -1;
-            for (int64_t base = e0; base < e1 && pick < 0; base += 32) {
-                const int64_t e = base + lane;
-                int32_t pv = -1;
-                S val = S(0);
-                if (e < e1) {
-                    pv = a.icol[e] - vlo;
-                    if (__ldcg(&fprev[(int64_t)pv * K + wj]) & bj) val = (S)__ldcg(&sig[(int64_t)pv * W + j]);
+            // four chunks of 32 candidates in flight (a hub's row is thousands long)
+            for (int64_t base = e0; base < e1 && pick < 0; base += 128) {
+                int32_t pv[4];
+                S val[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int64_t e = base + 32 * q + lane;
+                    pv[q] = e < e1 ? a.icol[e] - vlo : -1;
                 }
-                // running sums are exact (integers; FP64 sums of integers below 2^53)
-                const S cum = carry + warp_incl_scan<S>(val);
-                const unsigned hit = __ballot_sync(0xffffffffu, val > S(0) && (double)cum >= target);
-                if (hit) pick = __shfl_sync(0xffffffffu, pv, __ffs(hit) - 1);
-                carry = __shfl_sync(0xffffffffu, cum, 31);
+                bool at[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) at[q] = pv[q] >= 0 && (__ldcg(&fprev[(int64_t)pv[q] * K + wj]) & bj);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) val[q] = at[q] ? (S)__ldcg(&sig[(int64_t)pv[q] * W + j]) : S(0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (pick >= 0 || !__any_sync(0xffffffffu, at[q])) continue;
+                    // running sums are exact (integers; FP64 sums of integers below 2^53)
+                    const S cum = carry + warp_incl_scan<S>(val[q]);
+                    const unsigned hit = __ballot_sync(0xffffffffu, val[q] > S(0) && (double)cum >= target);
+                    if (hit) pick = __shfl_sync(0xffffffffu, pv[q], __ffs(hit) - 1);
+                    carry = __shfl_sync(0xffffffffu, cum, 31);
+                }
             }
             if (pick < 0) {
                 if (lane == 0) atomicOr(status, DEV_BAD_PATH);
@@ -865,7 +1013,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
 // the grouping left in device memory (W lanes each, so a phase needs no host
 // round trip), or are the single batch given in the arguments.
 template <int K, bool INSTR, int SM>
-__global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(MsArgs a) {
+__global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ MsArgs a) {
     constexpr int W = 64 * K;
     MsCtl *ctl = a.ctl;
     GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
@@ -974,7 +1122,94 @@ percis_status launch_ms_k(percis_ctx *ctx, int K, MsArgs &a) {
     }
 }
 
-percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr) {
+// Number of walks of length k that end at a vertex, one step: next[v] += cur[u] over
+// the out-edges u -> v, and the largest entry of cur (k = 1: in-degrees) in *wmax.
+__global__ void k_walk_step(const int64_t *rp, const int32_t *col, int64_t n, const double *cur, double *next,
+                            unsigned long long *wmax) {
+    const int lane = threadIdx.x & 31, g = lane >> 3;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    unsigned long long m = 0ull;
+    for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; u0 < n; u0 += warps * 4) {
+        const int64_t u = u0 + g;
+        if (u >= n) continue;
+        const double c = cur[u];
+        m = max(m, (unsigned long long)__double_as_longlong(c));
+        if (!next || c == 0.0) continue;
+        const int64_t e1 = rp[u + 1];
+        for (int64_t e = rp[u] + (lane & 7); e < e1; e += 8) atomicAdd(&next[col[e]], c);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0 && m) atomicMax(wmax, m);
+}
+
+// in-degrees (the walks of length 1), or the vertices of in-degree > kBigRow
+__global__ void k_in_rows(const int64_t *irp, int64_t n, double *deg, int32_t *big, int32_t *nbig) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        const int64_t d = irp[v + 1] - irp[v];
+        if (deg) deg[v] = (double)d;
+        else if (d > kBigRow) big[atomicAdd(nbig, 1)] = (int32_t)v;
+    }
+}
+
+// The levels up to which no path count can reach 2^53: a count at level 4 q + r is at
+// most (walks of length 4)^q (walks of length r), each the largest over the vertices.
+__global__ void k_safe_levels(const unsigned long long *wmax, int32_t *lsafe) {
+    if (threadIdx.x != 0) return;
+    double w[5];
+    w[0] = 1.0;
+    for (int k = 1; k <= 4; ++k) w[k] = __longlong_as_double((long long)wmax[k]);
+    double p = 1.0;
+    int L = 0;
+    while (L < 4096 && p * w[4] < 0x1p52) {
+        if (w[4] < 2.0) {  // 0 or 1: the product stays
+            L = 4096;
+            break;
+        }
+        p *= w[4];
+        L += 4;
+    }
+    int r = 0;
+    while (r < 3 && p * w[r + 1] < 0x1p52) ++r;
+    *lsafe = L + r;
+}
+
+// The loaded graph's long in-rows, and for sampling phases the levels no count can
+// pass 2^53 in, on first use by a batched launch.
+percis_status prep_ms_graph(percis_ctx *ctx, bool full) {
+    const int64_t n = ctx->n;
+    const int64_t *irp = ctx->directed ? ctx->irp.as<int64_t>() : ctx->rp.as<int64_t>();
+    const int g = grid_for(ctx, n, 256);
+    PERCIS_TRY(ensure(ctx, ctx->ms_big, 64 + sizeof(int32_t) * (ctx->nnz / kBigRow + 1), "long rows"));
+    int32_t *nbig = ctx->ms_big.as<int32_t>(), *lsafe = nbig + 1;
+    unsigned long long *wmax = reinterpret_cast<unsigned long long *>(nbig + 2);  // [1..4] of five
+    if (!ctx->ms_rows_ready) {
+        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_big.p, 0, 64, ctx->stream));
+        k_in_rows<<<g, 256, 0, ctx->stream>>>(irp, n, nullptr, nbig + 16, nbig);
+        PERCIS_CHECK_LAUNCH(ctx, "long rows");
+        ctx->ms_rows_ready = true;
+    }
+    if (full || ctx->ms_walks_ready) return PERCIS_OK;
+    PERCIS_TRY(ensure(ctx, ctx->ms_walks, sizeof(double) * 2 * n, "walk counts"));
+    double *wa = ctx->ms_walks.as<double>(), *wb = wa + n;
+    k_in_rows<<<g, 256, 0, ctx->stream>>>(irp, n, wa, nullptr, nullptr);
+    PERCIS_CHECK_LAUNCH(ctx, "in-degrees");
+    for (int k = 1; k <= 4; ++k) {
+        if (k < 4) PERCIS_CUDA(ctx, cudaMemsetAsync(wb, 0, sizeof(double) * n, ctx->stream));
+        k_walk_step<<<grid_for(ctx, n * 8, 256), 256, 0, ctx->stream>>>(ctx->rp.as<int64_t>(), ctx->col.as<int32_t>(),
+                                                                      n, wa, k < 4 ? wb : nullptr, wmax + k);
+        PERCIS_CHECK_LAUNCH(ctx, "walk counts");
+        std::swap(wa, wb);
+    }
+    k_safe_levels<<<1, 32, 0, ctx->stream>>>(wmax, lsafe);
+    PERCIS_CHECK_LAUNCH(ctx, "walk bound");
+    ctx->ms_walks_ready = true;
+    return PERCIS_OK;
+}
+
+percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr, bool full) {
     const int64_t n = nr;  // vertices of the largest launch range
     const int K = W / 64;
     PERCIS_TRY(ensure(ctx, ctx->fq0, sizeof(int32_t) * n, "frontier queue"));
@@ -982,13 +1217,27 @@ percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr) {
     PERCIS_TRY(ensure(ctx, ctx->vis, sizeof(uint64_t) * n * K, "visited bits"));
     PERCIS_TRY(ensure(ctx, ctx->fhist, sizeof(uint64_t) * n * K * (int64_t)(Lcap + 1), "frontier history"));
     PERCIS_TRY(ensure(ctx, ctx->sigmaW, sizeof(double) * n * W, "lane sigma"));
+    if (!full) {
+        PERCIS_TRY(ensure(ctx, ctx->ms_need, sizeof(uint64_t) * n * K, "needed lanes"));
+        PERCIS_TRY(ensure(ctx, ctx->ms_list, sizeof(int32_t) * 2 * n, "needed vertices"));
+        PERCIS_TRY(ensure(ctx, ctx->ms_levels, (sizeof(int32_t) * 4 + sizeof(uint64_t) * K) * (size_t)(Lcap + 2),
+                          "level counts"));
+    }
     PERCIS_TRY(ensure(ctx, ctx->remaining, sizeof(int32_t) * 512, "lane remaining"));
     PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl), "ms ctl"));
     return PERCIS_OK;
 }
 
-void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap) {
+void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
     a.n = ctx->n;
+    a.big_count = ctx->ms_big.as<int32_t>();
+    a.lsafe = a.big_count + 1;
+    a.big = a.big_count + 16;
+    a.need = ctx->ms_need.as<uint64_t>();
+    a.nlist = ctx->ms_list.as<int32_t>();
+    a.ncap = 2 * nr;
+    a.cont = ctx->ms_levels.as<uint64_t>();
+    a.ncnt = reinterpret_cast<int32_t *>(a.cont + (size_t)(Lcap + 2) * K);
     a.irp = ctx->directed ? ctx->irp.as<int64_t>() : ctx->rp.as<int64_t>();
     a.icol = ctx->directed ? ctx->icol.as<int32_t>() : ctx->col.as<int32_t>();
     a.vis = ctx->vis.as<uint64_t>();
@@ -1045,7 +1294,8 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
         const int64_t lmem = (16ll << 30) / std::max<int64_t>(1, nr_max * K * 8) - 1;
         Lcap = (int)std::max<int64_t>(Lcap, std::min<int64_t>(ctx->vertex_diam + 3, std::min<int64_t>(lmem, 1 << 20)));
     }
-    PERCIS_TRY(ensure_ms(ctx, W, Lcap, nr_max));
+    PERCIS_TRY(prep_ms_graph(ctx, false));
+    PERCIS_TRY(ensure_ms(ctx, W, Lcap, nr_max, false));
     ctx->levels_alloc = Lcap;
     ctx->lanes_alloc = W;
     PERCIS_TRY(ensure(ctx, ctx->found, sizeof(int32_t) * (count + 1), "found"));
@@ -1053,7 +1303,7 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
     const int64_t B = ctx->multi ? (int64_t)plan.size() : (n_sources + W - 1) / W;
     *batches = B;
     MsArgs a{};
-    fill_common(ctx, a, Lcap);
+    fill_common(ctx, a, Lcap, K, nr_max);
     a.lane_src = ctx->lane_src.as<int32_t>();
     a.lane_off = ctx->lane_off.as<long long>();
     a.samp_t = ctx->samp_t.as<int32_t>();
@@ -1131,11 +1381,12 @@ percis_status msbfs_full(percis_ctx *ctx, int32_t nsrc, const int32_t *sources, 
     const int K = W / 64;
     int Lcap = std::max(ctx->levels_alloc, 32);
     for (int attempt = 0; attempt < 12; ++attempt) {
-        PERCIS_TRY(ensure_ms(ctx, W, Lcap, ctx->n));
+        PERCIS_TRY(prep_ms_graph(ctx, true));
+        PERCIS_TRY(ensure_ms(ctx, W, Lcap, ctx->n, true));
         ctx->levels_alloc = Lcap;
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream));
         MsArgs a{};
-        fill_common(ctx, a, Lcap);
+        fill_common(ctx, a, Lcap, K, ctx->n);
         a.lane_src = sources;
         a.lane_base = 0;
         a.nlanes = nsrc;

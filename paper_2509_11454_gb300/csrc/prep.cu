@@ -899,6 +899,7 @@ percis_status prep_graph(percis_ctx *ctx) {
         ctx->graph_pending = true;
     }
     ctx->vorder_ready = false;  // built on first use by the batched form
+    ctx->ms_rows_ready = ctx->ms_walks_ready = false;
     if (!ctx->skip_diam) {
         int64_t D = 0;
         PERCIS_TRY(vertex_diam_ub(ctx, &D));

@@ -112,3 +112,33 @@ def test_plain_bfs_rows_and_levels(binding, directed, hub):
     if not directed:
         assert binding.percis_get_prep(eng.ctx)["vertex_diam"] == oracle.vertex_diam_ub(og)
     eng.close()
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("lanes,direction", [(64, 2), (128, 0), (256, 1), (512, 0), (512, 1)])
+def test_batched_rows_and_needed_counts(binding, lanes, direction, directed):
+    """The batched form where its work splits: rows around 32, 64 and 256 edges (a
+    vertex's eight lanes, a warp, a block), samples whose ancestors alone are counted
+    (short levels) and ones counted everywhere (a tail of 40 vertices beyond the levels
+    that are safe), against the oracle's one-sided samples."""
+    rng = np.random.default_rng(lanes)
+    src, dst, n = [], [], 0
+    for k in (31, 32, 33, 64, 65, 256, 257, 1500):  # stars, each hub tied to the next star
+        src += [np.full(k, n), [n + k], [n + k]]
+        dst += [np.arange(n + 1, n + k + 1), [n], [n + k + 1]]
+        n += k + 1
+    src += [rng.integers(0, n, 6 * n), np.arange(n, n + 40)]
+    dst += [rng.integers(0, n, 6 * n), np.arange(n + 1, n + 41)]
+    src.append([5])
+    dst.append([n])
+    n += 41
+    g = synth.csr_from_edges(n, np.concatenate(src), np.concatenate(dst), directed=directed)
+    x = synth.states_uniform(n, 2)
+    og, prep = oracle.from_synth(g), oracle.prepare(x)
+    eng = _engine(binding, g, x, lanes=lanes, direction=direction)
+    ph = eng.run_phase(7, 1, 400)
+    ref = oracle.run_samples(og, prep, 7, 1, 3, 0, 400, keep_paths=False)
+    assert not ref.overflow
+    for k in ("s", "t", "kind", "ilen", "cnt"):
+        assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
+    eng.close()
