@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(kPlainBlock, 1) k_plain_bfs(PlainArgs a) {
     if (a.kind && a.kind[a.idx] != 0) return;  // zero-weight pair: no path needed (uniform over the grid)
     __shared__ int s_cnt[3];  // block 0 alone: next frontier, its heavy rows, in-degree hubs
     __shared__ int s_found;
+    __shared__ int4 s_res;
     __shared__ double s_red[kPlainWarps];
     __shared__ int32_t s_buf[kPlainWarps][kClaimBuf];  // claimed vertices on their way to the frontier
     PlainCtl *ctl = a.ctl;
@@ -288,7 +289,9 @@ __global__ void __launch_bounds__(kPlainBlock, 1) k_plain_bfs(PlainArgs a) {
                 if (threadIdx.x == 0) ctl->solo[stint & 1] = make_int4(nq, nh, L, found);
             }
             if (!grid_sync(bar, status, a.budget_ns)) return;
-            const int4 res = __ldcg(&ctl->solo[stint & 1]);
+            if (threadIdx.x == 0) s_res = __ldcg(&ctl->solo[stint & 1]);  // (one request a block)
+            __syncthreads();
+            const int4 res = s_res;
             nq = res.x;
             nh = res.y;
             L = res.z;
@@ -315,10 +318,15 @@ __global__ void __launch_bounds__(kPlainBlock, 1) k_plain_bfs(PlainArgs a) {
             }
             expand(gw, nwarps, nq, L, cur, nxt, &ctl->qsize[nx], &ctl->hsize[nx], &ctl->nhub[nx]);
             if (!grid_sync(bar, status, a.budget_ns)) return;
-            nq = (int)ld_relaxed_u32((const uint32_t *)&ctl->qsize[nx]);
-            nh = (int)ld_relaxed_u32((const uint32_t *)&ctl->hsize[nx]);
+            if (threadIdx.x == 0)
+                s_res = make_int4((int)ld_relaxed_u32((const uint32_t *)&ctl->qsize[nx]),
+                                  (int)ld_relaxed_u32((const uint32_t *)&ctl->hsize[nx]),
+                                  (int)ld_relaxed_u32((const uint32_t *)&ctl->nhub[nx]), 0);
+            __syncthreads();
+            nq = s_res.x;
+            nh = s_res.y;
             if (!a.levels_only) {
-                const int nhub = (int)ld_relaxed_u32((const uint32_t *)&ctl->nhub[nx]);
+                const int nhub = s_res.z;
                 for (int64_t it = gw; it < (int64_t)nhub * kHeavyParts; it += nwarps) {
                     const double acc = hub_part(it / kHeavyParts, (int)(it % kHeavyParts), L);
                     if (lane == 0) a.part[it] = acc;
@@ -334,8 +342,11 @@ __global__ void __launch_bounds__(kPlainBlock, 1) k_plain_bfs(PlainArgs a) {
                     }
                     if (!grid_sync(bar, status, a.budget_ns)) return;
                 }
-                // (written between barriers of a grid level only)
-                found = (int)ld_relaxed_u32((const uint32_t *)&ctl->found);
+                if (t >= 0) {  // (written between barriers of a grid level only)
+                    if (threadIdx.x == 0) s_found = (int)ld_relaxed_u32((const uint32_t *)&ctl->found);
+                    __syncthreads();
+                    found = s_found;
+                }
             }
             ++L;
             ++step;

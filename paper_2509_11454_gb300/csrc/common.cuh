@@ -121,44 +121,56 @@ __device__ __forceinline__ int64_t ld_relaxed_s64(const int64_t *p) {
 }
 
 // ------------------------------------------------------------ grid barrier
-// Sense-by-generation barrier for cooperative launches (all blocks are
-// co-resident, so it cannot deadlock).  Every wait is bounded: after
-// budget_ns the waiting block sets DEV_TIMEOUT and every later barrier
-// returns false at once, so a kernel that sees `false` must exit.
-struct GridBarrier {
-    uint32_t count;
+// Barrier for cooperative launches (all blocks are co-resident, so it cannot
+// deadlock).  One 64-bit word counts arrivals and is never reset: an arrival that
+// finds `a` belongs to round a / blocks, which is over once the count reaches the
+// next multiple (a launch that ends without a timeout leaves a multiple, so the next
+// one may use the word as it stands, with any number of blocks only if it is zeroed).
+// A round costs one atomic and one polled acquire load, ~1.3 us over 608 blocks, where
+// separate arrival and generation words, full fences and a sleep between polls took
+// about 3 us more (batched estimate on Barabasi-Albert 100k 16.3 -> 16.0 ms, exact
+// centrality n = 3001 3.97 -> 3.80 ms).  Every wait is bounded: after
+// budget_ns the waiting block sets DEV_TIMEOUT and the word's top bit, which every
+// poll and later arrival sees, so that each barrier from there on returns false; a
+// kernel that sees `false` must exit.
+struct alignas(8) GridBarrier {
+    uint32_t count;  // low and high half of the arrivals
     uint32_t gen;
 };
 
 __device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, uint64_t budget_ns) {
     __shared__ int s_ok;
+    constexpr uint64_t kOver = 1ull << 63;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int ok = 1;
-        const uint32_t my_gen = ld_acquire_u32(&bar->gen);
-        __threadfence();
-        const uint32_t prev = atomicAdd(&bar->count, 1u);
-        if (prev == gridDim.x - 1) {
-            atomicExch(&bar->count, 0u);
-            __threadfence();
-            atomicAdd(&bar->gen, 1u);
-        } else {
-            const uint64_t t0 = globaltimer_ns();
-            while (ld_acquire_u32(&bar->gen) == my_gen) {
-                if (ld_relaxed_u32(status) & DEV_TIMEOUT) {
-                    ok = 0;
-                    break;
+        uint64_t *word = reinterpret_cast<uint64_t *>(bar);
+        uint64_t a;
+        // release: the block's writes (ordered before by the block barrier); acquire: for the last to arrive
+        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(a) : "l"(word), "l"(1ull) : "memory");
+        int ok = (a & kOver) == 0;
+        if (ok) {
+            const uint64_t g = gridDim.x;
+            const uint64_t round = a >> 32 ? a / g : (uint64_t)((uint32_t)a / (uint32_t)g);
+            const uint64_t target = (round + 1) * g;
+            if (a + 1 != target) {
+                const uint64_t t0 = globaltimer_ns();
+                for (;;) {
+                    uint64_t c;
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(word) : "memory");
+                    if (c & kOver) {
+                        ok = 0;
+                        break;
+                    }
+                    if (c >= target) break;
+                    if (globaltimer_ns() - t0 > budget_ns) {
+                        atomicOr(status, DEV_TIMEOUT);
+                        atomicOr(reinterpret_cast<unsigned long long *>(word), (unsigned long long)kOver);
+                        ok = 0;
+                        break;
+                    }
                 }
-                if (globaltimer_ns() - t0 > budget_ns) {
-                    atomicOr(status, DEV_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
             }
         }
-        __threadfence();
-        if (ld_relaxed_u32(status) & DEV_TIMEOUT) ok = 0;
         s_ok = ok;
     }
     __syncthreads();

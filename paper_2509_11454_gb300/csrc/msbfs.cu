@@ -43,6 +43,7 @@ constexpr int kGroupLanes = 8;      // lanes that share a vertex
 constexpr int64_t kMidRow = 64;     // rows above it: a whole warp
 constexpr int64_t kBigRow = 256;    // in-rows above it: a whole block (listed once per graph)
 constexpr int64_t kLightOut = 64;   // out-rows above it: a whole block
+constexpr int kBackChunks = 4;       // of 32 candidates, in flight in a backtrack step
 constexpr int kQueueBuf = 96;       // queue entries a warp gathers before it appends them
 constexpr int64_t kBlockDeg = PERCIS_BLOCK_DEG;  // in-degree above which a whole block counts one (vertex, word)
 
@@ -348,7 +349,8 @@ __device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo
 // anywhere can reach 2^53 (the number of walks of that length, *a.lsafe), so that
 // the overflow flag says the same; otherwise every vertex of a continuing lane is
 // counted, as in FP64 reruns.  Barabasi-Albert 100k, 512 lanes: 1.54 ms a batch
-// with counts everywhere (the gathers of the two largest levels), 0.70 ms.
+// with counts everywhere (the gathers of the two largest levels), 0.70 ms (0.57 with
+// the control words below read once a block).
 //
 // Eight lanes share a vertex, lane w mod K on its word w (8 / K edges side by side
 // for K < 8): an edge's K words are one coalesced access and the OR over a row
@@ -437,7 +439,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
     __shared__ unsigned long long s_act[K];
     __shared__ unsigned long long s_or[K];
     __shared__ int32_t s_q[kMsBlock / 32][kQueueBuf];
-    __shared__ int s_last;
+    __shared__ int s_last, s_ctl[3];
 
     // append the vertices of lanes with `any` (light from the front, heavy from the
     // back); a warp's light ones go out in runs.  Every lane of the warp calls it.
@@ -467,23 +469,32 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
 
     int L = 0;
     for (;;) {
+        // the level's control words, read by one warp of the block (every warp reading
+        // them queued 40,000 requests at one L2 line, 8 to 17 us after each barrier)
         if (threadIdx.x < K) {
             s_nonempty[threadIdx.x] = 0ull;
             s_act[threadIdx.x] = ld_relaxed_u64((const uint64_t *)&ctl->active[threadIdx.x]);
+        } else if (threadIdx.x == K) {
+            s_ctl[0] = (int)ld_relaxed_u32((const uint32_t *)&ctl->push_next);
+            s_ctl[1] = (int)ld_relaxed_u32((const uint32_t *)&ctl->qn[L & 1]);
+            s_ctl[2] = (int)ld_relaxed_u32((const uint32_t *)&ctl->qh[L & 1]);
         }
         __syncthreads();
         unsigned long long any_act = 0ull;
 #pragma unroll
         for (int q = 0; q < K; ++q) any_act |= s_act[q];
         if (!any_act) break;  // (the same in every block)
+        if (L + 1 > a.Lcap) {
+            if (tid == 0) atomicOr(status, DEV_NEED_LEVELS);
+            return false;
+        }
         const uint64_t actw = s_act[w];
         const uint64_t *fcur = a.fh + (int64_t)L * nk;
         uint64_t *fnext = a.fh + (int64_t)(L + 1) * nk;
         const int32_t *qcur = (L & 1) ? a.fq1 : a.fq0;
         int32_t *qnext = (L & 1) ? a.fq0 : a.fq1;
-        const bool push = ld_relaxed_u32((const uint32_t *)&ctl->push_next) != 0u;
-        const int64_t qn = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qn[L & 1]);
-        const int64_t qh = (int64_t)ld_relaxed_u32((const uint32_t *)&ctl->qh[L & 1]);
+        const bool push = s_ctl[0] != 0;
+        const int64_t qn = s_ctl[1], qh = s_ctl[2];
 
         // ---- discover level L+1 (frontier bits only)
         if (push) {
@@ -706,14 +717,6 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         }
         if (!grid_sync(bar, status, a.budget_ns)) return false;
         ++L;
-        bool more = false;
-#pragma unroll
-        for (int q = 0; q < K; ++q) more |= ld_relaxed_u64((const uint64_t *)&ctl->active[q]) != 0ull;
-        if (!more) break;
-        if (L + 1 > a.Lcap) {
-            if (tid == 0) atomicOr(status, DEV_NEED_LEVELS);
-            return false;
-        }
     }
 
     if (!a.full && L > 0) {
@@ -721,6 +724,12 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         const bool cone = !FPSIG && L <= (int)__ldg(a.lsafe);
         const int64_t cap = a.ncap;
         int64_t nl = 0, nh = 0;  // entries listed so far (deepest level first)
+        auto counts_at = [&](const int32_t *p) -> int2 {  // {light, heavy}, one request a block
+            __syncthreads();
+            if (threadIdx.x < 2) s_ctl[threadIdx.x] = __ldcg(&p[threadIdx.x]);
+            __syncthreads();
+            return make_int2(s_ctl[0], s_ctl[1]);
+        };
         for (int l = L; cone && l >= 1; --l) {
             const uint64_t *fl = a.fh + (int64_t)l * nk, *fp = a.fh + (int64_t)(l - 1) * nk;
             auto mark_parents = [&](int64_t e, int64_t e1, int64_t stride, uint64_t b) {
@@ -772,16 +781,17 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
             }
             flush(a.nlist + nl, &a.ncnt[2 * l], cap - nl);
             if (!grid_sync(bar, status, a.budget_ns)) return false;
-            nl += __ldcg(&a.ncnt[2 * l]);
-            nh += __ldcg(&a.ncnt[2 * l + 1]);
+            const int2 c = counts_at(a.ncnt + 2 * l);
+            nl += c.x;
+            nh += c.y;
         }
         // ---- their counts, level by level
         if (cone && nl + nh <= cap) {
             for (int l = 1; l <= L; ++l) {
-                const int64_t cl = __ldcg(&a.ncnt[2 * l]), ch = __ldcg(&a.ncnt[2 * l + 1]);
-                nl -= cl;
-                nh -= ch;
-                count_level<K, INSTR, SM>(a, n, vlo, irp, l, a.nlist + nl, cl, a.nlist + (cap - 1 - nh), ch, false,
+                const int2 c = counts_at(a.ncnt + 2 * l);
+                nl -= c.x;
+                nh -= c.y;
+                count_level<K, INSTR, SM>(a, n, vlo, irp, l, a.nlist + nl, c.x, a.nlist + (cap - 1 - nh), c.y, false,
                                           nullptr, &ovf, n_s);
                 if (!grid_sync(bar, status, a.budget_ns)) return false;
             }
@@ -806,8 +816,8 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 }
                 if (l > 0) {
                     const int32_t *q = (l & 1) ? a.fq0 : a.fq1;  // listed one round ago
-                    count_level<K, INSTR, SM>(a, n, vlo, irp, l, q, (int64_t)__ldcg(&dcnt[2 * l]), q + (n - 1),
-                                              (int64_t)__ldcg(&dcnt[2 * l + 1]), false,
+                    const int2 c = counts_at(dcnt + 2 * l);
+                    count_level<K, INSTR, SM>(a, n, vlo, irp, l, q, c.x, q + (n - 1), c.y, false,
                                               cone ? nullptr : a.cont + (int64_t)l * K, &ovf, n_s);
                 }
                 if (!grid_sync(bar, status, a.budget_ns)) return false;
@@ -965,22 +975,22 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
             const int64_t e0 = irp[w], e1 = irp[w + 1];
             S carry = S(0);
             int32_t pick = -1;
-            // four chunks of 32 candidates in flight (a hub's row is thousands long)
-            for (int64_t base = e0; base < e1 && pick < 0; base += 128) {
-                int32_t pv[4];
-                S val[4];
+            // kBackChunks chunks of 32 candidates in flight (a hub's row is thousands long)
+            for (int64_t base = e0; base < e1 && pick < 0; base += 32 * kBackChunks) {
+                int32_t pv[kBackChunks];
+                S val[kBackChunks];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < kBackChunks; ++q) {
                     const int64_t e = base + 32 * q + lane;
                     pv[q] = e < e1 ? a.icol[e] - vlo : -1;
                 }
-                bool at[4];
+                bool at[kBackChunks];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) at[q] = pv[q] >= 0 && (__ldcg(&fprev[(int64_t)pv[q] * K + wj]) & bj);
+                for (int q = 0; q < kBackChunks; ++q) at[q] = pv[q] >= 0 && (__ldcg(&fprev[(int64_t)pv[q] * K + wj]) & bj);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) val[q] = at[q] ? (S)__ldcg(&sig[(int64_t)pv[q] * W + j]) : S(0);
+                for (int q = 0; q < kBackChunks; ++q) val[q] = at[q] ? (S)__ldcg(&sig[(int64_t)pv[q] * W + j]) : S(0);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < kBackChunks; ++q) {
                     if (pick >= 0 || !__any_sync(0xffffffffu, at[q])) continue;
                     // running sums are exact (integers; FP64 sums of integers below 2^53)
                     const S cum = carry + warp_incl_scan<S>(val[q]);
@@ -1131,12 +1141,23 @@ __global__ void k_walk_step(const int64_t *rp, const int32_t *col, int64_t n, co
     unsigned long long m = 0ull;
     for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; u0 < n; u0 += warps * 4) {
         const int64_t u = u0 + g;
-        if (u >= n) continue;
-        const double c = cur[u];
+        const double c = u < n ? cur[u] : 0.0;
         m = max(m, (unsigned long long)__double_as_longlong(c));
-        if (!next || c == 0.0) continue;
-        const int64_t e1 = rp[u + 1];
-        for (int64_t e = rp[u] + (lane & 7); e < e1; e += 8) atomicAdd(&next[col[e]], c);
+        int64_t e0 = 0, e1 = 0;
+        if (next && c != 0.0) {
+            e0 = rp[u];
+            e1 = rp[u + 1];
+        }
+        const bool big = e1 - e0 > kMidRow;  // by the whole warp below
+        for (int64_t e = e0 + (lane & 7); e < e1 && !big; e += 8) atomicAdd(&next[col[e]], c);
+        for (unsigned b = __ballot_sync(0xffffffffu, big && (lane & 7) == 0); b; b &= b - 1) {
+            const int src = __ffs(b) - 1;
+            const int64_t f0 = __shfl_sync(0xffffffffu, e0, src), f1 = __shfl_sync(0xffffffffu, e1, src);
+            const double fc = __shfl_sync(0xffffffffu, c, src);
+#pragma unroll 4
+            for (int64_t e = f0 + lane; e < f1; e += 32) atomicAdd(&next[col[e]], fc);
+            __syncwarp();
+        }
     }
     __syncwarp();
 #pragma unroll
@@ -1253,7 +1274,7 @@ void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
     a.fq0 = ctx->fq0.as<int32_t>();
     a.fq1 = ctx->fq1.as<int32_t>();
     a.policy = ctx->opt.direction;
-    a.push_alpha = ctx->opt.push_alpha > 0.0 ? ctx->opt.push_alpha : 0.5;
+    a.push_alpha = ctx->opt.push_alpha > 0.0 ? ctx->opt.push_alpha : 1.0;
 }
 
 }  // namespace
