@@ -784,25 +784,45 @@ __global__ void k_groups(const double *xs, int64_t n, int32_t *glo, int32_t *ghi
 // ------------------------------------------------------------- transpose
 
 // key(v) = (highest-degree out-neighbour of v, ties to the smallest id) << 32 | v;
-// vertices without neighbours use themselves.
+// vertices without neighbours use themselves.  Eight lanes to a row, all of the warp
+// to rows above 64 edges (one thread a row left a hub's thousands of dependent loads to
+// one thread: Barabasi-Albert 100k 735 us, 114 us).
 __global__ void k_hub_keys(const int64_t *rp, const int32_t *col, int64_t n, uint64_t *keys, int32_t *vals) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        int32_t best = (int32_t)v;
-        int64_t bdeg = -1;
-        for (int64_t e = rp[v]; e < rp[v + 1]; ++e) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // largest (degree, ~id) of the row's neighbours e, e + step, ...
+    auto best_of = [&](int64_t e, int64_t e1, int64_t step) {
+        unsigned long long m = 0ull;
+        for (; e < e1; e += step) {
             const int32_t u = col[e];
-            const int64_t d = rp[u + 1] - rp[u];
-            if (d > bdeg || (d == bdeg && u < best)) {
-                bdeg = d;
-                best = u;
-            }
+            m = max(m, ((unsigned long long)(rp[u + 1] - rp[u]) << 32) | (0xffffffffu - (uint32_t)u));
         }
-        keys[v] = ((uint64_t)(uint32_t)best << 32) | (uint32_t)v;
-        vals[v] = (int32_t)v;
+        return m;
+    };
+    for (int64_t v0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; v0 < n; v0 += warps * 4) {
+        const int64_t v = v0 + (lane >> 3);
+        const int64_t e0 = v < n ? rp[v] : 0, e1 = v < n ? rp[v + 1] : 0;
+        const bool big = e1 - e0 > 64;
+        unsigned long long m = big ? 0ull : best_of(e0 + (lane & 7), e1, 8);
+        __syncwarp();
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        for (unsigned b = __ballot_sync(0xffffffffu, big && (lane & 7) == 0); b; b &= b - 1) {
+            const int src = __ffs(b) - 1;
+            unsigned long long w =
+                best_of(__shfl_sync(0xffffffffu, e0, src) + lane, __shfl_sync(0xffffffffu, e1, src), 32);
+            __syncwarp();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) w = max(w, __shfl_xor_sync(0xffffffffu, w, o));
+            if (lane == src) m = w;
+        }
+        if (v < n && (lane & 7) == 0) {
+            const uint32_t best = e1 > e0 ? 0xffffffffu - (uint32_t)m : (uint32_t)v;
+            keys[v] = ((uint64_t)best << 32) | (uint32_t)v;
+            vals[v] = (int32_t)v;
+        }
     }
 }
-
 
 }  // namespace
 
@@ -811,30 +831,19 @@ __global__ void k_hub_keys(const int64_t *rp, const int32_t *col, int64_t n, uin
 percis_status prep_vorder(percis_ctx *ctx) {
     if (ctx->vorder_ready) return PERCIS_OK;
     const int64_t n = ctx->n;
-    {
-        PERCIS_TRY(ensure(ctx, ctx->vorder, sizeof(int32_t) * n, "vertex order"));
-        DevBuf k1, k2, v2;
-        cudaError_t e = cudaMalloc(&k1.p, sizeof(uint64_t) * n);
-        if (e == cudaSuccess) e = cudaMalloc(&k2.p, sizeof(uint64_t) * n);
-        if (e == cudaSuccess) e = cudaMalloc(&v2.p, sizeof(int32_t) * n);
-        percis_status rs = PERCIS_OK;
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            rs = set_err(ctx, PERCIS_E_OOM, "vertex order scratch");
-        } else {
-            k_hub_keys<<<grid_for(ctx, n, 256), 256, 0, ctx->stream>>>(ctx->rp.as<int64_t>(), ctx->col.as<int32_t>(),
-                                                                     n, k1.as<uint64_t>(), ctx->vorder.as<int32_t>());
-            ctx->launches++;
-            // (the low word is the vertex id, already in order: a stable sort by the high word suffices)
-            rs = radix_sort_u64(ctx, k1.as<uint64_t>(), ctx->vorder.as<int32_t>(), k2.as<uint64_t>(),
-                                v2.as<int32_t>(), n, 32, 32);
-        }
-        cudaStreamSynchronize(ctx->stream);
-        cudaFree(k1.p);
-        cudaFree(k2.p);
-        cudaFree(v2.p);
-        if (rs != PERCIS_OK) return rs;
-    }
+    PERCIS_TRY(ensure(ctx, ctx->vorder, sizeof(int32_t) * n, "vertex order"));
+    // the state sort's scratch, kept in the context (freeing scratch of its own
+    // synchronised the device on every new graph)
+    PERCIS_TRY(ensure(ctx, ctx->pc_tmp, (sizeof(uint64_t) * 2 + sizeof(int32_t)) * n + 64, "vertex order scratch"));
+    uint64_t *k1 = ctx->pc_tmp.as<uint64_t>(), *k2 = k1 + n;
+    k_hub_keys<<<grid_for(ctx, n * 8, 256), 256, 0, ctx->stream>>>(ctx->rp.as<int64_t>(), ctx->col.as<int32_t>(), n,
+                                                                 k1, ctx->vorder.as<int32_t>());
+    PERCIS_CHECK_LAUNCH(ctx, "hub keys");
+    // (the low word is the vertex id, already in order: a stable sort by the high word's
+    // used bits suffices)
+    int bits = 1;
+    while (bits < 32 && (1ll << bits) < n) ++bits;
+    PERCIS_TRY(radix_sort_u64(ctx, k1, ctx->vorder.as<int32_t>(), k2, reinterpret_cast<int32_t *>(k2 + n), n, 32, bits));
     ctx->vorder_ready = true;
     return PERCIS_OK;
 }
