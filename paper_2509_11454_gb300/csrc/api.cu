@@ -70,6 +70,16 @@ double events_elapsed_ms(percis_ctx *ctx) {
     return tot;
 }
 
+// Pinned host words (status at 0, phase statistics at 64, state preparation at 128): asynchronous copies
+// there complete with the stream, so one synchronisation reads them all.
+char *host_mirror(percis_ctx *ctx) {
+    if (!ctx->hmirror && cudaMallocHost(&ctx->hmirror, 256) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->hmirror = nullptr;
+    }
+    return static_cast<char *>(ctx->hmirror);
+}
+
 namespace {
 
 struct DeviceGuard {
@@ -92,8 +102,8 @@ struct alignas(16) PhaseStats {
     long long pad[3];
 };
 
-__global__ void k_phase_stats(int64_t count, const int32_t *kind, const int32_t *ilen, int64_t n, const double *lam,
-                              const unsigned long long *cnt, const double *acc, PhaseStats *out) {
+__global__ void k_phase_stats(int64_t count, const int32_t *kind, const int32_t *ilen, int64_t n, const double *Cv,
+                              const double *dscal, const unsigned long long *cnt, const double *acc, PhaseStats *out) {
     long long s1 = 0, s2 = 0, zw = 0, un = 0;
     double pm = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -105,10 +115,11 @@ __global__ void k_phase_stats(int64_t count, const int32_t *kind, const int32_t 
         un += kind[i] == 2;
     }
     // the largest lambda_v cnt_v (the division by l is monotone, so it is applied
-    // once to the maximum, on the host); zero counts skip the FP64 product
+    // once to the maximum, on the host); zero counts skip the FP64 work
+    const double C = n > 0 ? dscal[0] : 0.0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const double c = acc ? acc[v] : (double)cnt[v];
-        if (c != 0.0) pm = fmax(pm, __dmul_rn(lam[v], c));
+        if (c != 0.0) pm = fmax(pm, __dmul_rn(__ddiv_rn(C, Cv[v]), c));
     }
     for (int off = 16; off > 0; off >>= 1) {
         s1 += __shfl_xor_sync(0xffffffffu, s1, off);
@@ -127,12 +138,13 @@ __global__ void k_phase_stats(int64_t count, const int32_t *kind, const int32_t 
 }
 
 // p~(v) = lambda_v cnt_v / l  (all-paths: lambda_v acc_v / l)
-__global__ void k_finalize(const double *lam, const unsigned long long *cnt, const double *acc, int64_t n, double ell,
+__global__ void k_finalize(const double *Cv, const double *dscal, const unsigned long long *cnt, const double *acc, int64_t n, double ell,
                            double *pc) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const double C = dscal[0];
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const double c = acc ? acc[v] : (double)cnt[v];
-        pc[v] = c == 0.0 ? 0.0 : __ddiv_rn(__dmul_rn(lam[v], c), ell);  // (lambda is finite: 0 stays +0)
+        pc[v] = c == 0.0 ? 0.0 : __ddiv_rn(__dmul_rn(__ddiv_rn(C, Cv[v]), c), ell);  // (lambda is finite: 0 stays +0)
     }
 }
 
@@ -167,16 +179,6 @@ percis_status need_states(percis_ctx *ctx) {
     return PERCIS_OK;
 }
 
-// Pinned host words (status at 0, phase statistics at 64): asynchronous copies
-// there complete with the stream, so one synchronisation reads them all.
-char *host_mirror(percis_ctx *ctx) {
-    if (!ctx->hmirror && cudaMallocHost(&ctx->hmirror, 256) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->hmirror = nullptr;
-    }
-    return static_cast<char *>(ctx->hmirror);
-}
-
 uint32_t read_status(percis_ctx *ctx) {
     char *hm = host_mirror(ctx);
     uint32_t st = 0, st2 = 0;
@@ -198,7 +200,7 @@ percis_status issue_phase_stats(percis_ctx *ctx, int64_t count, bool want_pmax) 
     PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->red.p, 0, sizeof(PhaseStats), ctx->stream));
     const int64_t nv = want_pmax ? ctx->n : 0;
     k_phase_stats<<<grid_for(ctx, std::max<int64_t>(std::max<int64_t>(count, nv), 1), 256), 256, 0, ctx->stream>>>(
-        count, ctx->kind.as<int32_t>(), ctx->ilen.as<int32_t>(), nv, ctx->lam.as<double>(),
+        count, ctx->kind.as<int32_t>(), ctx->ilen.as<int32_t>(), nv, ctx->Cv.as<double>(), ctx->dscal.as<double>(),
         ctx->cnt.as<unsigned long long>(), ctx->opt.estimator == 1 ? ctx->acc_ap.as<double>() : nullptr,
         ctx->red.as<PhaseStats>());
     PERCIS_CHECK_LAUNCH(ctx, "phase stats");
@@ -397,7 +399,7 @@ void percis_destroy(percis_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->aux) cudaStreamSynchronize(ctx->aux);
     DevBuf *bufs[] = {&ctx->rp, &ctx->col, &ctx->irp, &ctx->icol, &ctx->x, &ctx->xs, &ctx->perm, &ctx->w, &ctx->ci,
-                      &ctx->r, &ctx->Cv, &ctx->lam, &ctx->grp_lo, &ctx->grp_hi, &ctx->dscal, &ctx->stamp, &ctx->plain_hub, &ctx->ms_big, &ctx->ms_walks,
+                      &ctx->r, &ctx->Cv, &ctx->grp_lo, &ctx->grp_hi, &ctx->dscal, &ctx->stamp, &ctx->plain_hub, &ctx->ms_big, &ctx->ms_walks,
                       &ctx->ms_need, &ctx->ms_list, &ctx->ms_levels,
                       &ctx->sigma1, &ctx->qa, &ctx->qb, &ctx->plain_ctl, &ctx->vis, &ctx->fhist, &ctx->sigmaW,
                       &ctx->ms_ctl, &ctx->remaining, &ctx->found, &ctx->pair_s, &ctx->pair_t, &ctx->kind,
@@ -560,7 +562,7 @@ percis_status percis_estimate(percis_ctx *ctx, double eps, double delta, uint64_
         dst = ctx->pc_tmp.as<double>();
     }
     k_finalize<<<grid_for(ctx, ctx->n, 256), 256, 0, ctx->stream>>>(
-        ctx->lam.as<double>(), ctx->cnt.as<unsigned long long>(),
+        ctx->Cv.as<double>(), ctx->dscal.as<double>(), ctx->cnt.as<unsigned long long>(),
         ctx->opt.estimator == 1 ? ctx->acc_ap.as<double>() : nullptr, ctx->n, (double)ell, dst);
     PERCIS_CHECK_LAUNCH(ctx, "finalize");
     if (info) PERCIS_TRY(issue_phase_stats(ctx, ell, false));  // read after the synchronisation below
@@ -649,7 +651,7 @@ percis_status percis_get_prep(percis_ctx *ctx, int32_t *perm, double *xs, double
     PERCIS_TRY(cp(ci, ctx->ci, sizeof(double) * (n + 2)));
     PERCIS_TRY(cp(r, ctx->r, sizeof(double) * (n + 2)));
     PERCIS_TRY(cp(Cv, ctx->Cv, sizeof(double) * n));
-    PERCIS_TRY(cp(lambda, ctx->lam, sizeof(double) * n));
+    if (lambda) PERCIS_TRY(ctx->multi ? multi_lambda(ctx, lambda) : prep_lambda(ctx, lambda));
     if (c) *c = ctx->c_host;
     if (dhat) *dhat = ctx->dhat_host;
     PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

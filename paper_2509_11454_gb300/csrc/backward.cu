@@ -37,13 +37,17 @@ __global__ void k_bw_samples(int64_t count, const int32_t *s, const int32_t *t, 
     }
 }
 
-__global__ void k_bw_gamma(int64_t n, const int32_t *perm, const double *g, const double *lam,
+__global__ void k_bw_gamma(int64_t n, const int32_t *perm, const double *g, const double *dscal,
                            const unsigned long long *cnt, const double *Cv, double ell, double *gs) {
+    const double C = dscal[0];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const int32_t v = perm[i];
-        const double F = lam[v] * (double)cnt[v] / ell;
-        gs[i] = g[v] * F / Cv[v];
+        const unsigned long long k = cnt[v];
+        // (no path through v: F_v = 0, and its divisions are left out)
+        const double F = k ? C / Cv[v] * (double)k / ell : 0.0;
+        const double p = g[v] * F;
+        gs[i] = p == 0.0 ? p : p / Cv[v];
     }
 }
 
@@ -77,7 +81,7 @@ percis_status backward_fixed(percis_ctx *ctx, const double *g, double *grad) {
     double *gs = ctx->grad_tmp.as<double>();
     double *G = gs + n;
     k_bw_gamma<<<grid_for(ctx, n, block), block, 0, ctx->stream>>>(n, ctx->perm.as<int32_t>(), g,
-                                                                  ctx->lam.as<double>(),
+                                                                  ctx->dscal.as<double>(),
                                                                   ctx->cnt.as<unsigned long long>(),
                                                                   ctx->Cv.as<double>(), (double)ctx->last_ell, gs);
     PERCIS_CHECK_LAUNCH(ctx, "backward gamma");

@@ -78,7 +78,7 @@ struct percis_ctx {
 
     // states and preprocessing
     bool have_states = false;
-    percis::DevBuf x, xs, perm, w, ci, r, Cv, lam, grp_lo, grp_hi;
+    percis::DevBuf x, xs, perm, w, ci, r, Cv, grp_lo, grp_hi;
     double c_host = 0.0, dhat_host = 0.0;
     percis::DevBuf dscal;  // device scalars: [0] = c, [1] = dhat
 
@@ -192,6 +192,8 @@ percis_status ensure(percis_ctx *ctx, DevBuf &b, size_t bytes, const char *what)
         if (s__ != PERCIS_OK) return s__;      \
     } while (0)
 
+char *host_mirror(percis_ctx *ctx);  // pinned host words (nullptr if they cannot be had)
+
 // Next event of the context's pool (created on demand; nullptr if creation fails).
 cudaEvent_t next_event(percis_ctx *ctx);
 // Summed elapsed time of the event pairs recorded since ev_next was reset (stream synchronised).
@@ -213,6 +215,7 @@ percis_status transpose_finish(percis_ctx *ctx);  // in-adjacency: offsets (vali
 // prep.cu
 percis_status prep_graph(percis_ctx *ctx);  // transpose (directed), validation, VertexDiamUB
 percis_status prep_states(percis_ctx *ctx);  // sort, tables, C_v, lambda, d^
+percis_status prep_lambda(percis_ctx *ctx, double *lam);  // lambda_v of every vertex (device)
 percis_status prep_groups(percis_ctx *ctx);
 percis_status wait_graph(percis_ctx *ctx);  // the context stream waits for the in-adjacency  // tie groups of the sorted states (backward, on first use)
 percis_status prep_vorder(percis_ctx *ctx);  // lane order of the batched form (on first use)
@@ -276,6 +279,7 @@ struct LaneBatch {
     int64_t nr;
 };
 percis_status multi_plan_batches(percis_ctx *ctx, int64_t n_sources, int W, std::vector<LaneBatch> *out);
+percis_status multi_lambda(percis_ctx *ctx, double *lam);  // lambda_v of every graph's vertices
 int64_t multi_range(percis_ctx *ctx);  // vertex range of the batch buffers
 // for the bidirectional form: graph of every vertex, first id of every graph, largest graph
 void multi_graph_view(percis_ctx *ctx, const int32_t **gid, const int64_t **vbase, int64_t *largest);

@@ -33,7 +33,7 @@ struct MultiGraph {
     DevBuf gid;                         // graph of every vertex
     DevBuf vptr_dev;                    // first vertex id of every graph (device)
     int64_t largest = 0;
-    DevBuf soff_dev, ell_dev, stats, pmax;
+    DevBuf soff_dev, ell_dev, c_dev, stats, pmax;  // c_dev: C of every graph
     bool paths_scattered = false;
     // recorded per-graph sampling launches of each phase (pair tag 0 / 1), the
     // counts they were recorded for, and the device word they read the seed from
@@ -91,21 +91,26 @@ __global__ void k_stats_multi(int64_t count, const long long *soff, int32_t G, c
 }
 
 // per graph: max_v lambda_v cnt_v / l_g (non-negative, so the bit patterns order like the values)
-__global__ void k_pmax_multi(const double *lam, const unsigned long long *cnt, const double *acc, const int32_t *gid,
+__global__ void k_pmax_multi(const double *Cv, const double *C, const unsigned long long *cnt, const double *acc, const int32_t *gid,
                              const double *ell, int64_t n, unsigned long long *pmax) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int32_t g = gid[v];
-        const double p = lam[v] * (acc ? acc[v] : (double)cnt[v]) / ell[g];
+        const double k = acc ? acc[v] : (double)cnt[v];
+        if (k == 0.0) continue;
+        const double p = C[g] / Cv[v] * k / ell[g];
         if (p > 0.0) atomicMax(&pmax[g], (unsigned long long)__double_as_longlong(p));
     }
 }
 
-__global__ void k_finalize_multi(const double *lam, const unsigned long long *cnt, const double *acc,
+__global__ void k_finalize_multi(const double *Cv, const double *C, const unsigned long long *cnt, const double *acc,
                                  const int32_t *gid, const double *ell, int64_t n, double *pc) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-        pc[v] = lam[v] * (acc ? acc[v] : (double)cnt[v]) / ell[gid[v]];
+{
+        const double k = acc ? acc[v] : (double)cnt[v];
+        pc[v] = k == 0.0 ? 0.0 : C[gid[v]] / Cv[v] * k / ell[gid[v]];
+    }
 }
 
 // a graph's samples of the last phase in its own context: local ids, paths
@@ -133,11 +138,20 @@ void multi_free(percis_ctx *ctx) {
     drop_graph(m, 0);
     drop_graph(m, 1);
     for (percis_ctx *sub : m->subs) percis_destroy(sub);
-    DevBuf *bufs[] = {&m->gid, &m->soff_dev, &m->ell_dev, &m->stats, &m->pmax, &m->seed_dev, &m->vptr_dev};
+    DevBuf *bufs[] = {&m->gid, &m->soff_dev, &m->ell_dev, &m->c_dev, &m->stats, &m->pmax, &m->seed_dev, &m->vptr_dev};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     delete m;
     ctx->multi = nullptr;
+}
+
+percis_status multi_lambda(percis_ctx *ctx, double *lam) {
+    MultiGraph *m = ctx->multi;
+    for (int32_t g = 0; g < m->G; ++g) {
+        const percis_status st = prep_lambda(m->subs[g], lam + m->vptr[g]);
+        if (st != PERCIS_OK) return set_err(ctx, st, m->subs[g]->err);
+    }
+    return PERCIS_OK;
 }
 
 int64_t multi_range(percis_ctx *ctx) { return ctx->multi ? ctx->multi->range : ctx->n; }
@@ -281,7 +295,7 @@ percis_status multi_stats(percis_ctx *ctx, const std::vector<double> &ell, std::
         PERCIS_CHECK_LAUNCH(ctx, "graph stats");
     }
     k_pmax_multi<<<grid_for(ctx, ctx->n, 256), 256, 0, ctx->stream>>>(
-        ctx->lam.as<double>(), ctx->cnt.as<unsigned long long>(),
+        ctx->Cv.as<double>(), m->c_dev.as<double>(), ctx->cnt.as<unsigned long long>(),
         ctx->opt.estimator == 1 ? ctx->acc_ap.as<double>() : nullptr, m->gid.as<int32_t>(), m->ell_dev.as<double>(),
         ctx->n, m->pmax.as<unsigned long long>());
     PERCIS_CHECK_LAUNCH(ctx, "graph pmax");
@@ -395,7 +409,8 @@ percis_status percis::percis_multi_set_states(percis_ctx *ctx, const double *x, 
     ctx->have_paths = false;
     const int64_t n = ctx->n;
     PERCIS_TRY(ensure(ctx, ctx->x, sizeof(double) * n, "x"));
-    PERCIS_TRY(ensure(ctx, ctx->lam, sizeof(double) * n, "lambda"));
+    PERCIS_TRY(ensure(ctx, ctx->Cv, sizeof(double) * n, "Cv"));
+    PERCIS_TRY(ensure(ctx, m->c_dev, sizeof(double) * m->G, "graph C"));
     PERCIS_CUDA(ctx, cudaMemcpyAsync(ctx->x.p, x, sizeof(double) * n,
                                      on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->stream));
     for (int32_t g = 0; g < m->G; ++g) {
@@ -403,7 +418,9 @@ percis_status percis::percis_multi_set_states(percis_ctx *ctx, const double *x, 
         const int64_t lo = m->vptr[g], ng = m->vptr[g + 1] - lo;
         const percis_status st = percis_set_states(sub, ctx->x.as<double>() + lo, 1);
         if (st != PERCIS_OK) return set_err(ctx, st, "graph " + std::to_string(g) + ": " + sub->err);
-        PERCIS_CUDA(ctx, cudaMemcpyAsync(ctx->lam.as<double>() + lo, sub->lam.p, sizeof(double) * ng,
+        PERCIS_CUDA(ctx, cudaMemcpyAsync(ctx->Cv.as<double>() + lo, sub->Cv.p, sizeof(double) * ng,
+                                         cudaMemcpyDeviceToDevice, ctx->stream));
+        PERCIS_CUDA(ctx, cudaMemcpyAsync(m->c_dev.as<double>() + g, sub->dscal.p, sizeof(double),
                                          cudaMemcpyDeviceToDevice, ctx->stream));
     }
     PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -470,7 +487,7 @@ extern "C" percis_status percis_estimate_graphs(percis_ctx *ctx, double eps, dou
         dst = ctx->pc_tmp.as<double>();
     }
     k_finalize_multi<<<grid_for(ctx, ctx->n, 256), 256, 0, ctx->stream>>>(
-        ctx->lam.as<double>(), ctx->cnt.as<unsigned long long>(),
+        ctx->Cv.as<double>(), m->c_dev.as<double>(), ctx->cnt.as<unsigned long long>(),
         ctx->opt.estimator == 1 ? ctx->acc_ap.as<double>() : nullptr, m->gid.as<int32_t>(), m->ell_dev.as<double>(),
         ctx->n, dst);
     PERCIS_CHECK_LAUNCH(ctx, "finalize graphs");

@@ -70,29 +70,36 @@ __global__ void k_max_degree(const int64_t *rp, int64_t n, unsigned long long *o
     if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
 }
 
-__global__ void k_check_states(const double *x, int64_t n, uint32_t *status) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const double a = x[v];
-        if (!(a >= 0.0 && a <= 1.0)) atomicOr(status, DEV_BAD_STATE);
-    }
-}
-
 // ---------------------------------------------------------- state keys
 
-__global__ void k_state_keys(const double *x, int64_t n, uint64_t *keys, int32_t *vals) {
+// Checks the states, writes their sort keys, and counts the non-zero ones (the
+// zeros form the sorted suffix) into the int64 word at dscal + 2.
+__global__ void k_state_keys(const double *x, int64_t n, uint64_t *keys, int32_t *vals, uint32_t *status,
+                             double *dscal) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int nz = 0;
+    bool bad = false;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const double a = x[v] + 0.0;  // -0.0 -> +0.0
-        // x >= 0: larger value <-> larger bit pattern; complement sorts descending
-        keys[v] = ~(uint64_t)__double_as_longlong(a);
+        const double a = x[v];
+        // in [0, 1] by its bits (-0.0 counts as +0.0): non-negative doubles order like
+        // their bit patterns, and an FP64 comparison holds that pipe for ~64 cycles
+        const uint64_t b = (uint64_t)__double_as_longlong(a) == 0x8000000000000000ull
+                               ? 0ull : (uint64_t)__double_as_longlong(a);
+        bad |= b > 0x3ff0000000000000ull;
+        nz += b != 0ull;
+        keys[v] = ~b;  // larger value <-> larger bit pattern; the complement sorts descending
         vals[v] = (int32_t)v;
     }
+    if (bad) atomicOr(status, DEV_BAD_STATE);
+    nz = __reduce_add_sync(0xffffffffu, nz);
+    if ((threadIdx.x & 31) == 0 && nz)
+        atomicAdd(reinterpret_cast<unsigned long long *>(dscal + 2), (unsigned long long)nz);
 }
 
-__global__ void k_gather_sorted(const double *x, const int32_t *perm, int64_t n, double *xs) {
+__global__ void k_sorted_states(const uint64_t *keys, int64_t n, double *xs) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) xs[i] = x[perm[i]] + 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+        xs[i] = __longlong_as_double((long long)~keys[i]);
 }
 
 // ------------------------------------------------------- Algorithm 2 scan
@@ -211,6 +218,15 @@ struct SegSlot {
     double scross;            // resolved: sum after term b
 };
 
+// What the walk over the binades reads and leaves of a slot.
+struct SegWalk {
+    long long b;
+    double a;                 // value of the first term, then the sum after it
+    unsigned long long d[2];  // integer added by the binade's other terms, by parity
+    unsigned long long s0;
+    int prev;
+};
+
 // Control block of the cooperative table launch.
 struct TableCtl {
     GridBarrier bar;
@@ -305,6 +321,9 @@ __device__ bool running_sum_predicted(const double *src, int64_t soff, double *d
     __shared__ double s_bc;
     __shared__ SegRun s_bsr;
     __shared__ int s_key[kMaxSegs];
+    __shared__ SegWalk s_walk[kMaxSegs];
+    __shared__ int s_done;
+    __shared__ long long s_fail;
     __shared__ int s_pc[nw];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long nth = (long long)gridDim.x * kScanThreads;
@@ -312,7 +331,9 @@ __device__ bool running_sum_predicted(const double *src, int64_t soff, double *d
     const long long g = (long long)blockIdx.x * kScanThreads + tid;
     const long long k0 = min((long long)m, g * T), k1 = min((long long)m, k0 + T);
     // term k of the scan (k = 0 is position m)
-    auto term = [&](long long k) { return __ldcg(&src[m - k + soff]); };
+    // (a plain load: a thread's terms are consecutive, so each sector serves four of
+    // them from L1; the sector is first read after the barrier that follows its writes)
+    auto term = [&](long long k) { return src[m - k + soff]; };
 
     // 1. the prediction: exclusive FP64 prefix of the threads' sums
     if (blockIdx.x == 0 && tid == 0) ctl->conflict = 0u;  // (set only after the barrier below)
@@ -465,20 +486,35 @@ __device__ bool running_sum_predicted(const double *src, int64_t soff, double *d
             if (p1) s_key[at + p0] = E1;
         }
         __syncthreads();
+        // the binades' records side by side in shared memory: the walk is one thread's
+        // chain, and a record read from device memory at each step took ~1.5 us of it
+        // (n = 1000: 90 us for the launch, 54 us with it and the cached loads; 4.2M states:
+        // 393 us, 249 us)
+        if (tid < total && total <= kMaxSegs) {
+            const SegSlot *sg = &ctl->seg[s_key[tid]];
+            const RunMap *mr = tid + 1 < total ? &ctl->seg[s_key[tid + 1]].mprev : &ctl->mlast;
+            s_walk[tid].b = __ldcg(&sg->b);
+            s_walk[tid].prev = __ldcg(&sg->prev);
+            s_walk[tid].a = __ldcg(&sg->a);
+            s_walk[tid].d[0] = __ldcg(&mr->d0);
+            s_walk[tid].d[1] = __ldcg(&mr->d1);
+        }
+        __syncthreads();
         if (tid == 0) {
             long long fail = m;
+            int done = 0;
             double S = 0.0;
             if (__ldcg(&ctl->conflict) || total > kMaxSegs || total < 1 || __ldcg(&ctl->klast) != s_key[total - 1])
                 fail = 0;
             for (int i = 0; fail == m && i < total; ++i) {
                 const int E = s_key[i];
-                SegSlot *sg = &ctl->seg[E];
-                const long long b = __ldcg(&sg->b);
-                if ((i == 0) != (b == 0) || __ldcg(&sg->prev) != (i == 0 ? -1 : s_key[i - 1])) {
+                SegWalk &sg = s_walk[i];
+                const long long b = sg.b;
+                if ((i == 0) != (b == 0) || sg.prev != (i == 0 ? -1 : s_key[i - 1])) {
                     fail = i == 0 ? 0 : b;
                     break;
                 }
-                const double sc = __dadd_rn(S, __ldcg(&sg->a));
+                const double sc = __dadd_rn(S, sg.a);
                 if (sum_key(sc) != E) {  // the first term did not land in the predicted binade
                     fail = b;
                     break;
@@ -486,26 +522,35 @@ __device__ bool running_sum_predicted(const double *src, int64_t soff, double *d
                 const unsigned long long sb = (unsigned long long)__double_as_longlong(sc);
                 const int es = (int)((sb >> 52) & 0x7ff);
                 const unsigned long long S0 = (sb & ((1ull << 52) - 1)) | (es ? (1ull << 52) : 0ull);
-                const RunMap *mr = i + 1 < total ? &ctl->seg[s_key[i + 1]].mprev : &ctl->mlast;
-                const unsigned long long d = (S0 & 1ull) ? __ldcg(&mr->d1) : __ldcg(&mr->d0);
+                const unsigned long long d = sg.d[S0 & 1ull];
                 if (S0 + d >= kTwo53u) {  // the run leaves the binade before the next predicted start
                     fail = b;
                     break;
                 }
-                sg->s0 = S0;
-                sg->scross = sc;
+                sg.s0 = S0;
+                sg.a = sc;
+                ++done;
                 S = __longlong_as_double((long long)(((unsigned long long)(E - 1) << 52) + S0 + d));
             }
+            s_done = done;
             ctl->fail_b = fail;
             ctl->pos = m - fail;
             ctl->s = S;  // the sum before term `fail` (every binade before it resolved)
+        }
+        __syncthreads();
+        if (tid < s_done) {
+            SegSlot *sg = &ctl->seg[s_key[tid]];
+            sg->s0 = s_walk[tid].s0;
+            sg->scross = s_walk[tid].a;
         }
     }
     if (!grid_sync(&ctl->bar, &ctl->status, budget_ns)) return false;
 
     // 4. every term before the first failure: its binade's sum after the first
     // term plus the integer its run added, under that sum's parity
-    const long long fail = __ldcg(&ctl->fail_b);
+    if (tid == 0) s_fail = __ldcg(&ctl->fail_b);
+    __syncthreads();
+    const long long fail = s_fail;
     if (k0 < fail) {
         const long long kend = min(k1, fail);
         int cur = key_in;
@@ -683,19 +728,6 @@ __device__ bool grid_running_sum(const double *src, int64_t soff, double *dst, i
     return true;
 }
 
-// Number of non-zero sorted states (xs is non-increasing and >= 0, so the
-// zeros form a suffix), by bisection, into the int64 word at dscal + 2.
-__global__ void k_nonzero_prefix(const double *xs, int64_t n, double *dscal) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int64_t lo = 0, hi = n;  // first zero in [lo, hi]
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (xs[mid] == 0.0) hi = mid;
-        else lo = mid + 1;
-    }
-    *reinterpret_cast<long long *>(dscal + 2) = (long long)lo;
-}
-
 // Cooperative launch of G blocks (all co-resident): w, then c_i, then r.
 __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64_t n, double *w, double *ci,
                                                          double *r, double *dscal, TableCtl *ctl,
@@ -721,12 +753,17 @@ __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64
 }
 
 // C_v = c - A_v with A_i = (w_1 - w_i) - (i-1) x_i + (n-i) x_i - w_{i+1} for
-// sorted position i (the closed form of sum_u |x_i - x_u|), lambda = c / C_v.
-__global__ void k_cv_lambda(const double *xs, const int32_t *perm, const double *w, const double *dscal, int64_t n,
-                            double *Cv, double *lam, uint32_t *status) {
+// sorted position i (the closed form of sum_u |x_i - x_u|), and the bits of the
+// smallest into dscal[1].  lambda_v = c / C_v is formed where it is used (the vertices
+// a phase counted): a division for every vertex was most of this kernel's FP64 work,
+// and max_v lambda_v = c / min_v C_v (the rounded division is monotone).
+__global__ void k_cv(const double *xs, const int32_t *perm, const double *w, double *dscal, int64_t n, double *Cv,
+                     uint32_t *status) {
     const double c = dscal[0];
     const double w1 = w[1];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    unsigned long long m = ~0ull;
+    bool bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x + 1; i <= n; i += stride) {
         const double xi = xs[i - 1];
         double a = __dsub_rn(w1, w[i]);
@@ -734,28 +771,22 @@ __global__ void k_cv_lambda(const double *xs, const int32_t *perm, const double 
         a = __dadd_rn(a, __dmul_rn((double)(n - i), xi));
         a = __dsub_rn(a, w[i + 1]);
         const double cv = __dsub_rn(c, a);
-        const int32_t v = perm[i - 1];
-        Cv[v] = cv;
-        if (cv > 0.0) {
-            lam[v] = __ddiv_rn(c, cv);
-        } else {
-            lam[v] = __longlong_as_double(0x7ff0000000000000LL);
-            atomicOr(status, DEV_DEGENERATE);
-        }
+        Cv[perm[i - 1]] = cv;
+        // positive doubles order like their bit patterns; not positive: +0, the sign bit, NaN
+        const unsigned long long b = (unsigned long long)__double_as_longlong(cv);
+        if (b - 1ull < 0x7ff0000000000000ull) m = min(m, b);
+        else bad = true;
     }
+    if (bad) atomicOr(status, DEV_DEGENERATE);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0 && m != ~0ull) atomicMin(reinterpret_cast<unsigned long long *>(&dscal[1]), m);
 }
 
-__device__ __forceinline__ void atomic_max_pos_double(double *addr, double v) {
-    // non-negative doubles order like their bit patterns
-    atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
-}
-
-__global__ void k_max_lambda(const double *lam, int64_t n, double *dscal) {
-    double m = 0.0;
+__global__ void k_lambda(const double *Cv, const double *dscal, int64_t n, double *lam) {
+    const double c = dscal[0];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) m = fmax(m, lam[v]);
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) atomic_max_pos_double(&dscal[1], m);
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) lam[v] = __ddiv_rn(c, Cv[v]);
 }
 
 // Tie groups of the sorted states: positions [lo, hi] (1-based) with equal x.
@@ -929,78 +960,75 @@ percis_status prep_states(percis_ctx *ctx) {
     const int64_t n = ctx->n;
     uint32_t *st = ctx->status.as<uint32_t>();
     PERCIS_CUDA(ctx, cudaMemsetAsync(st, 0, 64, ctx->stream));
-    k_check_states<<<grid_for(ctx, n, 256), 256, 0, ctx->stream>>>(ctx->x.as<double>(), n, st);
-    PERCIS_CHECK_LAUNCH(ctx, "check states");
-
     PERCIS_TRY(ensure(ctx, ctx->xs, sizeof(double) * n, "xs"));
     PERCIS_TRY(ensure(ctx, ctx->perm, sizeof(int32_t) * n, "perm"));
     PERCIS_TRY(ensure(ctx, ctx->w, sizeof(double) * (n + 2), "w"));
     PERCIS_TRY(ensure(ctx, ctx->ci, sizeof(double) * (n + 2), "ci"));
     PERCIS_TRY(ensure(ctx, ctx->r, sizeof(double) * (n + 2), "r"));
     PERCIS_TRY(ensure(ctx, ctx->Cv, sizeof(double) * n, "Cv"));
-    PERCIS_TRY(ensure(ctx, ctx->lam, sizeof(double) * n, "lambda"));
     PERCIS_TRY(ensure(ctx, ctx->dscal, 64, "scalars"));
-    // sort scratch: keys, keys2, vals2 (reuse the sigma buffer space if large)
+    // sort scratch: keys, keys2, vals2
     PERCIS_TRY(ensure(ctx, ctx->pc_tmp, (sizeof(uint64_t) * 2 + sizeof(int32_t)) * n + 64, "sort scratch"));
+    char *hm = host_mirror(ctx);
+    if (!hm) return set_err(ctx, PERCIS_E_OOM, "pinned host words");
     uint64_t *k1 = ctx->pc_tmp.as<uint64_t>();
     uint64_t *k2 = k1 + n;
     int32_t *v2 = (int32_t *)(k2 + n);
     int32_t *perm = ctx->perm.as<int32_t>();
+    double *dscal = ctx->dscal.as<double>();  // c, smallest C_v, number of non-zero states
     const int g = grid_for(ctx, n, 256);
-    k_state_keys<<<g, 256, 0, ctx->stream>>>(ctx->x.as<double>(), n, k1, perm);
+    PERCIS_CUDA(ctx, cudaMemsetAsync(dscal, 0, 64, ctx->stream));
+    PERCIS_CUDA(ctx, cudaMemsetAsync(dscal + 1, 0x7f, sizeof(double), ctx->stream));  // 1.4e306, above every C_v
+    k_state_keys<<<g, 256, 0, ctx->stream>>>(ctx->x.as<double>(), n, k1, perm, st, dscal);
     PERCIS_CHECK_LAUNCH(ctx, "state keys");
     PERCIS_TRY(radix_sort_u64(ctx, k1, perm, k2, v2, n, 0, 64));
-    k_gather_sorted<<<g, 256, 0, ctx->stream>>>(ctx->x.as<double>(), perm, n, ctx->xs.as<double>());
-    PERCIS_CHECK_LAUNCH(ctx, "gather sorted");
-    k_nonzero_prefix<<<1, 32, 0, ctx->stream>>>(ctx->xs.as<double>(), n, ctx->dscal.as<double>());
-    PERCIS_CHECK_LAUNCH(ctx, "non-zero states");
-    {
-        // as many co-resident blocks as the non-zero states fill (read back: the launch
-        // size is set on the host)
-        long long nz = 0;
-        PERCIS_CUDA(ctx, cudaMemcpyAsync(&nz, ctx->dscal.as<double>() + 2, sizeof(nz), cudaMemcpyDeviceToHost,
-                                         ctx->stream));
-        PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        if (ctx->table_grid == 0) {
-            int per_sm = 0;
-            PERCIS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tables, kScanThreads, 0));
-            ctx->table_grid = std::min(kMaxTableBlocks, std::max(1, per_sm) * ctx->num_sms);
-        }
-        const int G = (int)std::max<long long>(1, std::min<long long>(ctx->table_grid, (nz + kScanChunk - 1) / kScanChunk));
-        PERCIS_TRY(ensure(ctx, ctx->table_ctl, sizeof(TableCtl), "table control"));
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->table_ctl.p, 0, sizeof(TableCtl), ctx->stream));
-        const double *xs = ctx->xs.as<double>();
-        double *w = ctx->w.as<double>(), *ci = ctx->ci.as<double>(), *r = ctx->r.as<double>();
-        double *dscal = ctx->dscal.as<double>();
-        TableCtl *tctl = ctx->table_ctl.as<TableCtl>();
-        uint64_t budget = (uint64_t)(ctx->opt.timeout_s * 1e9);
-        int64_t nn = n;
-        void *args[] = {&xs, &nn, &w, &ci, &r, &dscal, &tctl, &budget};
-        PERCIS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_tables, dim3(G), dim3(kScanThreads), args, 0,
-                                                     ctx->stream));
-        ctx->launches++;
-        uint32_t tst = 0;
-        PERCIS_CUDA(ctx, cudaMemcpyAsync(&tst, &tctl->status, 4, cudaMemcpyDeviceToHost, ctx->stream));
-        PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        if (tst & DEV_TIMEOUT) return set_err(ctx, PERCIS_E_TIMEOUT, "table scan wait exceeded its budget");
+    k_sorted_states<<<g, 256, 0, ctx->stream>>>(k1, n, ctx->xs.as<double>());
+    PERCIS_CHECK_LAUNCH(ctx, "sorted states");
+    // as many co-resident blocks as n terms fill (the kernel reads the number of
+    // non-zero ones: no host round trip)
+    if (ctx->table_grid == 0) {
+        int per_sm = 0;
+        PERCIS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tables, kScanThreads, 0));
+        ctx->table_grid = std::min(kMaxTableBlocks, std::max(1, per_sm) * ctx->num_sms);
     }
-    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->dscal.as<double>() + 1, 0, sizeof(double), ctx->stream));
-    k_cv_lambda<<<g, 256, 0, ctx->stream>>>(ctx->xs.as<double>(), perm, ctx->w.as<double>(), ctx->dscal.as<double>(),
-                                            n, ctx->Cv.as<double>(), ctx->lam.as<double>(), st);
-    PERCIS_CHECK_LAUNCH(ctx, "cv lambda");
-    k_max_lambda<<<g, 256, 0, ctx->stream>>>(ctx->lam.as<double>(), n, ctx->dscal.as<double>());
-    PERCIS_CHECK_LAUNCH(ctx, "max lambda");
+    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(ctx->table_grid, (n + kScanChunk - 1) / kScanChunk));
+    PERCIS_TRY(ensure(ctx, ctx->table_ctl, sizeof(TableCtl), "table control"));
+    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->table_ctl.p, 0, sizeof(TableCtl), ctx->stream));
+    const double *xs = ctx->xs.as<double>();
+    double *w = ctx->w.as<double>(), *ci = ctx->ci.as<double>(), *r = ctx->r.as<double>();
+    TableCtl *tctl = ctx->table_ctl.as<TableCtl>();
+    uint64_t budget = (uint64_t)(ctx->opt.timeout_s * 1e9);
+    int64_t nn = n;
+    void *args[] = {&xs, &nn, &w, &ci, &r, &dscal, &tctl, &budget};
+    PERCIS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_tables, dim3(G), dim3(kScanThreads), args, 0,
+                                                 ctx->stream));
+    ctx->launches++;
+    k_cv<<<g, 256, 0, ctx->stream>>>(xs, perm, w, dscal, n, ctx->Cv.as<double>(), st);
+    PERCIS_CHECK_LAUNCH(ctx, "C_v");
     ctx->groups_ready = false;  // built by the first backward pass that needs them
-    double sc[2];
-    uint32_t hst = 0;
-    PERCIS_CUDA(ctx, cudaMemcpyAsync(sc, ctx->dscal.p, sizeof(sc), cudaMemcpyDeviceToHost, ctx->stream));
-    PERCIS_CUDA(ctx, cudaMemcpyAsync(&hst, st, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    struct Back {
+        double c, cv_min;
+        uint32_t status, tables;
+    };
+    Back *b = reinterpret_cast<Back *>(hm + 128);
+    PERCIS_CUDA(ctx, cudaMemcpyAsync(&b->c, dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    PERCIS_CUDA(ctx, cudaMemcpyAsync(&b->status, st, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    PERCIS_CUDA(ctx, cudaMemcpyAsync(&b->tables, &tctl->status, 4, cudaMemcpyDeviceToHost, ctx->stream));
     PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (hst & DEV_BAD_STATE) return set_err(ctx, PERCIS_E_INVALID, "states must lie in [0,1] (no NaN)");
-    ctx->c_host = sc[0];
-    ctx->dhat_host = sc[1];
-    if (hst & DEV_DEGENERATE)
+    if (b->tables & DEV_TIMEOUT) return set_err(ctx, PERCIS_E_TIMEOUT, "table scan wait exceeded its budget");
+    if (b->status & DEV_BAD_STATE) return set_err(ctx, PERCIS_E_INVALID, "states must lie in [0,1] (no NaN)");
+    ctx->c_host = b->c;
+    ctx->dhat_host = b->c / b->cv_min;
+    if (b->status & DEV_DEGENERATE)
         return set_err(ctx, PERCIS_E_DEGENERATE, "some C_v <= 0: percolation centrality undefined (all other states equal)");
+    return PERCIS_OK;
+}
+
+// lambda_v = c / C_v for every vertex
+percis_status prep_lambda(percis_ctx *ctx, double *lam) {
+    k_lambda<<<grid_for(ctx, ctx->n, 256), 256, 0, ctx->stream>>>(ctx->Cv.as<double>(), ctx->dscal.as<double>(), ctx->n,
+                                                                lam);
+    PERCIS_CHECK_LAUNCH(ctx, "lambda");
     return PERCIS_OK;
 }
 
