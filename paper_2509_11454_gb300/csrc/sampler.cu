@@ -7,6 +7,34 @@ namespace percis {
 
 namespace {
 
+// The searches' test u <= fl(num / c), u in (0, 1], without the division wherever the
+// two sides differ by more than rounding: num against u c (1 -+ 2^-50).  Above the upper
+// bound num / c > u, so its rounding is >= u; below the lower one num / c < u (1 - 2^-51),
+// under the double before u.  In between, and where u c is not well inside the
+// normal range, the division decides.  A dependent FP64 division took most of a
+// search step (~25 operations of ~64 cycles): 200k states, both phases (1,000 and 29,270
+// samples) 71 us, 48 us; 1,000 states 42 us, 26 us.
+struct QuotientTest {
+    double u, c;
+    long long lo, hi;  // bits of the bounds (non-negative doubles order like their bits; a negative num is below)
+    __device__ __forceinline__ QuotientTest(double u_, double c_) : u(u_), c(c_) {
+        const double p = __dmul_rn(u, c);
+        if (p >= 0x1p-900 && p <= 0x1p900) {
+            lo = __double_as_longlong(__dmul_rn(p, 1.0 - 0x1p-50));
+            hi = __double_as_longlong(__dmul_rn(p, 1.0 + 0x1p-50));
+        } else {
+            lo = (long long)0x8000000000000000ll;
+            hi = 0x7fffffffffffffffll;
+        }
+    }
+    __device__ __forceinline__ bool operator()(double num) const {
+        const long long b = __double_as_longlong(num);
+        if (b >= hi) return true;
+        if (b <= lo) return false;
+        return u <= __ddiv_rn(num, c);
+    }
+};
+
 // One thread per sample: Philox4x32-10 gives (u_s, u_t); two binary searches
 // exactly as Algorithm 2 (appendix) over the 1-based tables, evaluated with
 // explicit round-to-nearest operations so no multiply-add is fused.
@@ -22,9 +50,9 @@ __global__ void k_sample_pairs(int64_t n, const double *__restrict__ xs, const i
         double us, ut;
         uniforms2(seed, (uint64_t)(i0 + k), tag, 0u, us, ut);
         int64_t a = 1, b = n, d = (a + b) >> 1;
+        const QuotientTest first(us, c);
         while (a <= b) {
-            const double kk = __ddiv_rn(__dsub_rn(c, r[d + 1]), c);
-            if (us <= kk) b = d - 1;
+            if (first(__dsub_rn(c, r[d + 1]))) b = d - 1;
             else a = d + 1;
             d = (a + b) >> 1;
         }
@@ -33,10 +61,10 @@ __global__ void k_sample_pairs(int64_t n, const double *__restrict__ xs, const i
         a = s;
         b = n;
         d = (a + b) >> 1;
+        const QuotientTest second(ut, css);
         while (a <= b) {
             const double num = __dadd_rn(__dsub_rn(__dmul_rn((double)(d - s + 1), xss), wss), w[d + 1]);
-            const double kk = __ddiv_rn(num, css);
-            if (ut <= kk) b = d - 1;
+            if (second(num)) b = d - 1;
             else a = d + 1;
             d = (a + b) >> 1;
         }

@@ -142,3 +142,27 @@ def test_batched_rows_and_needed_counts(binding, lanes, direction, directed):
     for k in ("s", "t", "kind", "ilen", "cnt"):
         assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
     eng.close()
+
+
+@pytest.mark.parametrize("n,scale", [(2, 1.0), (3, 1.0), (1000, 1.0), (4097, 1e-6), (1000, 1e-300), (500, 1e-318)])
+@pytest.mark.parametrize("kind", ["uniform", "ties", "seeds"])
+def test_pairs_without_divisions(binding, n, scale, kind):
+    """Algorithm 2's searches, whose comparisons divide only next to equality (and always
+    where the products leave the normal range): the oracle's pairs."""
+    rng = np.random.default_rng(n)
+    x = rng.random(n)
+    if kind == "ties":
+        x = np.round(x * 4) / 4
+    elif kind == "seeds":
+        x = np.where(x > 0.7, 1.0, 0.0)
+    x[: min(n, 3)] = (1.0, 0.5, 0.0)[: min(n, 3)]
+    x = x * scale
+    g = synth.csr_from_edges(n, np.arange(n), (np.arange(n) + 1) % n, directed=True)
+    prep = oracle.prepare(x)
+    if not np.all(prep.Cv > 0):
+        pytest.skip("undefined states")
+    eng = _engine(binding, g, x)
+    s, t = eng.sample_pairs(5, 1, 0, 4000)
+    rs, rt, _, _ = oracle.sample_pairs(prep, 5, 1, 0, 4000)
+    assert np.array_equal(_np(s), rs) and np.array_equal(_np(t), rt)
+    eng.close()
