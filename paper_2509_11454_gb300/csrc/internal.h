@@ -209,6 +209,11 @@ int grid_for(percis_ctx *ctx, int64_t work, int block);
 // (irp, icol) of the loaded directed CSR, every in-list ordered by source
 percis_status radix_sort_u64(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uint64_t *tk, int32_t *tv, int64_t n,
                              int lo_bit, int bits);
+// the states' sort (see radix.cu): it changes buffers state_sort_swaps times (an odd number
+// leaves the result in tk / tv); *status and *nheads are zeroed device words
+int state_sort_swaps(int64_t n, bool full);
+percis_status sort_states(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uint64_t *tk, int32_t *tv, int64_t n,
+                          bool full, uint32_t *status, uint64_t *nheads);
 percis_status transpose_sort(percis_ctx *ctx);    // in-adjacency: edges sorted by target (valid row_ptr)
 percis_status transpose_finish(percis_ctx *ctx);  // in-adjacency: offsets (valid columns)
 

@@ -956,7 +956,7 @@ percis_status wait_graph(percis_ctx *ctx) {
     return PERCIS_OK;
 }
 
-percis_status prep_states(percis_ctx *ctx) {
+static percis_status prep_states_once(percis_ctx *ctx, bool full_sort, bool *again) {
     const int64_t n = ctx->n;
     uint32_t *st = ctx->status.as<uint32_t>();
     PERCIS_CUDA(ctx, cudaMemsetAsync(st, 0, 64, ctx->stream));
@@ -975,13 +975,17 @@ percis_status prep_states(percis_ctx *ctx) {
     uint64_t *k2 = k1 + n;
     int32_t *v2 = (int32_t *)(k2 + n);
     int32_t *perm = ctx->perm.as<int32_t>();
+    // the buffers the sort starts in, so that it ends in k1 and perm
+    const bool odd = state_sort_swaps(n, full_sort) & 1;
+    uint64_t *ka = odd ? k2 : k1, *kb = odd ? k1 : k2;
+    int32_t *va = odd ? v2 : perm, *vb = odd ? perm : v2;
     double *dscal = ctx->dscal.as<double>();  // c, smallest C_v, number of non-zero states
     const int g = grid_for(ctx, n, 256);
     PERCIS_CUDA(ctx, cudaMemsetAsync(dscal, 0, 64, ctx->stream));
     PERCIS_CUDA(ctx, cudaMemsetAsync(dscal + 1, 0x7f, sizeof(double), ctx->stream));  // 1.4e306, above every C_v
-    k_state_keys<<<g, 256, 0, ctx->stream>>>(ctx->x.as<double>(), n, k1, perm, st, dscal);
+    k_state_keys<<<g, 256, 0, ctx->stream>>>(ctx->x.as<double>(), n, ka, va, st, dscal);
     PERCIS_CHECK_LAUNCH(ctx, "state keys");
-    PERCIS_TRY(radix_sort_u64(ctx, k1, perm, k2, v2, n, 0, 64));
+    PERCIS_TRY(sort_states(ctx, ka, va, kb, vb, n, full_sort, st, reinterpret_cast<uint64_t *>(st) + 4));
     k_sorted_states<<<g, 256, 0, ctx->stream>>>(k1, n, ctx->xs.as<double>());
     PERCIS_CHECK_LAUNCH(ctx, "sorted states");
     // as many co-resident blocks as n terms fill (the kernel reads the number of
@@ -1015,6 +1019,8 @@ percis_status prep_states(percis_ctx *ctx) {
     PERCIS_CUDA(ctx, cudaMemcpyAsync(&b->status, st, 4, cudaMemcpyDeviceToHost, ctx->stream));
     PERCIS_CUDA(ctx, cudaMemcpyAsync(&b->tables, &tctl->status, 4, cudaMemcpyDeviceToHost, ctx->stream));
     PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    *again = (b->status & DEV_LONG_RUN) != 0;
+    if (*again) return PERCIS_OK;
     if (b->tables & DEV_TIMEOUT) return set_err(ctx, PERCIS_E_TIMEOUT, "table scan wait exceeded its budget");
     if (b->status & DEV_BAD_STATE) return set_err(ctx, PERCIS_E_INVALID, "states must lie in [0,1] (no NaN)");
     ctx->c_host = b->c;
@@ -1022,6 +1028,12 @@ percis_status prep_states(percis_ctx *ctx) {
     if (b->status & DEV_DEGENERATE)
         return set_err(ctx, PERCIS_E_DEGENERATE, "some C_v <= 0: percolation centrality undefined (all other states equal)");
     return PERCIS_OK;
+}
+
+percis_status prep_states(percis_ctx *ctx) {
+    bool again = false;
+    PERCIS_TRY(prep_states_once(ctx, false, &again));
+    return again ? prep_states_once(ctx, true, &again) : PERCIS_OK;
 }
 
 // lambda_v = c / C_v for every vertex

@@ -166,3 +166,33 @@ def test_pairs_without_divisions(binding, n, scale, kind):
     rs, rt, _, _ = oracle.sample_pairs(prep, 5, 1, 0, 4000)
     assert np.array_equal(_np(s), rs) and np.array_equal(_np(t), rt)
     eng.close()
+
+
+@pytest.mark.parametrize("n", [2, 3, 4095, 4096, 4097, 8193, 262144, 262145, 300001])
+@pytest.mark.parametrize("kind", ["uniform", "ties", "close", "packed"])
+def test_state_sort(binding, n, kind):
+    """The states' sort at its tiles, merges and radix passes: ties by vertex id, states
+    that agree in their upper 40 bits in short runs (close) and in runs long enough for
+    the second sort (packed): the stable order, and the tables that follow from it."""
+    rng = np.random.default_rng(n)
+    x = rng.random(n)
+    if kind == "ties":
+        x = np.round(x * 7) / 8
+    elif kind == "close":
+        x = np.floor(x * (n // 4 + 1)) / (n + 1) + rng.integers(0, 3, n) * 2.0 ** -50
+    elif kind == "packed":
+        x = 0.5 + rng.integers(0, 1000, n) * 2.0 ** -53
+    x[:2] = (1.0, 0.0)
+    g = synth.csr_from_edges(n, np.arange(n), (np.arange(n) + 1) % n, directed=True)
+    if not np.all(oracle.prepare(x, cv_method="sorted").Cv > 0):  # undefined: reported
+        assert n <= 3
+        with pytest.raises(RuntimeError, match="C_v <= 0"):
+            _engine(binding, g, x)
+        return
+    eng = _engine(binding, g, x)
+    p = eng.prep()
+    perm = np.argsort(-x, kind="stable")
+    assert np.array_equal(_np(p["perm"]), perm) and np.array_equal(_np(p["xs"]), x[perm])
+    w = np.cumsum(x[perm][::-1])[::-1]
+    assert np.array_equal(_np(p["w"])[1:n + 1], w)
+    eng.close()
