@@ -179,7 +179,8 @@ percis_status need_states(percis_ctx *ctx) {
     return PERCIS_OK;
 }
 
-uint32_t read_status(percis_ctx *ctx) {
+// (plain: the plain form's word too)
+uint32_t read_status(percis_ctx *ctx, bool plain = true) {
     char *hm = host_mirror(ctx);
     uint32_t st = 0, st2 = 0;
     uint32_t *d1 = hm ? reinterpret_cast<uint32_t *>(hm) : &st, *d2 = hm ? reinterpret_cast<uint32_t *>(hm) + 1 : &st2;
@@ -187,7 +188,7 @@ uint32_t read_status(percis_ctx *ctx) {
     *d2 = 0u;
     if (ctx->ms_ctl.p)
         cudaMemcpyAsync(d1, &ctx->ms_ctl.as<MsCtl>()->status, 4, cudaMemcpyDeviceToHost, ctx->stream);
-    if (ctx->plain_ctl.p)
+    if (plain && ctx->plain_ctl.p)
         cudaMemcpyAsync(d2, &ctx->plain_ctl.as<PlainCtl>()->status, 4, cudaMemcpyDeviceToHost, ctx->stream);
     cudaStreamSynchronize(ctx->stream);
     return *d1 | *d2;
@@ -226,9 +227,9 @@ void read_phase_stats(percis_ctx *ctx, double ell, PhaseOut *po) {
 
 // Reset status words and grid-barrier counters (a launch that gave up on a
 // bounded wait may leave a barrier half-arrived).
-void clear_status(percis_ctx *ctx) {
+void clear_status(percis_ctx *ctx, bool plain = true) {
     if (ctx->ms_ctl.p) cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream);
-    if (ctx->plain_ctl.p) cudaMemsetAsync(ctx->plain_ctl.p, 0, sizeof(PlainCtl), ctx->stream);
+    if (plain && ctx->plain_ctl.p) cudaMemsetAsync(ctx->plain_ctl.p, 0, sizeof(PlainCtl), ctx->stream);
 }
 
 }  // namespace
@@ -255,9 +256,11 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
     }
     ctx->have_paths = false;
     if (ctx->opt.instrument) PERCIS_TRY(ensure(ctx, ctx->counters, sizeof(unsigned long long) * 8, "counters"));
+    PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl), "ms ctl"));
+    const bool plain = ctx->opt.form == PERCIS_FORM_PLAIN;
     ctx->sigma_mode = 0;
     for (int attempt = 0; attempt < 24; ++attempt) {
-        clear_status(ctx);
+        clear_status(ctx, plain);
         ctx->ev_next = 0;
         if (ctx->opt.instrument)
             PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long) * 8, ctx->stream));
@@ -267,8 +270,10 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
             PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->acc_ap.p, 0, sizeof(double) * n, ctx->stream));
         }
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->arena_top.p, 0, 64, ctx->stream));
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ilen.p, 0, sizeof(int32_t) * cap_count, ctx->stream));
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->path_off.p, 0, sizeof(long long) * cap_count, ctx->stream));
+        if (ctx->opt.form != PERCIS_FORM_BIDIR) {  // (which writes both for every sample)
+            PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ilen.p, 0, sizeof(int32_t) * cap_count, ctx->stream));
+            PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->path_off.p, 0, sizeof(long long) * cap_count, ctx->stream));
+        }
         if (ctx->multi)
             PERCIS_TRY(multi_sample_pairs(ctx, seed, (uint32_t)phase));
         else
@@ -295,7 +300,7 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
             if (U > 0) PERCIS_TRY(batched_phase(ctx, seed, (uint32_t)(2 + phase), count, U, batches));
         }
         if (po->want_stats) PERCIS_TRY(issue_phase_stats(ctx, count, po->stats_pmax));
-        const uint32_t st = read_status(ctx);
+        const uint32_t st = read_status(ctx, plain);
         PERCIS_CUDA(ctx, cudaGetLastError());
         if (st & DEV_TIMEOUT) return set_err(ctx, PERCIS_E_TIMEOUT, "device wait exceeded its budget");
         if (st & DEV_NEED_LEVELS) {

@@ -1523,8 +1523,6 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
                                          ctx->stream));
         ctx->bi_epoch = 0;
     }
-    PERCIS_TRY(ensure(ctx, ctx->red, 64, "sample counter"));
-    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->red.p, 0, sizeof(unsigned long long), ctx->stream));
     BiArgs a = common_args(ctx, seed, tag_path);
     a.count = count;
     a.count_dev = count_dev;
@@ -1537,7 +1535,7 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
     a.queue = ctx->bi_queue.as<int2>();
     a.region = nslot;
     a.qcap = nslot;
-    a.next = ctx->red.as<unsigned long long>();
+    a.next = ctx->arena_top.as<unsigned long long>() + (BT == kBiBlock ? 1 : 2);
     a.heavy_edges = heavy_edges;
     a.heavy_auto = heavy_auto;
     a.deferred = defer;
@@ -1556,9 +1554,6 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
 // samples with a heavy level, or that outgrow their table, are handed over
 // untouched and run afterwards with 1,024 threads in the direct store.
 percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int64_t count) {
-    PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl), "ms ctl"));
-    // the status word may be freshly allocated: it must start at zero
-    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream));
     ctx->phase_span = count;
     if (ctx->opt.instrument >= 2) {
         PERCIS_TRY(ensure(ctx, ctx->bi_trace, sizeof(unsigned long long) * 8 * std::max<int64_t>(count, 1),
@@ -1587,8 +1582,8 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
                       "handed-over samples"));
     unsigned long long *defer_cost = ctx->bi_defer.as<unsigned long long>();
     int32_t *defer = reinterpret_cast<int32_t *>(defer_cost + cd);
-    unsigned int *n_def = reinterpret_cast<unsigned int *>(defer + cd);
-    PERCIS_CUDA(ctx, cudaMemsetAsync(n_def, 0, sizeof(unsigned int), ctx->stream));
+    // (counters beside the arena's, zeroed with it: [1] and [2] the passes' next samples)
+    unsigned int *n_def = reinterpret_cast<unsigned int *>(ctx->arena_top.as<unsigned long long>() + 3);
     int64_t nslot = ctx->n;
     if (ctx->multi) {
         const int32_t *gid;
@@ -1641,8 +1636,6 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
             ctx->bi_hslots = slots;
             ctx->bi_h0 = h0;
         }
-        PERCIS_TRY(ensure(ctx, ctx->red, 64, "sample counter"));
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->red.p, 0, sizeof(unsigned long long), ctx->stream));
         BiArgs a = common_args(ctx, seed, tag_path);
         a.count = count;
         a.list = nullptr;
@@ -1650,7 +1643,7 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
         a.queue = ctx->bi_hq.as<int2>();
         a.region = region;
         a.qcap = qcap;
-        a.next = ctx->red.as<unsigned long long>();
+        a.next = ctx->arena_top.as<unsigned long long>() + 1;
         a.h0_log = h0;
         a.hmax_log = hmax;
         a.slot_epoch = ctx->bi_hep.as<uint32_t>();

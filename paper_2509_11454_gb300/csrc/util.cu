@@ -96,6 +96,27 @@ __global__ void k_tile_scan(const T *in, T *out, int64_t n, const T *partial) {
     }
 }
 
+// up to one tile: its sums, their scan and the total in one launch
+template <class T>
+__global__ void k_scan_one(const T *in, T *out, int64_t n) {
+    __shared__ T tot;
+    const int64_t base = (int64_t)threadIdx.x * kScanItems;
+    T v[kScanItems];
+    T s = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        v[k] = base + k < n ? in[base + k] : T(0);
+        s += v[k];
+    }
+    T ex = block_excl(s, &tot);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (base + k < n) out[base + k] = ex;
+        ex += v[k];
+    }
+    if (threadIdx.x == 0) out[n] = tot;
+}
+
 template <class T>
 percis_status scan_impl(percis_ctx *ctx, const T *in, T *out, int64_t n) {
     // out has n+1 slots: out[n] = total
@@ -104,6 +125,11 @@ percis_status scan_impl(percis_ctx *ctx, const T *in, T *out, int64_t n) {
     T *partial = ctx->scratch.as<T>();
     if (n == 0) {
         PERCIS_CUDA(ctx, cudaMemsetAsync(out, 0, sizeof(T), ctx->stream));
+        return PERCIS_OK;
+    }
+    if (tiles == 1) {
+        k_scan_one<T><<<1, kScanBlock, 0, ctx->stream>>>(in, out, n);
+        PERCIS_CHECK_LAUNCH(ctx, "scan");
         return PERCIS_OK;
     }
     k_tile_sums<T><<<(unsigned)tiles, kScanBlock, 0, ctx->stream>>>(in, n, partial);
