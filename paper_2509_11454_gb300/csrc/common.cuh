@@ -139,7 +139,8 @@ struct alignas(8) GridBarrier {
     uint32_t gen;
 };
 
-__device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, uint64_t budget_ns) {
+__device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, uint64_t budget_ns,
+                                          uint32_t blocks) {
     __shared__ int s_ok;
     constexpr uint64_t kOver = 1ull << 63;
     __syncthreads();
@@ -150,7 +151,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, ui
         asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(a) : "l"(word), "l"(1ull) : "memory");
         int ok = (a & kOver) == 0;
         if (ok) {
-            const uint64_t g = gridDim.x;
+            const uint64_t g = blocks;
             const uint64_t round = a >> 32 ? a / g : (uint64_t)((uint32_t)a / (uint32_t)g);
             const uint64_t target = (round + 1) * g;
             if (a + 1 != target) {
@@ -176,6 +177,10 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, ui
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+__device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, uint64_t budget_ns) {
+    return grid_sync(bar, status, budget_ns, gridDim.x);
 }
 
 // ------------------------------------------------------------ warp helpers

@@ -65,6 +65,7 @@ struct MsArgs {
     uint64_t *fh;
     void *sigma;
     MsCtl *ctl;
+    uint32_t *status;                 // one word for all groups
     int32_t Lcap;
     int32_t lane_base;
     int32_t nlanes;
@@ -114,6 +115,23 @@ struct MsArgs {
     unsigned long long *ap_tau;       // [ap_warps][n]
     int32_t *ap_stamp;                // [ap_warps][n]
     int32_t *ap_list;                 // [ap_warps][2n]
+};
+
+// A launch's blocks form `groups` groups, each with a batch of its own and the state for
+// one (the arguments of group g are g[g]).  A batch alternates between passes over its
+// vertices and waits for their slowest block: one batch at a time kept the issue slots
+// 14% busy, half of every warp's time at a barrier.  The groups' blocks alternate on the
+// SMs, so one batch's passes fill another's waits.  Batched estimate on Barabasi-Albert
+// 100k: 11.3 ms with one group, 8.5 with two, 7.8 with three, 7.0 to 7.4 with four, 6.7
+// with six, 7.2 with eight; all-paths estimate of 20k: 3.3, 2.3, 2.2, 2.2, 2.3, 2.1.
+constexpr int kMaxGroups = 4;
+struct MsLaunch {
+    MsArgs g[kMaxGroups];
+    int32_t groups;
+};
+// a block's place in its group, and the group's blocks
+struct Place {
+    int32_t block, blocks;
 };
 
 template <int K>
@@ -198,7 +216,7 @@ __device__ __forceinline__ void gather_chunk(const ST *sig, int W, int w, uint64
 // in-degree > 32, nh, from the back of hq): of a vertex's level-L lanes, all
 // (every), or those of `cont` and need.
 template <int K, bool INSTR, int SM>
-__device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo, const int64_t *irp, int L,
+__device__ __noinline__ void count_level(const MsArgs &a, const Place at, int64_t n, int32_t vlo, const int64_t *irp, int L,
                                          const int32_t *lq, int64_t nl, const int32_t *hq, int64_t nh, bool every,
                                          const uint64_t *cont, bool *ovf_out, unsigned long long *work) {
     constexpr int W = 64 * K;
@@ -209,8 +227,8 @@ __device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo
     __shared__ S s_red[kMsBlock / 32][64];  // per-warp partial sums of a block-wide gather
     ST *sig = static_cast<ST *>(a.sigma);
     const int lane = threadIdx.x & 31, warp_in_block = threadIdx.x >> 5;
-    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t gwarp = ((int64_t)at.block * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)at.blocks * blockDim.x) >> 5;
     const int64_t nk = n * K;
     const uint64_t *fl = a.fh + (int64_t)L * nk;
     bool ovf = false;
@@ -226,7 +244,7 @@ __device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo
         // in-degree > kBlockDeg: one block per (vertex, word), its warps
         // splitting the edges; the partial sums meet in shared memory
         // (integer sums, so the order does not matter)
-        for (int64_t hi = blockIdx.x; hi < nh * K; hi += gridDim.x) {
+        for (int64_t hi = at.block; hi < nh * K; hi += at.blocks) {
             const int64_t h = hi / K;
             const int wd = (int)(hi - h * K);
             const int32_t v = __ldcg(&hq[-h]);
@@ -356,7 +374,7 @@ __device__ __noinline__ void count_level(const MsArgs &a, int64_t n, int32_t vlo
 // for K < 8): an edge's K words are one coalesced access and the OR over a row
 // stays in registers.
 template <int K, bool INSTR, int SM>
-__device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_base, const int32_t nlanes,
+__device__ __forceinline__ bool ms_batch(const MsArgs &a, const Place at, const int32_t lane_base, const int32_t nlanes,
                                          const int32_t vlo, const int64_t n, const int64_t *rp, const int64_t *irp,
                                          const int32_t ap_epoch) {
     constexpr int W = 64 * K;
@@ -372,11 +390,11 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
     unsigned long long n_s[2] = {0, 0}, n_uv = 0, n_ue = 0;  // sigma reads and writes; frontier vertices, edges
     MsCtl *ctl = a.ctl;
     GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
-    uint32_t *status = &ctl->status;
+    uint32_t *status = a.status;
     const int lane = threadIdx.x & 31;
     const int warp_in_block = threadIdx.x >> 5;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int64_t tid = (int64_t)at.block * blockDim.x + threadIdx.x;
+    const int64_t nthreads = (int64_t)at.blocks * blockDim.x;
     const int64_t gwarp = tid >> 5;
     const int64_t nwarps = nthreads >> 5;
     const int64_t nk = n * K;
@@ -398,7 +416,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         for (int64_t i = tid; i < 4 * (int64_t)(a.Lcap + 2); i += nthreads) a.ncnt[i] = 0;
     if (INSTR)
         for (int64_t i = tid; i < (int64_t)W * (a.Lcap + 1); i += nthreads) a.levdeg[i] = 0ull;
-    if (blockIdx.x == 0) {
+    if (at.block == 0) {
         for (int j = threadIdx.x; j < W; j += blockDim.x) a.remaining[j] = 0;
         if (threadIdx.x < K) {
             const int lo = threadIdx.x * 64;
@@ -418,7 +436,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
             ctl->t_start = globaltimer_ns();
         }
     }
-    if (!grid_sync(bar, status, a.budget_ns)) return false;
+    if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
     for (int64_t j = tid; j < nlanes; j += nthreads) {
         const int32_t v = a.lane_src[lane_base + j] - vlo;
         const uint64_t bit = 1ull << (j & 63);
@@ -433,7 +451,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
             a.remaining[j] = (int32_t)(q1 - q0);
         }
     }
-    if (!grid_sync(bar, status, a.budget_ns)) return false;
+    if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
 
     __shared__ unsigned long long s_nonempty[K];
     __shared__ unsigned long long s_act[K];
@@ -512,7 +530,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 }
             };
             // long rows one block each, then one warp per vertex
-            for (int64_t r = blockIdx.x; r < qh; r += gridDim.x) {
+            for (int64_t r = at.block; r < qh; r += at.blocks) {
                 const int32_t u = __ldcg(&qcur[n - 1 - r]);
                 push_edges(rp[u] + threadIdx.x / K, rp[u + 1], EB, __ldcg(&fcur[(int64_t)u * K + w]) & actw);
             }
@@ -523,7 +541,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         } else {
             // every vertex with unvisited active lanes; a row's scan stops once each
             // such lane has found a parent
-            for (int b = blockIdx.x; b < nbig; b += gridDim.x) {  // rows above kBigRow: a block each
+            for (int b = at.block; b < nbig; b += at.blocks) {  // rows above kBigRow: a block each
                 const int64_t v = (int64_t)a.big[b] - vlo;
                 if (v < 0 || v >= n) continue;  // (the same for the whole block)
                 const uint64_t c = actw & ~__ldcg(&a.vis[v * K + w]);
@@ -594,8 +612,8 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         }
         // full traversal: the counts of level L, whose frontier is settled, meanwhile
         if (a.full && L > 0)
-            count_level<K, INSTR, SM>(a, n, vlo, irp, L, qcur, qn, qcur + (n - 1), qh, true, nullptr, &ovf, n_s);
-        if (!grid_sync(bar, status, a.budget_ns)) return false;
+            count_level<K, INSTR, SM>(a, at, n, vlo, irp, L, qcur, qn, qcur + (n - 1), qh, true, nullptr, &ovf, n_s);
+        if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
         if (tid == 0 && L < 32) ctl->lvl_rec[L][4] = globaltimer_ns() - ctl->t_start;
 
         // ---- settle the new frontier: visited bits, non-empty lanes, the queue of its
@@ -674,7 +692,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
-            s_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+            s_last = atomicAdd(&ctl->ticket, 1u) == (uint32_t)at.blocks - 1u;
         }
         __syncthreads();
         if (s_last) {
@@ -715,7 +733,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 ctl->push_next = a.policy == 1 || (a.policy == 2 && a.push_alpha * (double)fe < (double)ue);
             }
         }
-        if (!grid_sync(bar, status, a.budget_ns)) return false;
+        if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
         ++L;
     }
 
@@ -745,7 +763,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                         if (m[q]) atomicOr((unsigned long long *)&a.need[(int64_t)u[q] * K + w], (unsigned long long)m[q]);
                 }
             };
-            for (int b = blockIdx.x; l > 1 && b < nbig; b += gridDim.x) {  // rows above kBigRow: a block each
+            for (int b = at.block; l > 1 && b < nbig; b += at.blocks) {  // rows above kBigRow: a block each
                 const int64_t v = (int64_t)a.big[b] - vlo;
                 if (v < 0 || v >= n) continue;
                 const uint64_t bits = __ldcg(&a.need[v * K + w]) & __ldcg(&fl[v * K + w]);
@@ -780,7 +798,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 }
             }
             flush(a.nlist + nl, &a.ncnt[2 * l], cap - nl);
-            if (!grid_sync(bar, status, a.budget_ns)) return false;
+            if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
             const int2 c = counts_at(a.ncnt + 2 * l);
             nl += c.x;
             nh += c.y;
@@ -791,9 +809,9 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 const int2 c = counts_at(a.ncnt + 2 * l);
                 nl -= c.x;
                 nh -= c.y;
-                count_level<K, INSTR, SM>(a, n, vlo, irp, l, a.nlist + nl, c.x, a.nlist + (cap - 1 - nh), c.y, false,
+                count_level<K, INSTR, SM>(a, at, n, vlo, irp, l, a.nlist + nl, c.x, a.nlist + (cap - 1 - nh), c.y, false,
                                           nullptr, &ovf, n_s);
-                if (!grid_sync(bar, status, a.budget_ns)) return false;
+                if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
             }
         } else {
             // every vertex of the lanes that go on, and what is needed of the others: the
@@ -817,10 +835,10 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                 if (l > 0) {
                     const int32_t *q = (l & 1) ? a.fq0 : a.fq1;  // listed one round ago
                     const int2 c = counts_at(dcnt + 2 * l);
-                    count_level<K, INSTR, SM>(a, n, vlo, irp, l, q, c.x, q + (n - 1), c.y, false,
+                    count_level<K, INSTR, SM>(a, at, n, vlo, irp, l, q, c.x, q + (n - 1), c.y, false,
                                               cone ? nullptr : a.cont + (int64_t)l * K, &ovf, n_s);
                 }
-                if (!grid_sync(bar, status, a.budget_ns)) return false;
+                if (!grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return false;
             }
         }
     }
@@ -984,14 +1002,14 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
                     const int64_t e = base + 32 * q + lane;
                     pv[q] = e < e1 ? a.icol[e] - vlo : -1;
                 }
-                bool at[kBackChunks];
+                bool in[kBackChunks];
 #pragma unroll
-                for (int q = 0; q < kBackChunks; ++q) at[q] = pv[q] >= 0 && (__ldcg(&fprev[(int64_t)pv[q] * K + wj]) & bj);
+                for (int q = 0; q < kBackChunks; ++q) in[q] = pv[q] >= 0 && (__ldcg(&fprev[(int64_t)pv[q] * K + wj]) & bj);
 #pragma unroll
-                for (int q = 0; q < kBackChunks; ++q) val[q] = at[q] ? (S)__ldcg(&sig[(int64_t)pv[q] * W + j]) : S(0);
+                for (int q = 0; q < kBackChunks; ++q) val[q] = in[q] ? (S)__ldcg(&sig[(int64_t)pv[q] * W + j]) : S(0);
 #pragma unroll
                 for (int q = 0; q < kBackChunks; ++q) {
-                    if (pick >= 0 || !__any_sync(0xffffffffu, at[q])) continue;
+                    if (pick >= 0 || !__any_sync(0xffffffffu, in[q])) continue;
                     // running sums are exact (integers; FP64 sums of integers below 2^53)
                     const S cum = carry + warp_incl_scan<S>(val[q]);
                     const unsigned hit = __ballot_sync(0xffffffffu, val[q] > S(0) && (double)cum >= target);
@@ -1023,11 +1041,14 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const int32_t lane_bas
 // the grouping left in device memory (W lanes each, so a phase needs no host
 // round trip), or are the single batch given in the arguments.
 template <int K, bool INSTR, int SM>
-__global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ MsArgs a) {
+__global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ MsLaunch l) {
     constexpr int W = 64 * K;
-    MsCtl *ctl = a.ctl;
-    GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
-    uint32_t *status = &ctl->status;
+    // (the groups' blocks alternate, so that every SM holds some of each)
+    const int32_t grp = (int32_t)blockIdx.x % l.groups;
+    const Place at{(int32_t)blockIdx.x / l.groups, (int32_t)gridDim.x / l.groups};
+    const MsArgs &a = l.g[grp];
+    GridBarrier *bar = reinterpret_cast<GridBarrier *>(a.ctl);
+    uint32_t *status = a.status;
     int64_t B = 1;
     long long U = 0;
     if (a.plan) {
@@ -1036,7 +1057,7 @@ __global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ M
         U = *a.u_dev;
         B = (U + W - 1) / W;
     }
-    for (int64_t b = 0; b < B; ++b) {
+    for (int64_t b = grp; b < B; b += l.groups) {
         int32_t lane_base = a.lane_base, nlanes = a.nlanes, vlo = a.vlo;
         int64_t n = a.n;
         if (a.plan) {
@@ -1048,9 +1069,9 @@ __global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ M
             lane_base = (int32_t)(b * W);
             nlanes = (int32_t)min((long long)W, U - b * W);
         }
-        // the previous batch's backtrack reads what this batch's prologue clears
-        if (b > 0 && !grid_sync(bar, status, a.budget_ns)) return;
-        if (!ms_batch<K, INSTR, SM>(a, lane_base, nlanes, vlo, n, a.rp + vlo, a.irp + vlo, a.ap_epoch)) return;
+        // the group's previous batch's backtrack reads what this batch's prologue clears
+        if (b > grp && !grid_sync(bar, status, a.budget_ns, (uint32_t)at.blocks)) return;
+        if (!ms_batch<K, INSTR, SM>(a, at, lane_base, nlanes, vlo, n, a.rp + vlo, a.irp + vlo, a.ap_epoch)) return;
     }
 }
 
@@ -1095,9 +1116,9 @@ int ms_grid(percis_ctx *ctx) {
 }
 
 template <int K, bool INSTR, int SM>
-percis_status launch_ms(percis_ctx *ctx, MsArgs &a) {
-    void *args[] = {&a};
-    const int grid = ms_grid<K, INSTR, SM>(ctx);
+percis_status launch_ms(percis_ctx *ctx, MsLaunch &l) {
+    void *args[] = {&l};
+    const int grid = ms_grid<K, INSTR, SM>(ctx) / l.groups * l.groups;
     PERCIS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_msbfs<K, INSTR, SM>, dim3(grid), dim3(kMsBlock),
                                                  args, 0, ctx->stream));
     ctx->launches++;
@@ -1105,8 +1126,8 @@ percis_status launch_ms(percis_ctx *ctx, MsArgs &a) {
 }
 
 template <int SM>
-percis_status launch_ms_k2(percis_ctx *ctx, int K, MsArgs &a) {
-    const bool instr = a.counters != nullptr;
+percis_status launch_ms_k2(percis_ctx *ctx, int K, MsLaunch &a) {
+    const bool instr = a.g[0].counters != nullptr;
     switch (K) {
         case 1: return instr ? launch_ms<1, true, SM>(ctx, a) : launch_ms<1, false, SM>(ctx, a);
         case 2: return instr ? launch_ms<2, true, SM>(ctx, a) : launch_ms<2, false, SM>(ctx, a);
@@ -1124,7 +1145,7 @@ int ms_grid_for(percis_ctx *ctx, int K) {
     }
 }
 
-percis_status launch_ms_k(percis_ctx *ctx, int K, MsArgs &a) {
+percis_status launch_ms_k(percis_ctx *ctx, int K, MsLaunch &a) {
     switch (ctx->sigma_mode) {
         case 0: return launch_ms_k2<0>(ctx, K, a);
         case 1: return launch_ms_k2<1>(ctx, K, a);
@@ -1230,23 +1251,66 @@ percis_status prep_ms_graph(percis_ctx *ctx, bool full) {
     return PERCIS_OK;
 }
 
-percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr, bool full) {
-    const int64_t n = nr;  // vertices of the largest launch range
-    const int K = W / 64;
-    PERCIS_TRY(ensure(ctx, ctx->fq0, sizeof(int32_t) * n, "frontier queue"));
-    PERCIS_TRY(ensure(ctx, ctx->fq1, sizeof(int32_t) * n, "frontier queue"));
-    PERCIS_TRY(ensure(ctx, ctx->vis, sizeof(uint64_t) * n * K, "visited bits"));
-    PERCIS_TRY(ensure(ctx, ctx->fhist, sizeof(uint64_t) * n * K * (int64_t)(Lcap + 1), "frontier history"));
-    PERCIS_TRY(ensure(ctx, ctx->sigmaW, sizeof(double) * n * W, "lane sigma"));
+// one group's share of each buffer, a multiple of 256 bytes
+size_t group_share(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+struct MsSizes {
+    size_t queue, vis, hist, sigma, list, levels;
+};
+MsSizes ms_sizes(int W, int Lcap, int64_t n) {
+    const size_t K = (size_t)W / 64;
+    MsSizes z;
+    z.queue = group_share(sizeof(int32_t) * (size_t)n);
+    z.vis = group_share(sizeof(uint64_t) * (size_t)n * K);
+    z.hist = group_share(sizeof(uint64_t) * (size_t)n * K * (size_t)(Lcap + 1));
+    z.sigma = group_share(sizeof(double) * (size_t)n * W);
+    z.list = group_share(sizeof(int32_t) * 2 * (size_t)n);
+    z.levels = group_share((sizeof(int32_t) * 4 + sizeof(uint64_t) * K) * (size_t)(Lcap + 2));
+    return z;
+}
+
+percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr, bool full, int groups) {
+    const MsSizes z = ms_sizes(W, Lcap, nr);  // nr: vertices of the largest launch range
+    PERCIS_TRY(ensure(ctx, ctx->fq0, z.queue * groups, "frontier queue"));
+    PERCIS_TRY(ensure(ctx, ctx->fq1, z.queue * groups, "frontier queue"));
+    PERCIS_TRY(ensure(ctx, ctx->vis, z.vis * groups, "visited bits"));
+    PERCIS_TRY(ensure(ctx, ctx->fhist, z.hist * groups, "frontier history"));
+    PERCIS_TRY(ensure(ctx, ctx->sigmaW, z.sigma * groups, "lane sigma"));
     if (!full) {
-        PERCIS_TRY(ensure(ctx, ctx->ms_need, sizeof(uint64_t) * n * K, "needed lanes"));
-        PERCIS_TRY(ensure(ctx, ctx->ms_list, sizeof(int32_t) * 2 * n, "needed vertices"));
-        PERCIS_TRY(ensure(ctx, ctx->ms_levels, (sizeof(int32_t) * 4 + sizeof(uint64_t) * K) * (size_t)(Lcap + 2),
-                          "level counts"));
+        PERCIS_TRY(ensure(ctx, ctx->ms_need, z.vis * groups, "needed lanes"));
+        PERCIS_TRY(ensure(ctx, ctx->ms_list, z.list * groups, "needed vertices"));
+        PERCIS_TRY(ensure(ctx, ctx->ms_levels, z.levels * groups, "level counts"));
     }
-    PERCIS_TRY(ensure(ctx, ctx->remaining, sizeof(int32_t) * 512, "lane remaining"));
-    PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl), "ms ctl"));
+    PERCIS_TRY(ensure(ctx, ctx->remaining, sizeof(int32_t) * 512 * groups, "lane remaining"));
+    PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl) * groups, "ms ctl"));
     return PERCIS_OK;
+}
+
+// Group g's arguments: those of group 0 with its own share of every buffer.
+MsArgs group_args(const MsArgs &a0, const MsSizes &z, int g, int64_t ap_n) {
+    MsArgs a = a0;
+    auto at = [g](auto *p, size_t bytes) {
+        using T = decltype(p);
+        return reinterpret_cast<T>(reinterpret_cast<char *>(p) + bytes * (size_t)g);
+    };
+    a.ctl = a0.ctl + g;
+    a.fq0 = at(a0.fq0, z.queue);
+    a.fq1 = at(a0.fq1, z.queue);
+    a.vis = at(a0.vis, z.vis);
+    a.fh = at(a0.fh, z.hist);
+    a.sigma = reinterpret_cast<char *>(a0.sigma) + z.sigma * (size_t)g;
+    a.need = at(a0.need, z.vis);
+    a.nlist = at(a0.nlist, z.list);
+    a.cont = at(a0.cont, z.levels);
+    a.ncnt = at(a0.ncnt, z.levels);
+    a.remaining = a0.remaining + 512 * g;
+    if (a0.allpaths) {
+        const int64_t w = (int64_t)a0.ap_warps * g;
+        a.ap_tau = a0.ap_tau + w * ap_n;
+        a.ap_stamp = a0.ap_stamp + w * ap_n;
+        a.ap_list = a0.ap_list + 2 * w * ap_n;
+    }
+    return a;
 }
 
 void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
@@ -1265,6 +1329,7 @@ void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
     a.fh = ctx->fhist.as<uint64_t>();
     a.sigma = ctx->sigmaW.p;
     a.ctl = ctx->ms_ctl.as<MsCtl>();
+    a.status = &a.ctl->status;
     a.Lcap = Lcap;
     a.budget_ns = (uint64_t)(ctx->opt.timeout_s * 1e9);
     a.rp = ctx->rp.as<int64_t>();
@@ -1315,13 +1380,21 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
         const int64_t lmem = (16ll << 30) / std::max<int64_t>(1, nr_max * K * 8) - 1;
         Lcap = (int)std::max<int64_t>(Lcap, std::min<int64_t>(ctx->vertex_diam + 3, std::min<int64_t>(lmem, 1 << 20)));
     }
+    const int64_t B = ctx->multi ? (int64_t)plan.size() : (n_sources + W - 1) / W;
+    // batches side by side, while their state stays within 24 GiB (the work counters and
+    // the level records are those of one batch at a time)
+    int G = 1;
+    if (!ctx->opt.instrument) {
+        const MsSizes z = ms_sizes(W, Lcap, nr_max);
+        const size_t each = 2 * z.queue + 2 * z.vis + z.hist + z.sigma + z.list + z.levels;
+        while (G < kMaxGroups && G + 1 <= B && (size_t)(G + 1) * each <= (24ull << 30)) ++G;
+    }
     PERCIS_TRY(prep_ms_graph(ctx, false));
-    PERCIS_TRY(ensure_ms(ctx, W, Lcap, nr_max, false));
+    PERCIS_TRY(ensure_ms(ctx, W, Lcap, nr_max, false, G));
     ctx->levels_alloc = Lcap;
     ctx->lanes_alloc = W;
     PERCIS_TRY(ensure(ctx, ctx->found, sizeof(int32_t) * (count + 1), "found"));
-    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream));
-    const int64_t B = ctx->multi ? (int64_t)plan.size() : (n_sources + W - 1) / W;
+    PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl) * G, ctx->stream));
     *batches = B;
     MsArgs a{};
     fill_common(ctx, a, Lcap, K, nr_max);
@@ -1353,7 +1426,9 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
         const int64_t n = nr_max;
         const int64_t per_warp = 20 * n;
         const int64_t warps = (int64_t)ms_grid_for(ctx, K) * (kMsBlock / 32);
-        const int64_t ap_warps = std::max<int64_t>(1, std::min<int64_t>(warps, (8ll << 30) / per_warp));
+        // (a group's warps have their own)
+        const int64_t ap_group = std::max<int64_t>(1, std::min<int64_t>(warps, (8ll << 30) / per_warp) / G);
+        const int64_t ap_warps = ap_group * G;
         if (ctx->ap_warps != ap_warps || ctx->ap_n != n) {
             PERCIS_TRY(ensure(ctx, ctx->ap_tau, sizeof(unsigned long long) * n * ap_warps, "all-paths tau"));
             PERCIS_TRY(ensure(ctx, ctx->ap_stamp, sizeof(int32_t) * n * ap_warps, "all-paths stamps"));
@@ -1367,7 +1442,7 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
             PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ap_stamp.p, 0, sizeof(int32_t) * n * ap_warps, ctx->stream));
             ctx->ap_epoch = 0;
         }
-        a.ap_warps = (int32_t)ap_warps;
+        a.ap_warps = (int32_t)ap_group;
         a.acc_ap = ctx->acc_ap.as<double>();
         a.ap_tau = ctx->ap_tau.as<unsigned long long>();
         a.ap_stamp = ctx->ap_stamp.as<int32_t>();
@@ -1389,7 +1464,13 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
     // every batch of the phase in one persistent launch
     cudaEvent_t e0 = next_event(ctx), e1 = next_event(ctx);
     if (e0) cudaEventRecord(e0, ctx->stream);
-    PERCIS_TRY(launch_ms_k(ctx, K, a));
+    MsLaunch l{};
+    l.groups = G;
+    {
+        const MsSizes z = ms_sizes(W, Lcap, nr_max);
+        for (int g = 0; g < G; ++g) l.g[g] = group_args(a, z, g, nr_max);
+    }
+    PERCIS_TRY(launch_ms_k(ctx, K, l));
     if (e1) cudaEventRecord(e1, ctx->stream);
     return PERCIS_OK;
 }
@@ -1403,7 +1484,7 @@ percis_status msbfs_full(percis_ctx *ctx, int32_t nsrc, const int32_t *sources, 
     int Lcap = std::max(ctx->levels_alloc, 32);
     for (int attempt = 0; attempt < 12; ++attempt) {
         PERCIS_TRY(prep_ms_graph(ctx, true));
-        PERCIS_TRY(ensure_ms(ctx, W, Lcap, ctx->n, true));
+        PERCIS_TRY(ensure_ms(ctx, W, Lcap, ctx->n, true, 1));
         ctx->levels_alloc = Lcap;
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream));
         MsArgs a{};
@@ -1413,7 +1494,10 @@ percis_status msbfs_full(percis_ctx *ctx, int32_t nsrc, const int32_t *sources, 
         a.nlanes = nsrc;
         a.remaining = ctx->remaining.as<int32_t>();
         a.full = 1;
-        PERCIS_TRY(launch_ms_k(ctx, K, a));
+        MsLaunch l{};
+        l.groups = 1;
+        l.g[0] = a;
+        PERCIS_TRY(launch_ms_k(ctx, K, l));
         MsCtl hc;
         PERCIS_CUDA(ctx, cudaMemcpyAsync(&hc, ctx->ms_ctl.p, sizeof(hc), cudaMemcpyDeviceToHost, ctx->stream));
         PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

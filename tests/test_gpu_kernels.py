@@ -196,3 +196,31 @@ def test_state_sort(binding, n, kind):
     w = np.cumsum(x[perm][::-1])[::-1]
     assert np.array_equal(_np(p["w"])[1:n + 1], w)
     eng.close()
+
+
+@pytest.mark.parametrize("count", [2, 40, 90, 200, 600])
+@pytest.mark.parametrize("estimator", ["", "allpaths"])
+def test_batches_side_by_side(binding, count, estimator):
+    """Batches of 64 lanes from one to more than the groups that run side by side: every
+    group's state is its own (counts and paths equal the oracle's; the all-paths sums
+    equal those of one batch at a time to the rounding of their additions)."""
+    g = synth.barabasi_albert(500, 3, 2)
+    x = synth.states_uniform(g.n, 2)
+    if estimator:
+        est = []
+        for instrument in (0, 1):
+            eng = _engine(binding, g, x, estimator="allpaths", lanes=64, ell1=count, ell=count, instrument=instrument)
+            pc, _ = eng.estimate(0.05, 0.1, 4)
+            est.append(_np(pc))
+            eng.close()
+        # each sum has at most `count` positive terms, in any order: (count - 1) roundings a
+        # side, and a few after it
+        assert np.all(np.abs(est[0] - est[1]) <= 2 * (count + 4) * 2.0 ** -53 * est[1])
+        return
+    eng = _engine(binding, g, x, lanes=64)
+    ph = eng.run_phase(4, 1, count)
+    ptr, nodes = (_np(v) for v in eng.get_paths(count))
+    ref = oracle.run_samples(oracle.from_synth(g), oracle.prepare(x), 4, 1, 3, 0, count, keep_paths=True)
+    assert np.array_equal(_np(ph["cnt"]), ref.cnt)
+    assert np.array_equal(_np(ph["ilen"]), ref.ilen) and np.array_equal(nodes, ref.path_nodes)
+    eng.close()
