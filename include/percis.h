@@ -95,8 +95,8 @@ typedef struct {
                                  gets sigma_sv sigma_vt / sigma_st (same expectation; the
                                  Rao-Blackwellised form; batched form only; no backward) */
     double push_alpha;        /* direction 2 threshold; 0 = default (1) */
-    int32_t cuda_graphs;      /* 1: a many-graph context records the per-graph pair-sampling
-                                 launches of a phase once in a CUDA graph and replays it while
+    int32_t cuda_graphs;      /* 1: a many-graph context records the pair-sampling launch of
+                                 a phase once in a CUDA graph and replays it while
                                  the per-graph sample counts repeat (phase 1 always does);
                                  the seed is read from device memory, results are unchanged */
     int32_t bi_table_log;     /* bidirectional form, store of the first pass: 0 (default) = the

@@ -17,23 +17,35 @@ namespace percis {
 
 namespace {
 
+// The sampled pairs' terms.  Eight lanes share a sample: a path's divisions (~25 FP64
+// operations each, the chain of one thread) run side by side, where one thread a sample
+// took 31 us on paths of a hundred vertices.  One launch covers the samples of many
+// graphs (gid: graph of every vertex; C and l are per graph).
 __global__ void k_bw_samples(int64_t count, const int32_t *s, const int32_t *t, const int32_t *kind,
                              const int32_t *ilen, const long long *path_off, const int32_t *arena, const double *g,
-                             const double *Cv, const double *x, const double *dscal, double ell, double *grad) {
-    const double C = dscal[0];
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
-        if (kind[i] != 0) continue;
-        const int32_t si = s[i], ti = t[i];
+                             const double *Cv, const double *x, const double *C, const int32_t *gid,
+                             const double *ells, double ell, double *grad) {
+    const int sub = threadIdx.x & 7;
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < count; i += stride) {
+        if (kind[i] != 0) continue;  // (the same for the eight lanes)
+        const int32_t si = s[i], ti = t[i], len = ilen[i];
         const long long off = path_off[i];
         double S = 0.0;
-        for (int q = 0; q < ilen[i]; ++q) {
+        for (int q = sub; q < len; q += 8) {
             const int32_t v = arena[off + q];
             S += g[v] / Cv[v];
         }
-        const double coef = (C / ell) * S / (x[si] - x[ti]);
-        atomicAdd(&grad[si], coef);
-        atomicAdd(&grad[ti], -coef);
+        const unsigned m = 0xffu << (threadIdx.x & 24);
+        S += __shfl_xor_sync(m, S, 1);
+        S += __shfl_xor_sync(m, S, 2);
+        S += __shfl_xor_sync(m, S, 4);
+        if (sub < 2) {
+            const int32_t gr = gid ? gid[si] : 0;
+            const double coef = (C[gr] / (ells ? ells[gr] : ell)) * S / (x[si] - x[ti]);
+            if (sub == 0) atomicAdd(&grad[si], coef);
+            else atomicAdd(&grad[ti], -coef);
+        }
     }
 }
 
@@ -68,22 +80,27 @@ __global__ void k_bw_final(int64_t n, const int32_t *perm, const int32_t *glo, c
 
 }  // namespace
 
-percis_status backward_fixed(percis_ctx *ctx, const double *g, double *grad) {
-    const int64_t n = ctx->n, count = ctx->phase_count;
-    PERCIS_CUDA(ctx, cudaMemsetAsync(grad, 0, sizeof(double) * n, ctx->stream));
-    const int block = 256;
-    k_bw_samples<<<grid_for(ctx, count, block), block, 0, ctx->stream>>>(
+percis_status backward_samples(percis_ctx *ctx, int64_t count, const double *g, double *grad, const double *C, const int32_t *gid,
+                               const double *ells) {
+    PERCIS_CUDA(ctx, cudaMemsetAsync(grad, 0, sizeof(double) * ctx->n, ctx->stream));
+    k_bw_samples<<<grid_for(ctx, count * 8, 256), 256, 0, ctx->stream>>>(
         count, ctx->pair_s.as<int32_t>(), ctx->pair_t.as<int32_t>(), ctx->kind.as<int32_t>(),
         ctx->ilen.as<int32_t>(), ctx->path_off.as<long long>(), ctx->arena.as<int32_t>(), g, ctx->Cv.as<double>(),
-        ctx->x.as<double>(), ctx->dscal.as<double>(), (double)ctx->last_ell, grad);
+        ctx->x.as<double>(), C, gid, ells, (double)ctx->last_ell, grad);
     PERCIS_CHECK_LAUNCH(ctx, "backward samples");
+    return PERCIS_OK;
+}
+
+percis_status backward_vertices(percis_ctx *ctx, const double *g, const unsigned long long *cnt, double ell,
+                                double *grad) {
+    const int64_t n = ctx->n;
+    const int block = 256;
     PERCIS_TRY(ensure(ctx, ctx->grad_tmp, sizeof(double) * (2 * n + 2), "backward scan"));
     double *gs = ctx->grad_tmp.as<double>();
     double *G = gs + n;
     k_bw_gamma<<<grid_for(ctx, n, block), block, 0, ctx->stream>>>(n, ctx->perm.as<int32_t>(), g,
-                                                                  ctx->dscal.as<double>(),
-                                                                  ctx->cnt.as<unsigned long long>(),
-                                                                  ctx->Cv.as<double>(), (double)ctx->last_ell, gs);
+                                                                  ctx->dscal.as<double>(), cnt,
+                                                                  ctx->Cv.as<double>(), ell, gs);
     PERCIS_CHECK_LAUNCH(ctx, "backward gamma");
     PERCIS_TRY(scan_exclusive_f64(ctx, gs, G, n));
     PERCIS_TRY(prep_groups(ctx));
@@ -92,6 +109,11 @@ percis_status backward_fixed(percis_ctx *ctx, const double *g, double *grad) {
                                                                   ctx->grp_hi.as<int32_t>(), gs, G, grad);
     PERCIS_CHECK_LAUNCH(ctx, "backward final");
     return PERCIS_OK;
+}
+
+percis_status backward_fixed(percis_ctx *ctx, const double *g, double *grad) {
+    PERCIS_TRY(backward_samples(ctx, ctx->phase_count, g, grad, ctx->dscal.as<double>(), nullptr, nullptr));
+    return backward_vertices(ctx, g, ctx->cnt.as<unsigned long long>(), (double)ctx->last_ell, grad);
 }
 
 }  // namespace percis

@@ -91,6 +91,18 @@ __device__ __forceinline__ double uniform_at(uint64_t seed, uint64_t i, uint32_t
     return __dmul_rn((double)((w >> 11) + 1), 0x1p-53);
 }
 
+// ------------------------------------------------------------ many graphs
+// graph of sample i: soff[g] <= i < soff[g + 1]
+__device__ __forceinline__ int32_t graph_of_sample(const long long *soff, int32_t G, long long i) {
+    int32_t lo = 0, hi = G;  // soff[lo] <= i < soff[hi]
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (soff[mid] <= i) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
 // ------------------------------------------------------------ timers/atomics
 
 __device__ __forceinline__ uint64_t globaltimer_ns() {

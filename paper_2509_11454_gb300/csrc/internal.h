@@ -42,6 +42,14 @@ struct alignas(16) MsCtl {
                                         // time after phase A, time after the queue build
 };
 
+// A graph's sampling tables (Algorithm 2) on the device; vlo: its first vertex in a union.
+struct PairTables {
+    int64_t n;
+    const double *xs, *w, *ci, *r, *dscal, *x;
+    const int32_t *perm;
+    int32_t vlo;
+};
+
 struct PlainCtl {
     uint32_t bar_count, bar_gen;
     uint32_t status;
@@ -226,9 +234,11 @@ percis_status wait_graph(percis_ctx *ctx);  // the context stream waits for the 
 percis_status prep_vorder(percis_ctx *ctx);  // lane order of the batched form (on first use)
 
 // sampler.cu
+PairTables pair_tables(percis_ctx *ctx, int32_t vlo);
 percis_status sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag, int64_t i0, int64_t count, int32_t *s,
-                           int32_t *t, int32_t *kind, const uint64_t *seed_dev = nullptr,
-                           cudaStream_t stream = nullptr);
+                           int32_t *t, int32_t *kind);
+percis_status sample_pairs_multi(percis_ctx *ctx, const PairTables *tab, const long long *soff, int32_t G,
+                                 uint64_t seed, const uint64_t *seed_dev, uint32_t tag, int64_t total);
 percis_status group_by_source(percis_ctx *ctx, int64_t count, int64_t *n_sources, int64_t *n_valid);
 
 // bfs_plain.cu
@@ -250,6 +260,12 @@ int choose_lanes(percis_ctx *ctx, int64_t n_sources);
 
 // backward.cu
 percis_status backward_fixed(percis_ctx *ctx, const double *g, double *grad);
+// its two halves: the sampled pairs' terms (grad is cleared first; C, ells: one value, or
+// one per graph with gid the graph of every vertex), and the vertices' terms
+percis_status backward_samples(percis_ctx *ctx, int64_t count, const double *g, double *grad, const double *C, const int32_t *gid,
+                               const double *ells);
+percis_status backward_vertices(percis_ctx *ctx, const double *g, const unsigned long long *cnt, double ell,
+                                double *grad);
 
 // exact.cu
 percis_status exact_pc(percis_ctx *ctx, double *pc);

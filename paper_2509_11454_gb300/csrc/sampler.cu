@@ -35,46 +35,73 @@ struct QuotientTest {
     }
 };
 
-// One thread per sample: Philox4x32-10 gives (u_s, u_t); two binary searches
-// exactly as Algorithm 2 (appendix) over the 1-based tables, evaluated with
-// explicit round-to-nearest operations so no multiply-add is fused.
-__global__ void k_sample_pairs(int64_t n, const double *__restrict__ xs, const int32_t *__restrict__ perm,
-                               const double *__restrict__ w, const double *__restrict__ ci,
-                               const double *__restrict__ r, const double *__restrict__ dscal,
-                               const double *__restrict__ x, uint64_t seed, const uint64_t *seed_dev, uint32_t tag,
-                               int64_t i0, int64_t count, int32_t *s_out, int32_t *t_out, int32_t *kind) {
-    const double c = dscal[0];
-    if (seed_dev) seed = *seed_dev;  // a recorded launch reads the seed of the current call
+// One pair from (u_s, u_t): two binary searches exactly as Algorithm 2 (appendix) over
+// the 1-based tables, evaluated with explicit round-to-nearest operations so no
+// multiply-add is fused.
+__device__ __forceinline__ void sample_pair(const PairTables &q, double us, double ut, int32_t &s_out, int32_t &t_out,
+                                            int32_t &kind) {
+    const double *__restrict__ xs = q.xs, *__restrict__ w = q.w, *__restrict__ r = q.r;
+    const int64_t n = q.n;
+    const double c = q.dscal[0];
+    int64_t a = 1, b = n, d = (a + b) >> 1;
+    const QuotientTest first(us, c);
+    while (a <= b) {
+        if (first(__dsub_rn(c, r[d + 1]))) b = d - 1;
+        else a = d + 1;
+        d = (a + b) >> 1;
+    }
+    const int64_t s = b + 1;
+    const double xss = xs[s - 1], wss = w[s], css = q.ci[s];
+    a = s;
+    b = n;
+    d = (a + b) >> 1;
+    const QuotientTest second(ut, css);
+    while (a <= b) {
+        const double num = __dadd_rn(__dsub_rn(__dmul_rn((double)(d - s + 1), xss), wss), w[d + 1]);
+        if (second(num)) b = d - 1;
+        else a = d + 1;
+        d = (a + b) >> 1;
+    }
+    // t <= n whenever c_s > 0, which holds for every s the first search can
+    // return; the clamp only keeps the index in bounds.
+    const int64_t t = b + 1 <= n ? b + 1 : n;
+    s_out = q.perm[s - 1];
+    t_out = q.perm[t - 1];
+    kind = (__dsub_rn(q.x[s_out], q.x[t_out]) > 0.0) ? 0 : 1;
+}
+
+// One thread per sample: Philox4x32-10 gives (u_s, u_t).
+__global__ void k_sample_pairs(const __grid_constant__ PairTables q, uint64_t seed, uint32_t tag, int64_t i0,
+                               int64_t count, int32_t *s_out, int32_t *t_out, int32_t *kind) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += stride) {
         double us, ut;
         uniforms2(seed, (uint64_t)(i0 + k), tag, 0u, us, ut);
-        int64_t a = 1, b = n, d = (a + b) >> 1;
-        const QuotientTest first(us, c);
-        while (a <= b) {
-            if (first(__dsub_rn(c, r[d + 1]))) b = d - 1;
-            else a = d + 1;
-            d = (a + b) >> 1;
-        }
-        const int64_t s = b + 1;
-        const double xss = xs[s - 1], wss = w[s], css = ci[s];
-        a = s;
-        b = n;
-        d = (a + b) >> 1;
-        const QuotientTest second(ut, css);
-        while (a <= b) {
-            const double num = __dadd_rn(__dsub_rn(__dmul_rn((double)(d - s + 1), xss), wss), w[d + 1]);
-            if (second(num)) b = d - 1;
-            else a = d + 1;
-            d = (a + b) >> 1;
-        }
-        // t <= n whenever c_s > 0, which holds for every s the first search can
-        // return; the clamp only keeps the index in bounds.
-        const int64_t t = b + 1 <= n ? b + 1 : n;
-        const int32_t sn = perm[s - 1], tn = perm[t - 1];
+        int32_t sn, tn, kd;
+        sample_pair(q, us, ut, sn, tn, kd);
         if (s_out) s_out[k] = sn;
         if (t_out) t_out[k] = tn;
-        if (kind) kind[k] = (__dsub_rn(x[sn], x[tn]) > 0.0) ? 0 : 1;
+        if (kind) kind[k] = kd;
+    }
+}
+
+// The same for the samples of many graphs in one launch (graph g's samples are
+// soff[g] .. soff[g + 1] - 1; ids of the union).  A launch a graph, one after the other,
+// paid the searches' latency (~15 us) for every graph.
+__global__ void k_sample_pairs_multi(const PairTables *tab, const long long *soff, int32_t G, uint64_t seed,
+                                     const uint64_t *seed_dev, uint32_t tag, int64_t total, int32_t *s_out,
+                                     int32_t *t_out, int32_t *kind) {
+    if (seed_dev) seed = *seed_dev;  // a recorded launch reads the seed of the current call
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        const PairTables q = tab[graph_of_sample(soff, G, i)];
+        double us, ut;
+        uniforms2(seed, (uint64_t)i, tag, 0u, us, ut);
+        int32_t sn, tn, kd;
+        sample_pair(q, us, ut, sn, tn, kd);
+        s_out[i] = sn + q.vlo;
+        t_out[i] = tn + q.vlo;
+        kind[i] = kd;
     }
 }
 
@@ -131,15 +158,35 @@ __global__ void k_lane_tables(const long long *src_count, const long long *src_o
 
 }  // namespace
 
+PairTables pair_tables(percis_ctx *ctx, int32_t vlo) {
+    return {ctx->n,
+            ctx->xs.as<double>(),
+            ctx->w.as<double>(),
+            ctx->ci.as<double>(),
+            ctx->r.as<double>(),
+            ctx->dscal.as<double>(),
+            ctx->x.as<double>(),
+            ctx->perm.as<int32_t>(),
+            vlo};
+}
+
 percis_status sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag, int64_t i0, int64_t count, int32_t *s,
-                           int32_t *t, int32_t *kind, const uint64_t *seed_dev, cudaStream_t stream) {
+                           int32_t *t, int32_t *kind) {
     if (count <= 0) return PERCIS_OK;
     const int block = 256;
-    k_sample_pairs<<<grid_for(ctx, count, block), block, 0, stream ? stream : ctx->stream>>>(
-        ctx->n, ctx->xs.as<double>(), ctx->perm.as<int32_t>(), ctx->w.as<double>(), ctx->ci.as<double>(),
-        ctx->r.as<double>(), ctx->dscal.as<double>(), ctx->x.as<double>(), seed, seed_dev, tag, i0, count, s, t,
-        kind);
+    k_sample_pairs<<<grid_for(ctx, count, block), block, 0, ctx->stream>>>(pair_tables(ctx, 0), seed, tag, i0, count,
+                                                                         s, t, kind);
     PERCIS_CHECK_LAUNCH(ctx, "sample pairs");
+    return PERCIS_OK;
+}
+
+percis_status sample_pairs_multi(percis_ctx *ctx, const PairTables *tab, const long long *soff, int32_t G,
+                                 uint64_t seed, const uint64_t *seed_dev, uint32_t tag, int64_t total) {
+    if (total <= 0) return PERCIS_OK;
+    k_sample_pairs_multi<<<grid_for(ctx, total, 256), 256, 0, ctx->stream>>>(
+        tab, soff, G, seed, seed_dev, tag, total, ctx->pair_s.as<int32_t>(), ctx->pair_t.as<int32_t>(),
+        ctx->kind.as<int32_t>());
+    PERCIS_CHECK_LAUNCH(ctx, "sample pairs of many graphs");
     return PERCIS_OK;
 }
 

@@ -224,3 +224,30 @@ def test_batches_side_by_side(binding, count, estimator):
     assert np.array_equal(_np(ph["cnt"]), ref.cnt)
     assert np.array_equal(_np(ph["ilen"]), ref.ilen) and np.array_equal(nodes, ref.path_nodes)
     eng.close()
+
+
+def test_many_graphs_sampling_and_backward_in_one_launch(binding):
+    """Path graphs whose samples have up to 1, 7, 8, 9, 16, 17 and 38 internal vertices
+    (eight lanes share a sample): pairs, counts and gradients of each graph in the batch
+    are the oracle's."""
+    sizes = [3, 9, 10, 11, 18, 19, 40]
+    graphs = [synth.csr_from_edges(n, np.arange(n - 1), np.arange(1, n), directed=False) for n in sizes]
+    vptr, rp, col = synth.union_csr(graphs)
+    x = synth.states_uniform(int(vptr[-1]), 3)
+    fixed = 300
+    eng = binding.PercIS(0)
+    eng.set_options(form="bidir", ell1=100, ell=fixed)
+    eng.load_graphs(vptr, rp, col)
+    eng.set_states(x)
+    pc = _np(eng.estimate_graphs(0.05, 0.1, seed=2)[0])
+    gvec = np.random.default_rng(3).standard_normal(int(vptr[-1]))
+    gx = _np(eng.backward(torch.as_tensor(gvec, device="cuda")))
+    for g, graph in enumerate(graphs):
+        lo, hi = vptr[g], vptr[g + 1]
+        prep = oracle.prepare(x[lo:hi], cv_method="sorted")
+        ph = oracle.run_samples(oracle.from_synth(graph), prep, 2, 1, 3, g * fixed, fixed, keep_paths=True, bidir=True)
+        F = prep.lam * ph.cnt / fixed
+        assert np.max(np.abs(pc[lo:hi] - F)) <= 1e-9, g
+        ref = oracle.vjp_fixed(prep, fixed, ph, F, gvec[lo:hi])
+        assert np.linalg.norm(gx[lo:hi] - ref) <= 1e-10 * np.linalg.norm(ref), g
+    eng.close()
