@@ -54,11 +54,15 @@ constexpr int kBiBlock = PERCIS_BI_BLOCK;
 #ifndef PERCIS_MEET_CAP
 #define PERCIS_MEET_CAP 256
 #endif
+#ifndef PERCIS_HEAVY_BLOCK
+#define PERCIS_HEAVY_BLOCK 1024
+#endif
+constexpr int kHeavyBlock = PERCIS_HEAVY_BLOCK;  // threads per sample in the heavy pass
+constexpr int kSmallBlock = 128;  // threads per sample on small graphs (see small_graph)
 constexpr int kMeetCap = PERCIS_MEET_CAP;  // meeting-layer members kept in shared memory
 constexpr int kMeetBuckets = 1024;          // id buckets per round of the large-layer search
 constexpr int kBackWarp = 256;              // candidate lists up to this length: one warp per backtrack step
 constexpr int kLvCap = 64;                  // levels per side whose queue ranges are kept (reverse backtrack)
-constexpr int kFlat = 512;  // frontier vertices per chunk whose edges are spread over the block
 #ifndef PERCIS_EDGE_BATCH
 #define PERCIS_EDGE_BATCH 2
 #endif
@@ -288,9 +292,12 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
     // side's vertices in shared memory (two hashes of the vertex id): a vertex
     // whose bits are not both set is not in the meeting layer, and its entry is
     // never loaded.  (The first pass has no room for it.)
-    constexpr bool BLOOM = BT != kBiBlock || kBloomWordsFirst > 0;
-    constexpr int NBW = BT == kBiBlock ? kBloomWordsFirst : kBloomWords;  // filter words
-    constexpr int NBB = BT == kBiBlock ? 17 : kHeavyBloomLog;              // filter bits (log2)
+    constexpr bool FIRST = BT != kHeavyBlock;  // (not the heavy pass)
+    constexpr bool BLOOM = !FIRST || kBloomWordsFirst > 0;
+    constexpr int NBW = FIRST ? kBloomWordsFirst : kBloomWords;  // filter words
+    constexpr int NBB = FIRST ? 17 : kHeavyBloomLog;              // filter bits (log2)
+    // frontier vertices per chunk, whose edges are spread over the block
+    constexpr int kFlat = BT == kSmallBlock ? 256 : 512;
     extern __shared__ uint32_t s_bloom[];  // NBW words
     auto bloom_bits = [](int32_t v, uint32_t &h1, uint32_t &h2) {
         const unsigned long long m = (unsigned long long)(uint32_t)v * 0x9E3779B97F4A7C15ull;
@@ -311,7 +318,27 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
     // claims of a level go to counter set it % 3; thread 0 clears set (it + 1) % 3
     // at the start of level it, two barriers after its last readers
     __shared__ int s_new[3], s_meet, s_full;
-    __shared__ u64 s_bkt[kMeetBuckets];
+    // one region for the arrays that are never in use together: a level's chunk, the
+    // meeting step's id buckets, and the lists of the meeting and backtrack steps (13 KB
+    // of shared memory in place of 27).  What the blocks of an SM do not take is the L1
+    // cache, where the adjacency rows and the spilled registers are: at 128 threads, 27 KB
+    // in place of 20 took the estimate of a 300 x 300 grid from 26.4 to 35.4 ms
+    struct Chunk {
+        int64_t fe[kFlat];       // first edge of each frontier vertex of a chunk
+        u64 fs[kFlat];           // its path count
+        int64_t pre[kFlat + 1];  // prefix sums of the chunk's degrees
+    };
+    struct Lists {
+        u64 mw[kMeetCap];
+        int32_t mv[kMeetCap], mp[kMeetCap];
+        int32_t mj[kMeetCap];  // a reverse backtrack candidate's place in the list
+    };
+    union Region {
+        Chunk chunk;
+        Lists lists;
+        u64 bkt[kMeetBuckets];
+    };
+    __shared__ Region s_r;
     __shared__ int s_sel;
     __shared__ u64 s_base;
     __shared__ u64 s_off;               // the sample's path slot in the arena
@@ -330,17 +357,10 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
     __shared__ int s_tstar, s_tlast;      // segment of a long candidate list holding the choice
     __shared__ u64 s_tpre;
     __shared__ int32_t s_lv[2][kLvCap + 2];  // queue range of level L of a side: [s_lv[L], s_lv[L+1])
-    __shared__ int32_t s_mj[kMeetCap];       // a reverse backtrack candidate's place in the list
     __shared__ int s_nc;
     __shared__ unsigned long long s_newcost[3];
-    __shared__ int32_t s_mv[kMeetCap];
-    __shared__ int32_t s_mp[kMeetCap];
-    __shared__ u64 s_mw[kMeetCap];
     __shared__ u64 s_redc[nw];
     __shared__ unsigned long long s_best[nw];
-    __shared__ int64_t s_fe[kFlat];  // first edge of each frontier vertex of a chunk
-    __shared__ u64 s_fs[kFlat];      // its path count
-    __shared__ int64_t s_pre[kFlat + 1];  // prefix sums of the chunk's degrees
     __shared__ unsigned long long s_work[6];
     __shared__ long long s_wsum[nw];    // per-warp degree sums of a chunk
     __shared__ int s_wbits[nw];         // per-warp largest count (bits)
@@ -439,7 +459,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
         bool met = s != t, handed = false;
         // expected hits that try a level for its meeting layer first (lower where the
         // filter makes a scan that finds no member cheap)
-        float meet_hits = BT != kBiBlock ? kMeetOnlyHitsBloom : kMeetOnlyHits;
+        float meet_hits = FIRST ? kMeetOnlyHits : kMeetOnlyHitsBloom;
         // counts of the sides' frontiers are below 2^ub0, 2^ub1; fp: the sample's counts
         // are FP64 values (block-uniform)
         int ub0 = 1, ub1 = 1;
@@ -692,7 +712,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                         }
                     }
                 };
-                constexpr int EB = BT == kBiBlock ? kEdgeBatch : kHeavyEdgeBatch;
+                constexpr int EB = BT == kSmallBlock ? 1 : FIRST ? kEdgeBatch : kHeavyEdgeBatch;
                 // A level likely to meet the other side (the edges it scans times the
                 // vertices the other side holds reach kMeetOnlyHits n) is first scanned for
                 // the meeting layer alone: only vertices the other side holds are claimed,
@@ -743,8 +763,8 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 if (k < fc) {
                                     const int2 qe = qx[c0 + k];
                                     const int64_t e0 = px[qe.x];
-                                    s_fe[k] = e0;
-                                    s_fs[k] = __ldcg(&tab[4ll * qe.y + xs + 1]);
+                                    s_r.chunk.fe[k] = e0;
+                                    s_r.chunk.fs[k] = __ldcg(&tab[4ll * qe.y + xs + 1]);
                                     dg = px[qe.x + 1] - e0;
                                 }
                                 loc[r] = tot;
@@ -763,18 +783,18 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
     #pragma unroll
                             for (int r = 0; r < per; ++r) {
                                 const int k = (int)threadIdx.x * per + r;
-                                if (k < fc) s_pre[k] = first + loc[r];
+                                if (k < fc) s_r.chunk.pre[k] = first + loc[r];
                             }
-                            if (threadIdx.x == BT - 1) s_pre[fc] = first + tot;  // (vertices past fc add 0)
+                            if (threadIdx.x == BT - 1) s_r.chunk.pre[fc] = first + tot;  // (vertices past fc add 0)
                         }
                         __syncthreads();
-                        const int64_t E = s_pre[fc];
+                        const int64_t E = s_r.chunk.pre[fc];
                         if (threadIdx.x == 0) ne += (unsigned long long)E;
-                        auto vertex_of = [&](int64_t j) -> int {  // last k with s_pre[k] <= j
+                        auto vertex_of = [&](int64_t j) -> int {  // last k with s_r.chunk.pre[k] <= j
                             int klo = 0, khi = fc - 1;
                             while (klo < khi) {
                                 const int mid = (klo + khi + 1) >> 1;
-                                if (s_pre[mid] <= j) klo = mid;
+                                if (s_r.chunk.pre[mid] <= j) klo = mid;
                                 else khi = mid - 1;
                             }
                             return klo;
@@ -796,9 +816,9 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                     vv[b] = -1;
                                     kk[b] = k;
                                     if (e < je) {
-                                        while (s_pre[k + 1] <= e) ++k;  // (s_pre[fc] = E > e)
+                                        while (s_r.chunk.pre[k + 1] <= e) ++k;  // (s_r.chunk.pre[fc] = E > e)
                                         kk[b] = k;
-                                        vv[b] = ax[s_fe[k] + (e - s_pre[k])];
+                                        vv[b] = ax[s_r.chunk.fe[k] + (e - s_r.chunk.pre[k])];
                                     }
                                 }
     #pragma unroll
@@ -813,7 +833,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 for (int b = 0; b < kMeetBatch; ++b) {
                                     if (vv[b] < 0) continue;
                                     Pre pr = prefetch(vv[b]);
-                                    resolve(pr, s_fs[kk[b]], true);
+                                    resolve(pr, s_r.chunk.fs[kk[b]], true);
                                 }
                             }
                         } else {
@@ -825,14 +845,14 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 for (int b = 0; b < EB; ++b) {
                                     const int64_t jb = j + (int64_t)b * BT;
                                     kk[b] = jb < E ? vertex_of(jb) : 0;
-                                    vv[b] = jb < E ? ax[s_fe[kk[b]] + (jb - s_pre[kk[b]])] : -1;
+                                    vv[b] = jb < E ? ax[s_r.chunk.fe[kk[b]] + (jb - s_r.chunk.pre[kk[b]])] : -1;
                                 }
     #pragma unroll
                                 for (int b = 0; b < EB; ++b)
                                     if (vv[b] >= 0) pr[b] = prefetch(vv[b]);
     #pragma unroll
                                 for (int b = 0; b < EB; ++b)
-                                    if (vv[b] >= 0) resolve(pr[b], s_fs[kk[b]], meet_only);
+                                    if (vv[b] >= 0) resolve(pr[b], s_r.chunk.fs[kk[b]], meet_only);
                             }
                         }
                         if (c0 + kFlat < hi) __syncthreads();  // the chunk's shared arrays are reused
@@ -927,7 +947,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                 auto weight = [&](const int2 qe) -> C {
                     return side_count(__ldcg(&tab[4ll * qe.y + 1])) * side_count(__ldcg(&tab[4ll * qe.y + 3]));
                 };
-                C *const mw = reinterpret_cast<C *>(s_mw), *const redc = reinterpret_cast<C *>(s_redc);
+                C *const mw = reinterpret_cast<C *>(s_r.lists.mw), *const redc = reinterpret_cast<C *>(s_redc);
                 C part = C(0);
                 for (int m = threadIdx.x; m < nm; m += BT) {
                     const int2 qe = memb[m];
@@ -937,8 +957,8 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     }
                     part += p;
                     if (m < kMeetCap) {
-                        s_mv[m] = qe.x;
-                        s_mp[m] = qe.y;
+                        s_r.lists.mv[m] = qe.x;
+                        s_r.lists.mp[m] = qe.y;
                         mw[m] = p;
                     }
                 }
@@ -958,11 +978,11 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     // own reach the target; the meeting vertex is the smallest such id
                     u64 best = ~0ull;  // vertex << 32 | entry
                     for (int j = threadIdx.x; j < nm; j += BT) {
-                        const int32_t vj = s_mv[j];
+                        const int32_t vj = s_r.lists.mv[j];
                         C pre = C(0);
                         for (int k2 = 0; k2 < nm; ++k2)
-                            if (s_mv[k2] <= vj) pre += mw[k2];
-                        if (pre >= target) best = min(best, ((u64)(uint32_t)vj << 32) | (uint32_t)s_mp[j]);
+                            if (s_r.lists.mv[k2] <= vj) pre += mw[k2];
+                        if (pre >= target) best = min(best, ((u64)(uint32_t)vj << 32) | (uint32_t)s_r.lists.mp[j]);
                     }
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
@@ -973,7 +993,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     if (bk == ~0ull) {  // (FP64 counts) no member reaches the target: the last one takes it
                         u64 lk = 0ull;
                         for (int j = 0; j < nm; ++j)
-                            lk = max(lk, ((u64)(uint32_t)s_mv[j] << 32) | (uint32_t)s_mp[j]);
+                            lk = max(lk, ((u64)(uint32_t)s_r.lists.mv[j] << 32) | (uint32_t)s_r.lists.mp[j]);
                         bk = lk;
                     }
                     vm = (int32_t)(bk >> 32);
@@ -985,7 +1005,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     // bucket whose running total reaches the target holds the answer, and
                     // the next round splits that bucket (exact integer sums, so the same id
                     // as a sequential scan; three rounds for 2^30 ids)
-                    C *const bkt = reinterpret_cast<C *>(s_bkt);
+                    C *const bkt = reinterpret_cast<C *>(s_r.bkt);
                     int64_t lo_id = 0, span = n;
                     C base = C(0);  // weight of the members below lo_id
                     while (span > 1) {
@@ -1214,7 +1234,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                         const uint32_t Lp = lw - 1;
                         const long long lq0 = Lp + 1 <= (uint32_t)kLvCap ? s_lv[z][Lp] : 0;
                         const long long lq1 = Lp + 1 <= (uint32_t)kLvCap ? s_lv[z][Lp + 1] : 0;
-                        C *const mw = reinterpret_cast<C *>(s_mw);
+                        C *const mw = reinterpret_cast<C *>(s_r.lists.mw);
                         if (a.sorted && Lp + 1 <= (uint32_t)kLvCap && lq1 - lq0 <= kMeetCap) {
                             // a long list and a small previous level: the candidates are that
                             // level's vertices found in w's (sorted) list by bisection, their
@@ -1233,20 +1253,20 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                 }
                                 if (blo < e1 && bc[blo] == qe.x) {
                                     const int c = atomicAdd(&s_nc, 1);
-                                    s_mv[c] = qe.x;
-                                    s_mp[c] = qe.y;
+                                    s_r.lists.mv[c] = qe.x;
+                                    s_r.lists.mp[c] = qe.y;
                                     mw[c] = count_of<C>(__ldcg(&tab[4ll * qe.y + zs + 1]));
-                                    s_mj[c] = (int32_t)(blo - e0);
+                                    s_r.lists.mj[c] = (int32_t)(blo - e0);
                                 }
                             }
                             __syncthreads();
                             const int nc = s_nc;
                             u64 best = ~0ull, lastc = 0ull;  // place << 32 | candidate
                             for (int c = threadIdx.x; c < nc; c += BT) {
-                                const int32_t jc = s_mj[c];
+                                const int32_t jc = s_r.lists.mj[c];
                                 C pre = C(0);
                                 for (int c2 = 0; c2 < nc; ++c2)
-                                    if (s_mj[c2] <= jc) pre += mw[c2];
+                                    if (s_r.lists.mj[c2] <= jc) pre += mw[c2];
                                 const u64 key = ((u64)(uint32_t)jc << 32) | (uint32_t)c;
                                 if (mw[c] > C(0)) {
                                     if (pre >= tg) best = min(best, key);
@@ -1274,9 +1294,9 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                                     bk = lk ? lk - 1ull : ~0ull;
                                 }
                                 const int c = bk == ~0ull ? -1 : (int)(uint32_t)bk;
-                                s_pick = c < 0 ? -1 : s_mv[c];
-                                s_pickp = c < 0 ? -1 : s_mp[c];
-                                s_pickc = c < 0 ? 0ull : s_mw[c];
+                                s_pick = c < 0 ? -1 : s_r.lists.mv[c];
+                                s_pickp = c < 0 ? -1 : s_r.lists.mp[c];
+                                s_pickc = c < 0 ? 0ull : s_r.lists.mw[c];
                             }
                         } else {
                             const int64_t seg = (e1 - e0 + BT - 1) / BT;
@@ -1377,7 +1397,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
             tr[1] = globaltimer_ns();
             tr[2] = smp_edges;
             tr[3] = (unsigned long long)smp_levels | ((unsigned long long)(HASH ? 0 : 1) << 32) |
-                    ((unsigned long long)slot << 33) | ((unsigned long long)(BT != kBiBlock) << 63);
+                    ((unsigned long long)slot << 33) | ((unsigned long long)!FIRST << 63);
             tr[4] = t_levels;
             tr[5] = t_meet ? t_meet : t_levels;
         }
@@ -1430,10 +1450,6 @@ __global__ void __launch_bounds__(1024) k_order_heavy(int32_t *defer, const unsi
     for (int j = threadIdx.x; j < nd; j += blockDim.x) defer[j] = (int32_t)(uint32_t)s_k[j];
 }
 
-#ifndef PERCIS_HEAVY_BLOCK
-#define PERCIS_HEAVY_BLOCK 1024
-#endif
-constexpr int kHeavyBlock = PERCIS_HEAVY_BLOCK;  // threads per sample in the heavy pass
 constexpr unsigned long long kDefaultHeavyEdges = 16384;  // a level scanning more edges is heavy
 constexpr int64_t kDefaultScratchGiB = 48;  // direct store: one heavy-pass block per SM up to n = 6M
 
@@ -1441,7 +1457,7 @@ template <bool HASH, int BT>
 int blocks_per_sm(int *cache) {
     if (!*cache) {
         int per_sm = 0;
-        const int dyn = (int)(sizeof(uint32_t) * (BT == kBiBlock ? kBloomWordsFirst : kBloomWords));
+        const int dyn = (int)(sizeof(uint32_t) * (BT != kHeavyBlock ? kBloomWordsFirst : kBloomWords));
         if (dyn > 48 * 1024)
             cudaFuncSetAttribute(k_bibfs<HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bibfs<HASH, BT>, BT, dyn) !=
@@ -1458,7 +1474,7 @@ int blocks_per_sm(int *cache) {
 template <bool HASH, int BT>
 void launch(percis_ctx *ctx, int grid, const BiArgs &a) {
     // the heavy pass's Bloom filter (dynamic shared memory)
-    const int dyn = (int)(sizeof(uint32_t) * (BT == kBiBlock ? kBloomWordsFirst : kBloomWords));
+    const int dyn = (int)(sizeof(uint32_t) * (BT != kHeavyBlock ? kBloomWordsFirst : kBloomWords));
     if (dyn > 48 * 1024) {
         cudaFuncSetAttribute(k_bibfs<HASH, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     }
@@ -1503,7 +1519,9 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
     int64_t nslot = ctx->n;
     if (ctx->multi) multi_graph_view(ctx, &gid, &vbase, &nslot);
     const size_t per_slot = (size_t)nslot * (sizeof(unsigned long long) * 4 + sizeof(int2) * 3);
-    int per_sm = blocks_per_sm<false, BT>(BT == kBiBlock ? &ctx->bi_per_sm : &ctx->bi_heavy_per_sm);
+    int per_sm = blocks_per_sm<false, BT>(BT == kHeavyBlock   ? &ctx->bi_heavy_per_sm
+                                          : BT == kSmallBlock ? &ctx->bi_small_per_sm
+                                                              : &ctx->bi_per_sm);
     if (BT == kBiBlock && ctx->opt.bi_blocks_per_sm > 0) per_sm = std::min(per_sm, ctx->opt.bi_blocks_per_sm);
     const int64_t budget = (int64_t)(ctx->opt.bi_scratch_gib > 0 ? ctx->opt.bi_scratch_gib : kDefaultScratchGiB) << 30;
     int64_t slots = std::min<int64_t>((int64_t)per_sm * ctx->num_sms, std::max<int64_t>(1, budget / (int64_t)per_slot));
@@ -1535,22 +1553,38 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
     a.queue = ctx->bi_queue.as<int2>();
     a.region = nslot;
     a.qcap = nslot;
-    a.next = ctx->arena_top.as<unsigned long long>() + (BT == kBiBlock ? 1 : 2);
+    a.next = ctx->arena_top.as<unsigned long long>() + (BT != kHeavyBlock ? 1 : 2);
     a.heavy_edges = heavy_edges;
     a.heavy_auto = heavy_auto;
     a.deferred = defer;
     a.defer_cost = defer_cost;
     a.n_deferred = n_def;
     launch<false, BT>(ctx, (int)slots, a);
-    PERCIS_CHECK_LAUNCH(ctx, BT == kBiBlock ? "bidirectional sigma-BFS (direct)" : "bidirectional sigma-BFS (heavy)");
+    PERCIS_CHECK_LAUNCH(ctx, BT != kHeavyBlock ? "bidirectional sigma-BFS (direct)" : "bidirectional sigma-BFS (heavy)");
     return PERCIS_OK;
+}
+
+// Small graphs: 128 threads a sample and twice the samples in flight.  A level's edges there
+// rarely fill 256 threads, and its time is the chain of its loads and barriers.  Estimates
+// (ms, 256 / 128 threads): Barabasi-Albert (m = 4) n = 3k 1.72 / 1.21, 30k 2.54 / 1.81, 100k
+// 3.33 / 2.68, 300k 4.60 / 4.21; grids n = 5k 3.98 / 3.27, 20k 8.6 / 8.0, 40k 13.5 / 13.2, 90k
+// 23.6 / 25.6; Watts-Strogatz (10) n = 3k 0.74 / 0.70, 10k 0.85 / 0.84, 40k 1.05 / 1.17, 150k
+// 1.79 / 1.99; R-MAT n = 20k 0.71 / 0.65, 200k 1.26 / 1.51.  So: up to 2^15 vertices (beyond,
+// the gain is Barabasi-Albert's alone, and clearing twice the slots' entries, 7.8 GB at
+// 200k, would cost a context's first phase more than later ones win).  Phases of fewer
+// samples than 256-thread blocks fit the chip keep those, as does a set number of blocks
+// per SM.
+bool small_graph(percis_ctx *ctx, int64_t nslot, int64_t count, bool heavy_on) {
+    if (heavy_on || ctx->opt.bi_blocks_per_sm > 0) return false;
+    if (count <= (int64_t)blocks_per_sm<false, kBiBlock>(&ctx->bi_per_sm) * ctx->num_sms) return false;
+    return nslot <= (1 << 15);
 }
 
 }  // namespace
 
 // All samples of a phase (pairs, kinds already drawn): kinds of unreachable
 // targets, |I|, paths and counts, as the batched form leaves them.  Every
-// sample runs first with 256 threads (the direct store, or hashed tables);
+// sample runs first with 256 or 128 threads (the direct store, or hashed tables);
 // samples with a heavy level, or that outgrow their table, are handed over
 // untouched and run afterwards with 1,024 threads in the direct store.
 percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int64_t count) {
@@ -1600,7 +1634,10 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
         const int64_t full = (int64_t)blocks_per_sm<false, kBiBlock>(&ctx->bi_per_sm) * ctx->num_sms;
         direct = full * per_slot <= budget;
     }
-    if (direct) {
+    if (direct && small_graph(ctx, nslot, count, heavy_on)) {
+        PERCIS_TRY(
+            direct_pass<kSmallBlock>(ctx, seed, tag_path, count, nullptr, heavy, heavy_auto, defer, defer_cost, n_def));
+    } else if (direct) {
         PERCIS_TRY(
             direct_pass<kBiBlock>(ctx, seed, tag_path, count, nullptr, heavy, heavy_auto, defer, defer_cost, n_def));
     } else {

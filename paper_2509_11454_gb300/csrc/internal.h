@@ -94,6 +94,7 @@ struct percis_ctx {
     percis::DevBuf stamp, plain_hub, sigma1, qa, qb, plain_ctl;
     int32_t epoch = 0;
     int plain_grid = 0;  // cooperative grid of the plain BFS on this device (0 = not yet queried)
+    int bi_small_per_sm = 0;
     int bi_per_sm = 0;   // resident blocks per SM of the bidirectional kernel (0 = not yet queried)
 
     // batched BFS state

@@ -227,10 +227,10 @@ def test_batches_side_by_side(binding, count, estimator):
 
 
 def test_many_graphs_sampling_and_backward_in_one_launch(binding):
-    """Path graphs whose samples have up to 1, 7, 8, 9, 16, 17 and 38 internal vertices
+    """Path graphs whose samples have up to 2, 7, 8, 9, 16, 17 and 38 internal vertices
     (eight lanes share a sample): pairs, counts and gradients of each graph in the batch
     are the oracle's."""
-    sizes = [3, 9, 10, 11, 18, 19, 40]
+    sizes = [4, 9, 10, 11, 18, 19, 40]
     graphs = [synth.csr_from_edges(n, np.arange(n - 1), np.arange(1, n), directed=False) for n in sizes]
     vptr, rp, col = synth.union_csr(graphs)
     x = synth.states_uniform(int(vptr[-1]), 3)
@@ -250,4 +250,27 @@ def test_many_graphs_sampling_and_backward_in_one_launch(binding):
         assert np.max(np.abs(pc[lo:hi] - F)) <= 1e-9, g
         ref = oracle.vjp_fixed(prep, fixed, ph, F, gvec[lo:hi])
         assert np.linalg.norm(gx[lo:hi] - ref) <= 1e-10 * np.linalg.norm(ref), g
+    eng.close()
+
+
+@pytest.mark.parametrize("n", [300, 32768, 32769])
+@pytest.mark.parametrize("count", [607, 609, 1300])
+def test_bidir_small_graph_blocks(binding, n, count):
+    """Samples by 128 threads (graphs of up to 2^15 vertices, more samples than 256-thread
+    blocks fit the chip) and by 256: frontiers and meeting layers around a chunk of 256
+    vertices (a hub over the whole graph), the oracle's paths."""
+    rng = np.random.default_rng(n)
+    hub = np.arange(1, min(n, 700))
+    src = np.concatenate([np.zeros(len(hub), dtype=np.int64), rng.integers(0, n, 3 * n)])
+    dst = np.concatenate([hub, rng.integers(0, n, 3 * n)])
+    g = synth.csr_from_edges(n, src, dst, directed=False)
+    x = synth.states_uniform(n, 4)
+    eng = _engine(binding, g, x, form="bidir")
+    ph = eng.run_phase(6, 1, count)
+    ptr, nodes = (_np(v) for v in eng.get_paths(count))
+    ref = oracle.run_samples(oracle.from_synth(g), oracle.prepare(x), 6, 1, 3, 0, count, keep_paths=True, bidir=True)
+    assert not ref.overflow
+    for k in ("s", "t", "kind", "ilen", "cnt"):
+        assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
+    assert np.array_equal(nodes, ref.path_nodes)
     eng.close()
