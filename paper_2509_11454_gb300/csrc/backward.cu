@@ -31,15 +31,17 @@ __global__ void k_bw_samples(int64_t count, const int32_t *s, const int32_t *t, 
         if (kind[i] != 0) continue;  // (the same for the eight lanes)
         const int32_t si = s[i], ti = t[i], len = ilen[i];
         const long long off = path_off[i];
-        double S = 0.0;
-        for (int q = sub; q < len; q += 8) {
-            const int32_t v = arena[off + q];
-            S += g[v] / Cv[v];
-        }
         const unsigned m = 0xffu << (threadIdx.x & 24);
-        S += __shfl_xor_sync(m, S, 1);
-        S += __shfl_xor_sync(m, S, 2);
-        S += __shfl_xor_sync(m, S, 4);
+        double S = 0.0;
+        for (int q = 0; q < len; q += 8) {
+            double term = 0.0;
+            if (q + sub < len) {
+                const int32_t v = arena[off + q + sub];
+                term = g[v] / Cv[v];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) S += __shfl_sync(m, term, k, 8);  // in the path's order
+        }
         if (sub < 2) {
             const int32_t gr = gid ? gid[si] : 0;
             const double coef = (C[gr] / (ells ? ells[gr] : ell)) * S / (x[si] - x[ti]);
