@@ -1524,14 +1524,17 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
                                                               : &ctx->bi_per_sm);
     if (BT == kBiBlock && ctx->opt.bi_blocks_per_sm > 0) per_sm = std::min(per_sm, ctx->opt.bi_blocks_per_sm);
     const int64_t budget = (int64_t)(ctx->opt.bi_scratch_gib > 0 ? ctx->opt.bi_scratch_gib : kDefaultScratchGiB) << 30;
-    int64_t slots = std::min<int64_t>((int64_t)per_sm * ctx->num_sms, std::max<int64_t>(1, budget / (int64_t)per_slot));
-    slots = std::min<int64_t>(slots, std::max<int64_t>(count, 1));  // (count: at most that many with count_dev)
+    const int64_t full =
+        std::min<int64_t>((int64_t)per_sm * ctx->num_sms, std::max<int64_t>(1, budget / (int64_t)per_slot));
+    const int64_t slots = std::min<int64_t>(full, std::max<int64_t>(count, 1));  // (count: at most, with count_dev)
     if (ctx->bi_slots < slots || ctx->bi_n != nslot) {
-        PERCIS_TRY(ensure(ctx, ctx->bi_info, sizeof(unsigned long long) * 4 * nslot * slots, "bidirectional records"));
-        PERCIS_TRY(ensure(ctx, ctx->bi_queue, sizeof(int2) * 3 * nslot * slots, "bidirectional queues"));
+        // (phase 1 has 1,000 samples or more: all slots now, not 1,000 and then again for phase 2)
+        const int64_t have = 2 * slots >= full ? full : slots;
+        PERCIS_TRY(ensure(ctx, ctx->bi_info, sizeof(unsigned long long) * 4 * nslot * have, "bidirectional records"));
+        PERCIS_TRY(ensure(ctx, ctx->bi_queue, sizeof(int2) * 3 * nslot * have, "bidirectional queues"));
         // level words of no sample (epoch 0)
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->bi_info.p, 0, sizeof(unsigned long long) * 4 * nslot * slots, ctx->stream));
-        ctx->bi_slots = slots;
+        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->bi_info.p, 0, sizeof(unsigned long long) * 4 * nslot * have, ctx->stream));
+        ctx->bi_slots = have;
         ctx->bi_n = nslot;
         ctx->bi_epoch = 0;
     }
