@@ -161,7 +161,8 @@ struct BiArgs {
     int32_t *deferred;           // samples handed to the heavy pass
     unsigned long long *defer_cost;  // edges of the level each was handed over at
     unsigned int *n_deferred;
-    int32_t sorted;              // every adjacency list strictly increasing (reverse backtrack allowed)
+    int32_t sorted;              // every adjacency list strictly increasing: no parallel edges, and a
+                                 // reverse backtrack allowed
     unsigned long long heavy_edges;  // a level scanning more edges than this hands the sample over (0: never)
     const unsigned long long *max_degree;  // largest out- or in-degree of the graph (device word)
     int32_t heavy_auto;          // heavy_edges applies only where max_degree >= kHubDegree
@@ -548,7 +549,10 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                         tab = ntab;
                     }
                 }
-                // A new count is at most the sum of the frontier's counts, below 2^nb.
+                // A new count is a sum over the edges into one vertex from the frontier, below
+                // 2^nb: at most one edge from each frontier vertex where no row holds a column
+                // twice (strictly increasing rows), else (parallel edges count one by one) at
+                // most the level's edges, and at most the largest degree.
                 // Where that could pass 2^52 the frontier's largest count is looked up, and
                 // if it still could, the sample's counts become FP64 values here, before the
                 // level: integer counts never reach 2^53, so they need no check per addition
@@ -556,7 +560,9 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                 // pipe 57% busy on Barabasi-Albert 30k), and a phase whose counts pass it is
                 // not run a second time in FP64 (estimate on a 300 x 300 grid 55.7 -> 28.5 ms,
                 // on Barabasi-Albert 200k with new states 3.90 -> 3.67 ms).
-                int nb = (x ? ub1 : ub0) + ceil_log2(hi - lo);
+                long long into = hi - lo;
+                if (!a.sorted) into = (long long)min(x ? cost[1] : cost[0], __ldg(a.max_degree));
+                int nb = (x ? ub1 : ub0) + ceil_log2(into);
                 if (!fp && nb > 52) {
                     const int2 *qf = x ? queue1 : queue0;
                     const int fs = x ? 3 : 1;
@@ -567,7 +573,7 @@ __global__ void __launch_bounds__(BT, BT == kBiBlock ? PERCIS_BI_MINB : 1024 / B
                     if (lane == 0) s_wbits[warp] = mb;
                     __syncthreads();
                     for (int q = 0; q < nw; ++q) mb = max(mb, s_wbits[q]);
-                    nb = mb + ceil_log2(hi - lo);
+                    nb += mb - (x ? ub1 : ub0);
                     if (nb > 52) {
                         fp = true;
                         for (int z = 0; z < 2; ++z) {

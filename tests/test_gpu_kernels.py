@@ -274,3 +274,45 @@ def test_bidir_small_graph_blocks(binding, n, count):
         assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
     assert np.array_equal(nodes, ref.path_nodes)
     eng.close()
+
+
+def _csr_with_copies(n, src, dst, copies, directed, rng=None):
+    """CSR that keeps every edge as often as it is given (rng: rows in random order)."""
+    src, dst = np.repeat(src, copies), np.repeat(dst, copies)
+    if not directed:
+        src, dst = np.concatenate([src, dst]), np.concatenate([dst, src])
+    order = np.lexsort((dst if rng is None else rng.random(len(dst)), src))
+    row_ptr = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))]).astype(np.int64)
+    return synth.Graph(n=n, row_ptr=row_ptr, col=dst[order].astype(np.int32), directed=directed, name="copies")
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("table_log", [0, 10])
+@pytest.mark.parametrize("kind", ["path2", "path3", "diamonds", "simple"])
+def test_bidir_parallel_edges(binding, kind, table_log, shuffled, directed):
+    """Rows that hold a column several times count one path per copy: counts far past 2^53
+    (2^199, 3^199, 3^60) on frontiers of one or two vertices.  Every sum has two terms, or
+    equal ones, so FP64 counts round alike in any order: pairs, lengths, counts and paths
+    are the oracle's exactly, and the flag is raised where the oracle raises it."""
+    if kind == "diamonds":  # v -> a, v -> b twice, a -> v', b -> v'
+        k = 60
+        n, v = 3 * k + 1, 3 * np.arange(k)
+        src, dst = np.concatenate([v, v, v + 1, v + 2]), np.concatenate([v + 1, v + 2, v + 3, v + 3])
+        copies = np.concatenate([np.ones(k, int), np.full(k, 2), np.ones(2 * k, int)])
+    else:
+        n = 200
+        src, dst = np.arange(n - 1), np.arange(1, n)
+        copies = np.full(n - 1, {"path2": 2, "path3": 3, "simple": 1}[kind])
+    g = _csr_with_copies(n, src, dst, copies, directed, np.random.default_rng(1) if shuffled else None)
+    x = np.linspace(1.0, 0.0, n)
+    eng = _engine(binding, g, x, form="bidir", bi_table_log=table_log, ell1=240, ell=240)
+    ph = eng.run_phase(3, 1, 240)
+    ptr, nodes = (_np(a) for a in eng.get_paths(240))
+    ref = oracle.run_samples(oracle.from_synth(g), oracle.prepare(x), 3, 1, 3, 0, 240, keep_paths=True, bidir=True)
+    for key in ("s", "t", "kind", "ilen", "cnt"):
+        assert np.array_equal(_np(ph[key]), getattr(ref, key)), key
+    assert np.array_equal(nodes, ref.path_nodes)
+    assert ref.overflow == (kind != "simple")
+    assert eng.estimate(0.05, 0.1, 3)[1]["sigma_overflow"] == int(ref.overflow)
+    eng.close()
