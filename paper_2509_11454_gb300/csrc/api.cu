@@ -438,6 +438,7 @@ percis_status percis_set_stream(percis_ctx *ctx, void *stream) {
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     ctx->own_stream = false;
     ctx->stream = (cudaStream_t)stream;
+    multi_set_stream(ctx);
     return PERCIS_OK;
 }
 

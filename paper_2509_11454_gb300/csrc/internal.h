@@ -290,6 +290,7 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
 // multi.cu
 void multi_free(percis_ctx *ctx);
 void multi_set_options(percis_ctx *ctx);  // the graphs' contexts follow the union's options
+void multi_set_stream(percis_ctx *ctx);   // and its stream: calls on the union order theirs
 percis_status percis_multi_set_states(percis_ctx *ctx, const double *x, int on_device);
 percis_status percis_multi_backward(percis_ctx *ctx, const double *grad_pc, double *grad_x, int on_device);
 // pairs of a phase of a many-graph context: graph g draws its counts[g]

@@ -135,6 +135,11 @@ void multi_set_options(percis_ctx *ctx) {
     for (percis_ctx *sub : ctx->multi->subs) sub->opt = ctx->opt;
 }
 
+void multi_set_stream(percis_ctx *ctx) {
+    if (!ctx->multi) return;
+    for (percis_ctx *sub : ctx->multi->subs) sub->stream = ctx->stream;  // (theirs was the union's, never their own)
+}
+
 percis_status multi_sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag) {
     MultiGraph *m = ctx->multi;
     auto issue = [&](const uint64_t *seed_dev) {

@@ -198,3 +198,67 @@ def test_cuda_graph_sampling_matches_eager(binding, batch):
         assert [f["ell"] for f in ia] == [f["ell"] for f in ib]
     eager.close()
     rec.close()
+
+
+@pytest.mark.parametrize("own", [False, True])
+@pytest.mark.parametrize("form", ["batched", "bidir"])
+def test_stream_switch(binding, form, own):
+    """percis_set_stream after the graphs are loaded (on a caller's stream, or on the
+    context's own, which ends with the switch) and again between states, estimate and
+    backward: the graphs' contexts follow, so nothing is left on a former stream.  The
+    former streams are kept busy for about 50 ms meanwhile.  Estimates are those without
+    a switch, and so are gradients to the rounding of their sums."""
+    graphs = synth.graph_batch([60, 90, 40], 3)
+    vptr, rp, col = synth.union_csr(graphs)
+    n = int(vptr[-1])
+    x, x2 = synth.states_uniform(n, 1), synth.states_uniform(n, 2)
+    gvec = torch.as_tensor(np.random.default_rng(3).standard_normal(n), device="cuda")
+    busy = 100_000_000  # cycles
+
+    def run(streams):
+        with torch.cuda.stream(streams[0]):
+            eng = binding.PercIS(0)
+        if own:
+            binding.percis_destroy(eng.ctx)
+            eng.ctx = binding.percis_create(0, None)
+        eng.set_options(form=form, ell1=100, ell=400)
+        eng.load_graphs(vptr, rp, col)
+        out = []
+        for k, states in enumerate((x, x2)):
+            def switch(s):
+                if len(set(streams)) > 1:
+                    binding.percis_set_stream(eng.ctx, s.cuda_stream)
+                    with torch.cuda.stream(streams[0] if s is streams[1] else streams[1]):
+                        torch.cuda._sleep(busy)
+
+            switch(streams[1])
+            eng.set_states(states)
+            out.append(eng.estimate_graphs(0.05, 0.1, seed=5)[0].cpu().numpy())
+            lam = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            switch(streams[1])
+            binding.percis_get_prep(eng.ctx, lam=lam)
+            with torch.cuda.stream(streams[1]):
+                out.append(lam.cpu().numpy())
+            grad = torch.full((n,), 7.0, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            switch(streams[1])
+            binding.percis_backward(eng.ctx, gvec, grad)
+            with torch.cuda.stream(streams[1]):
+                out.append(grad.cpu().numpy())
+            switch(streams[0])
+        torch.cuda.synchronize()
+        eng.close()
+        return out
+
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    plain, switched = run((a, a)), run((a, b))
+    for k, (p, q) in enumerate(zip(plain, switched)):
+        if k % 3 < 2:
+            assert np.array_equal(p, q), k
+        else:
+            assert np.linalg.norm(p - q) <= 1e-10 * np.linalg.norm(p), k
+    for g in range(3):
+        lo, hi = vptr[g], vptr[g + 1]
+        lam = oracle.prepare(x[lo:hi], cv_method="sorted").lam
+        assert np.max(np.abs(switched[1][lo:hi] - lam) / lam) <= 1e-12
