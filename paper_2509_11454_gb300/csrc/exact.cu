@@ -26,8 +26,32 @@ namespace {
 // edges a whole block shares an item (a hub's 8 words one after the other on one warp,
 // edge by edge, set the time of every launch).  Barabasi-Albert n = 3001, m = 4:
 // 93.6 -> 1.9 ms in all launches, error against 64 bits 2.8e-16 -> 1.4e-16 relative.
+// R(x_s - x_w) is 0 or at least 2^-53 x_s, so y is at least 2^-53 x_s / sigma.  Where that
+// could be subnormal (FP64 counts, or states below kTinyState; unscaled, states of 1e-300
+// lost digits from counts of 2^27 on and gave 0 from 2^78) a source's y is carried times
+// the power of two that takes x_s to [2^60, 2^61), which every term of num takes out
+// again, both exactly.
+constexpr unsigned long long kTinyState = 123ull << 52;  // 2^-900, as bits
 constexpr int kDepBlock = 256;
 constexpr int64_t kDepBlockDeg = 128;
+
+// 2^k, |k| < 1023
+__device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
+
+// v 2^k, |k| < 2000
+__device__ __forceinline__ double scaled(double v, int k) {
+    const int lo = max(-1000, min(1000, k));
+    const double r = v * pow2(lo);
+    return k == lo ? r : r * pow2(k - lo);  // (a second factor for states below 2^-940 alone)
+}
+
+// the exponent of source state x's scale
+template <int SM>
+__device__ __forceinline__ int state_scale(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if (SM < 2 && b - 1ull >= kTinyState) return 0;  // (x = 0 has no ramp: no scale)
+    return 60 - (b >> 52 ? (int)(b >> 52) - 1023 : -1011 - __clzll((long long)b));
+}
 
 template <int K, int SM>
 __global__ void __launch_bounds__(kDepBlock) k_dependency(int64_t n, const int64_t *rp, const int32_t *col,
@@ -79,18 +103,34 @@ __global__ void __launch_bounds__(kDepBlock) k_dependency(int64_t n, const int64
             }
         }
     };
-    // the item's results from its sums: y of its sources and its share of num
+    // the item's results from its sums: y of its sources and its share of num (every lane
+    // of the warp calls it)
     auto finish = [&](int64_t v, int w, uint64_t bits, double a0, double a1) {
         double vsum = 0.0;
         const double xv = x[v];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = 64 * w + 32 * h + lane;
-            if (!((bits >> (lane + 32 * h)) & 1ull) || j >= nlanes) continue;
+        const int j0 = 64 * w + lane;
+        const double xs[2] = {j0 < nlanes ? x[src0 + j0] : 0.0, j0 + 32 < nlanes ? x[src0 + j0 + 32] : 0.0};
+        auto half = [&](int h, int k, auto rescale) {
+            const int j = j0 + 32 * h;
+            if (!((bits >> (lane + 32 * h)) & 1ull) || j >= nlanes) return;
             const double a = h ? a1 : a0, sv = (double)sigma[v * W + j];
-            const double ramp = x[src0 + j] - xv;
-            y[v * W + j] = ramp > 0.0 ? a + ramp / sv : a;
-            vsum += sv * a;
+            const double ramp = xs[h] - xv;
+            if constexpr (rescale) {
+                y[v * W + j] = ramp > 0.0 ? a + scaled(ramp, k) / sv : a;
+                vsum += scaled(sv * a, -k);
+            } else {
+                y[v * W + j] = ramp > 0.0 ? a + ramp / sv : a;
+                vsum += sv * a;
+            }
+        };
+        // (apart, so that ordinary states' two divisions stay side by side)
+        const int k0 = state_scale<SM>(xs[0]), k1 = state_scale<SM>(xs[1]);
+        if (__any_sync(0xffffffffu, (k0 | k1) != 0)) {
+            half(0, k0, std::true_type{});
+            half(1, k1, std::true_type{});
+        } else {
+            half(0, 0, std::false_type{});
+            half(1, 0, std::false_type{});
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) vsum += __shfl_xor_sync(0xffffffffu, vsum, off);

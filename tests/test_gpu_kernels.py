@@ -316,3 +316,31 @@ def test_bidir_parallel_edges(binding, kind, table_log, shuffled, directed):
     assert ref.overflow == (kind != "simple")
     assert eng.estimate(0.05, 0.1, 3)[1]["sigma_overflow"] == int(ref.overflow)
     eng.close()
+
+
+@pytest.mark.parametrize("layers", [[10], [18], [28], [500], [24, 40]])
+@pytest.mark.parametrize("scale", [1.0, 1e-300])
+def test_exact_centrality_scale_and_counts(binding, layers, scale):
+    """Exact centrality where counts are stored in 32 and 64 bits and as FP64 (4^9, 4^17,
+    4^27, 4^499 paths over layers of four vertices) and with states of any scale, one
+    component's a thousand orders of two below the other's: each value relative to itself.
+    A dependency is a sum of non-negative terms over at most `layers` levels, four edges
+    and a few roundings each, and a value sums n of them: 2 (8 layers + n) 2^-53."""
+    src, dst, xs, lo = [], [], [], 0
+    rng = np.random.default_rng(len(layers) + layers[0])
+    for c, depth in enumerate(layers):
+        at = lo + 4 * np.arange(depth - 1)
+        for a in range(4):
+            for b in range(4):
+                src.append(at + a)
+                dst.append(at + 4 + b)
+        xs.append(rng.random(4 * depth) * 2.0 ** (-990 * c))
+        lo += 4 * depth
+    x = np.concatenate(xs) * (scale if len(layers) == 1 else 1.0)
+    g = synth.csr_from_edges(lo, np.concatenate(src), np.concatenate(dst), directed=False)
+    eng = _engine(binding, g, x)
+    ref = oracle.exact_pc(oracle.from_synth(g), x, oracle.prepare(x, cv_method="sorted").Cv)
+    got = _np(eng.exact())
+    assert np.all(np.abs(got - ref) <= 2 * (8 * max(layers) + lo) * 2.0 ** -53 * ref)
+    assert np.count_nonzero(got) > lo // 2
+    eng.close()
