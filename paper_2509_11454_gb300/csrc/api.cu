@@ -39,6 +39,10 @@ percis_status ensure(percis_ctx *ctx, DevBuf &b, size_t bytes, const char *what)
     }
     const size_t want = bytes + bytes / 16;
     cudaError_t e = cudaMalloc(&b.p, want);
+    if (e == cudaErrorMemoryAllocation && !ctx->ms_live && ms_give_back(ctx)) {
+        cudaGetLastError();
+        e = cudaMalloc(&b.p, want);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         b.p = nullptr;
@@ -297,7 +301,11 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
             int64_t U = 0, valid = 0;
             PERCIS_TRY(group_by_source(ctx, count, &U, &valid));
             *sources = U;
-            if (U > 0) PERCIS_TRY(batched_phase(ctx, seed, (uint32_t)(2 + phase), count, U, batches));
+            percis_status bs = PERCIS_OK;
+            do {  // (with fewer batches side by side where the memory for them cannot be had)
+                if (U > 0) bs = batched_phase(ctx, seed, (uint32_t)(2 + phase), count, U, batches);
+            } while (bs == PERCIS_E_OOM && ms_give_back(ctx));
+            PERCIS_TRY(bs);
         }
         if (po->want_stats) PERCIS_TRY(issue_phase_stats(ctx, count, po->stats_pmax));
         const uint32_t st = read_status(ctx, plain);
@@ -472,6 +480,7 @@ percis_status percis_load_csr(percis_ctx *ctx, int64_t n, int64_t nnz, const int
         return set_err(ctx, PERCIS_E_INVALID, "need n >= 2 (int32 ids) and valid pointers");
     DeviceGuard g(ctx->device);
     multi_free(ctx);
+    ctx->ms_max_groups = 0;
     ctx->have_graph = false;
     ctx->have_states = false;
     ctx->have_paths = false;

@@ -104,6 +104,9 @@ struct percis_ctx {
     int sigma_mode = 0;  // batched sigma storage: 0 = 32-bit, 1 = 64-bit integers, 2 = FP64
     percis::DevBuf fq0, fq1;  // frontier queues
     percis::DevBuf ms_need, ms_list, ms_levels;  // needed lanes of every vertex, their lists, counts per level
+    int ms_groups = 0;      // batches side by side the buffers above were last sized for (the most since given back)
+    int ms_max_groups = 0;  // and may be, since memory ran out on this graph (0: no limit)
+    bool ms_live = false;   // a batched launch is being set up: its buffers are not to be given back
     percis::DevBuf acc_ap, ap_tau, ap_stamp, ap_list;  // all-paths estimator
     percis::DevBuf plan_dev;                           // lane batches of a many-graph phase
     percis::DevBuf bi_info, bi_queue;                  // bidirectional form, direct store: per-slot scratch
@@ -256,6 +259,9 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
 // msbfs.cu
 percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int64_t count, int64_t n_sources,
                             int64_t *batches);
+// frees the batched form's buffers where they hold more than one batch, and halves the
+// batches that may run side by side from now on; false if there is nothing to free
+bool ms_give_back(percis_ctx *ctx);
 percis_status msbfs_full(percis_ctx *ctx, int32_t nsrc, const int32_t *sources, int32_t *dist, double *sigma);
 int choose_lanes(percis_ctx *ctx, int64_t n_sources);
 

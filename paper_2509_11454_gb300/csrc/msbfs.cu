@@ -1271,6 +1271,7 @@ MsSizes ms_sizes(int W, int Lcap, int64_t n) {
 
 percis_status ensure_ms(percis_ctx *ctx, int W, int Lcap, int64_t nr, bool full, int groups) {
     const MsSizes z = ms_sizes(W, Lcap, nr);  // nr: vertices of the largest launch range
+    ctx->ms_groups = std::max(ctx->ms_groups, groups);
     PERCIS_TRY(ensure(ctx, ctx->fq0, z.queue * groups, "frontier queue"));
     PERCIS_TRY(ensure(ctx, ctx->fq1, z.queue * groups, "frontier queue"));
     PERCIS_TRY(ensure(ctx, ctx->vis, z.vis * groups, "visited bits"));
@@ -1313,6 +1314,14 @@ MsArgs group_args(const MsArgs &a0, const MsSizes &z, int g, int64_t ap_n) {
     return a;
 }
 
+struct MsLive {
+    percis_ctx *ctx;
+    explicit MsLive(percis_ctx *c) : ctx(c) { ctx->ms_live = true; }
+    ~MsLive() { ctx->ms_live = false; }
+    MsLive(const MsLive &) = delete;
+    MsLive &operator=(const MsLive &) = delete;
+};
+
 void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
     a.n = ctx->n;
     a.big_count = ctx->ms_big.as<int32_t>();
@@ -1343,6 +1352,22 @@ void fill_common(percis_ctx *ctx, MsArgs &a, int Lcap, int K, int64_t nr) {
 }
 
 }  // namespace
+
+// More batches side by side are an option of speed alone: where an allocation fails, the
+// memory they hold goes first (one batch at a time took a quarter of it, and a call that
+// fits with that still runs).
+bool ms_give_back(percis_ctx *ctx) {
+    if (ctx->ms_groups <= 1) return false;
+    cudaStreamSynchronize(ctx->stream);
+    for (DevBuf *b : {&ctx->fq0, &ctx->fq1, &ctx->vis, &ctx->fhist, &ctx->sigmaW, &ctx->ms_need, &ctx->ms_list,
+                      &ctx->ms_levels}) {
+        if (b->p) cudaFree(b->p);
+        *b = DevBuf{};
+    }
+    ctx->ms_max_groups = ctx->ms_groups / 2;
+    ctx->ms_groups = 0;
+    return true;
+}
 
 int choose_lanes(percis_ctx *ctx, int64_t n_sources) {
     int W = ctx->opt.lanes;
@@ -1387,8 +1412,10 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
     if (!ctx->opt.instrument) {
         const MsSizes z = ms_sizes(W, Lcap, nr_max);
         const size_t each = 2 * z.queue + 2 * z.vis + z.hist + z.sigma + z.list + z.levels;
-        while (G < kMaxGroups && G + 1 <= B && (size_t)(G + 1) * each <= (24ull << 30)) ++G;
+        const int most = ctx->ms_max_groups ? std::min(kMaxGroups, ctx->ms_max_groups) : kMaxGroups;
+        while (G < most && G + 1 <= B && (size_t)(G + 1) * each <= (24ull << 30)) ++G;
     }
+    MsLive live(ctx);
     PERCIS_TRY(prep_ms_graph(ctx, false));
     PERCIS_TRY(ensure_ms(ctx, W, Lcap, nr_max, false, G));
     ctx->levels_alloc = Lcap;
@@ -1430,6 +1457,7 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
         const int64_t ap_group = std::max<int64_t>(1, std::min<int64_t>(warps, (8ll << 30) / per_warp) / G);
         const int64_t ap_warps = ap_group * G;
         if (ctx->ap_warps != ap_warps || ctx->ap_n != n) {
+            ctx->ap_warps = 0;  // (an allocation may fail)
             PERCIS_TRY(ensure(ctx, ctx->ap_tau, sizeof(unsigned long long) * n * ap_warps, "all-paths tau"));
             PERCIS_TRY(ensure(ctx, ctx->ap_stamp, sizeof(int32_t) * n * ap_warps, "all-paths stamps"));
             PERCIS_TRY(ensure(ctx, ctx->ap_list, sizeof(int32_t) * 2 * n * ap_warps, "all-paths lists"));
@@ -1483,8 +1511,11 @@ percis_status msbfs_full(percis_ctx *ctx, int32_t nsrc, const int32_t *sources, 
     const int K = W / 64;
     int Lcap = std::max(ctx->levels_alloc, 32);
     for (int attempt = 0; attempt < 12; ++attempt) {
+        MsLive live(ctx);
         PERCIS_TRY(prep_ms_graph(ctx, true));
-        PERCIS_TRY(ensure_ms(ctx, W, Lcap, ctx->n, true, 1));
+        percis_status es = ensure_ms(ctx, W, Lcap, ctx->n, true, 1);
+        if (es == PERCIS_E_OOM && ms_give_back(ctx)) es = ensure_ms(ctx, W, Lcap, ctx->n, true, 1);
+        PERCIS_TRY(es);
         ctx->levels_alloc = Lcap;
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->ms_ctl.p, 0, sizeof(MsCtl), ctx->stream));
         MsArgs a{};

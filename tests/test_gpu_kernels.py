@@ -344,3 +344,52 @@ def test_exact_centrality_scale_and_counts(binding, layers, scale):
     assert np.all(np.abs(got - ref) <= 2 * (8 * max(layers) + lo) * 2.0 ** -53 * ref)
     assert np.count_nonzero(got) > lo // 2
     eng.close()
+
+
+def _fill(leave):
+    """A block of device memory that leaves about `leave` bytes free."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+def test_batches_side_by_side_in_little_memory(binding):
+    """Batches side by side are given up where their memory cannot be had: in a phase that
+    fits one batch's state and not two (1.8 GB each), and for a later call that needs what
+    they hold.  Counts, paths and distances are those with the memory free."""
+    n, count = 1 << 18, 4000
+    rng = np.random.default_rng(1)
+    src = np.concatenate([np.arange(n), rng.integers(0, n, 2 * n)])
+    dst = np.concatenate([(np.arange(n) + 1) % n, rng.integers(0, n, 2 * n)])
+    g = synth.csr_from_edges(n, src, dst, directed=False)
+    x = synth.states_uniform(n, 1)
+    m = 4 * n
+    rp2, col2 = np.arange(m + 1, dtype=np.int64) * 4, rng.integers(0, m, 4 * m).astype(np.int32)
+
+    def phase(eng):
+        ph = eng.run_phase(7, 1, count)
+        return [_np(ph[k]) for k in ("cnt", "ilen")] + [_np(eng.get_paths(count)[1])]
+
+    wide = _engine(binding, g, x, lanes=512)
+    free = torch.cuda.mem_get_info()[0]
+    ref = phase(wide)
+    assert free - torch.cuda.mem_get_info()[0] > 6 << 30  # (four batches)
+    filler = _fill(64 << 20)
+    wide.load_csr(rp2, col2, directed=True)  # needs more than is free
+    dist = _np(wide.bfs(0)[0])
+    wide.close()
+    del filler
+    torch.cuda.empty_cache()
+    eng = binding.PercIS(0)
+    eng.load_csr(rp2, col2, directed=True)
+    assert np.array_equal(_np(eng.bfs(0)[0]), dist)
+    eng.close()
+    narrow = _engine(binding, g, x, lanes=512)
+    filler = _fill(3 << 30)
+    for a, b in zip(phase(narrow), ref):
+        assert np.array_equal(a, b)
+    del filler
+    torch.cuda.empty_cache()
+    for a, b in zip(phase(narrow), ref):
+        assert np.array_equal(a, b)
+    narrow.close()
