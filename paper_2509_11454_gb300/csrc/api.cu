@@ -481,6 +481,7 @@ percis_status percis_load_csr(percis_ctx *ctx, int64_t n, int64_t nnz, const int
     DeviceGuard g(ctx->device);
     multi_free(ctx);
     ctx->ms_max_groups = 0;
+    ctx->bi_max_slots = 0;
     ctx->have_graph = false;
     ctx->have_states = false;
     ctx->have_paths = false;

@@ -1532,12 +1532,28 @@ percis_status direct_pass(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
     const int64_t budget = (int64_t)(ctx->opt.bi_scratch_gib > 0 ? ctx->opt.bi_scratch_gib : kDefaultScratchGiB) << 30;
     const int64_t full =
         std::min<int64_t>((int64_t)per_sm * ctx->num_sms, std::max<int64_t>(1, budget / (int64_t)per_slot));
-    const int64_t slots = std::min<int64_t>(full, std::max<int64_t>(count, 1));  // (count: at most, with count_dev)
+    int64_t slots = std::min<int64_t>(full, std::max<int64_t>(count, 1));  // (count: at most, with count_dev)
+    if (ctx->bi_max_slots) slots = std::min(slots, ctx->bi_max_slots);
     if (ctx->bi_slots < slots || ctx->bi_n != nslot) {
         // (phase 1 has 1,000 samples or more: all slots now, not 1,000 and then again for phase 2)
-        const int64_t have = 2 * slots >= full ? full : slots;
-        PERCIS_TRY(ensure(ctx, ctx->bi_info, sizeof(unsigned long long) * 4 * nslot * have, "bidirectional records"));
-        PERCIS_TRY(ensure(ctx, ctx->bi_queue, sizeof(int2) * 3 * nslot * have, "bidirectional queues"));
+        int64_t have = 2 * slots >= full && !ctx->bi_max_slots ? full : slots;
+        ctx->bi_slots = 0;  // (an allocation may fail)
+        for (;;) {
+            percis_status st =
+                ensure(ctx, ctx->bi_info, sizeof(unsigned long long) * 4 * nslot * have, "bidirectional records");
+            if (st == PERCIS_OK) st = ensure(ctx, ctx->bi_queue, sizeof(int2) * 3 * nslot * have, "bidirectional queues");
+            if (st == PERCIS_OK) break;
+            // a sample needs one slot, and more are an option of speed: as many as are
+            // wanted now, then half as many, until the memory can be had
+            for (DevBuf *b : {&ctx->bi_info, &ctx->bi_queue}) {
+                if (b->p) cudaFree(b->p);
+                *b = DevBuf{};
+            }
+            if (st != PERCIS_E_OOM || have == 1) return st;
+            have = have > slots ? slots : (have + 1) / 2;
+            ctx->bi_max_slots = have;
+        }
+        slots = std::min(slots, have);
         // level words of no sample (epoch 0)
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->bi_info.p, 0, sizeof(unsigned long long) * 4 * nslot * have, ctx->stream));
         ctx->bi_slots = have;

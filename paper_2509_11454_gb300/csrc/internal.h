@@ -111,6 +111,7 @@ struct percis_ctx {
     percis::DevBuf plan_dev;                           // lane batches of a many-graph phase
     percis::DevBuf bi_info, bi_queue;                  // bidirectional form, direct store: per-slot scratch
     int64_t bi_slots = 0, bi_n = 0, bi_epoch = 0;
+    int64_t bi_max_slots = 0;  // slots that could be had when memory ran out on this graph (0: no limit)
     percis::DevBuf bi_hent, bi_hq, bi_hep, bi_defer;   // bidirectional form, hashed store: tables, queues,
                                                        // slot epochs, samples handed to the direct store
     int64_t bi_hregion = 0, bi_hslots = 0;

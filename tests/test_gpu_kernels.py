@@ -393,3 +393,34 @@ def test_batches_side_by_side_in_little_memory(binding):
     for a, b in zip(phase(narrow), ref):
         assert np.array_equal(a, b)
     narrow.close()
+
+
+@pytest.mark.parametrize("n,count,leave", [(1 << 18, 400, 7.0), (1 << 18, 400, 2.0), (1 << 15, 1300, 1.6)])
+def test_bidir_slots_in_little_memory(binding, n, count, leave):
+    """The direct store's slots (14.7 MB each at 2^18 vertices, 608 of them; 1.8 MB and 1,216
+    at 2^15) in `leave` GB: as many as can be had, with the same counts and paths."""
+    rng = np.random.default_rng(n)
+    src, dst = np.arange(n), (np.arange(n) + 1) % n
+    src, dst = np.concatenate([src, rng.integers(0, n, 2 * n)]), np.concatenate([dst, rng.integers(0, n, 2 * n)])
+    g = synth.csr_from_edges(n, src, dst, directed=False)
+    x = synth.states_uniform(n, 1)
+
+    def phase(eng):
+        ph = eng.run_phase(7, 1, count)
+        return [_np(ph[k]) for k in ("cnt", "ilen")] + [_np(eng.get_paths(count)[1])]
+
+    eng = _engine(binding, g, x, form="bidir", bi_table_log=-1)
+    ref = phase(eng)
+    eng.close()
+    eng = _engine(binding, g, x, form="bidir", bi_table_log=-1)
+    filler = _fill(int(leave * 1e9))
+    for k in range(2):
+        for a, b in zip(phase(eng), ref):
+            assert np.array_equal(a, b), k
+    del filler
+    torch.cuda.empty_cache()
+    eng.load_csr(g.row_ptr, g.col)
+    eng.set_states(x)
+    for a, b in zip(phase(eng), ref):
+        assert np.array_equal(a, b)
+    eng.close()
