@@ -246,6 +246,7 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
     int32_t *overflow = &po->overflow;
     const int64_t n = ctx->n;
     const int64_t cap_count = std::max<int64_t>(count, 1);
+    ctx->have_paths = false;  // (from here on: an allocation that fails has given up the last phase's buffer)
     PERCIS_TRY(ensure(ctx, ctx->pair_s, sizeof(int32_t) * cap_count, "pairs"));
     PERCIS_TRY(ensure(ctx, ctx->pair_t, sizeof(int32_t) * cap_count, "pairs"));
     PERCIS_TRY(ensure(ctx, ctx->kind, sizeof(int32_t) * cap_count, "kinds"));
@@ -255,10 +256,10 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
     PERCIS_TRY(ensure(ctx, ctx->arena_top, 64, "arena top"));
     if (ctx->arena_cap < cap_count * 8) {
         const int64_t cap = cap_count * 8;
+        ctx->arena_cap = 0;  // (an allocation may fail)
         PERCIS_TRY(ensure(ctx, ctx->arena, sizeof(int32_t) * cap, "path arena"));
         ctx->arena_cap = cap;
     }
-    ctx->have_paths = false;
     if (ctx->opt.instrument) PERCIS_TRY(ensure(ctx, ctx->counters, sizeof(unsigned long long) * 8, "counters"));
     PERCIS_TRY(ensure(ctx, ctx->ms_ctl, sizeof(MsCtl), "ms ctl"));
     const bool plain = ctx->opt.form == PERCIS_FORM_PLAIN;
@@ -319,6 +320,7 @@ percis_status run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count
             unsigned long long top = 0;
             PERCIS_CUDA(ctx, cudaMemcpy(&top, ctx->arena_top.p, sizeof(top), cudaMemcpyDeviceToHost));
             const int64_t cap = (int64_t)top + (int64_t)top / 4 + 1024;
+            ctx->arena_cap = 0;
             PERCIS_TRY(ensure(ctx, ctx->arena, sizeof(int32_t) * cap, "path arena"));
             ctx->arena_cap = cap;
             continue;

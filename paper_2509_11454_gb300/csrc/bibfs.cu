@@ -1688,6 +1688,7 @@ percis_status bidir_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, int
         const size_t ent_bytes = sizeof(unsigned long long) * 4 * (size_t)region * slots;
         const size_t q_bytes = sizeof(int2) * 3 * (size_t)qcap * slots;
         if (ctx->bi_hregion != region || ctx->bi_hslots != slots || ctx->bi_h0 != h0) {
+            ctx->bi_hregion = 0;  // (an allocation may fail)
             PERCIS_TRY(ensure(ctx, ctx->bi_hent, ent_bytes, "hashed entries"));
             PERCIS_TRY(ensure(ctx, ctx->bi_hq, q_bytes, "hashed queues"));
             PERCIS_TRY(ensure(ctx, ctx->bi_hep, sizeof(uint32_t) * slots, "slot epochs"));

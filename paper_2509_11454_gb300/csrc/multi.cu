@@ -345,9 +345,13 @@ extern "C" percis_status percis_load_graphs(percis_ctx *ctx, int32_t num_graphs,
         std::fill(gid.begin() + graph_vptr[g], gid.begin() + graph_vptr[g + 1], g);
     ctx->multi = m;
     m->largest = largest;
-    PERCIS_TRY(ensure(ctx, m->gid, sizeof(int32_t) * n, "graph ids"));
+    st = ensure(ctx, m->gid, sizeof(int32_t) * n, "graph ids");
+    if (st == PERCIS_OK) st = ensure(ctx, m->vptr_dev, sizeof(int64_t) * (num_graphs + 1), "graph offsets");
+    if (st != PERCIS_OK) {
+        multi_free(ctx);
+        return st;
+    }
     PERCIS_CUDA(ctx, cudaMemcpyAsync(m->gid.p, gid.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, ctx->stream));
-    PERCIS_TRY(ensure(ctx, m->vptr_dev, sizeof(int64_t) * (num_graphs + 1), "graph offsets"));
     PERCIS_CUDA(ctx, cudaMemcpyAsync(m->vptr_dev.p, graph_vptr, sizeof(int64_t) * (num_graphs + 1),
                                      cudaMemcpyHostToDevice, ctx->stream));
     PERCIS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

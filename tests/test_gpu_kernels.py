@@ -424,3 +424,30 @@ def test_bidir_slots_in_little_memory(binding, n, count, leave):
     for a, b in zip(phase(eng), ref):
         assert np.array_equal(a, b)
     eng.close()
+
+
+def test_phase_after_a_failed_allocation(binding):
+    """A phase that runs out of memory leaves no sample and no stale sizes: the path arena
+    (2^23 samples with 400 MB free) and the hashed store's tables (5 GB with 1 GB free);
+    the phases after it are as ever."""
+    g = synth.barabasi_albert(2000, 3, 1)
+    x = synth.states_uniform(g.n, 1)
+    eng = _engine(binding, g, x, form="bidir")
+
+    def phase():
+        ph = eng.run_phase(7, 1, 400)
+        return [_np(ph[k]) for k in ("cnt", "ilen")] + [_np(eng.get_paths(400)[1])]
+
+    ref = phase()
+    for leave, opts, count in ((400e6, {}, 1 << 23), (1e9, {"bi_table_log": 18, "bi_table_max_log": 18}, 400)):
+        eng.set_options(**opts)
+        filler = _fill(int(leave))
+        with pytest.raises(RuntimeError, match="OOM"):
+            binding.percis_run_phase(eng.ctx, 7, 1, count)
+        with pytest.raises(RuntimeError, match="NO_SAMPLE"):
+            binding.percis_get_paths(eng.ctx)
+        del filler
+        torch.cuda.empty_cache()
+        for a, b in zip(phase(), ref):
+            assert np.array_equal(a, b), leave
+    eng.close()
