@@ -728,10 +728,13 @@ __device__ bool grid_running_sum(const double *src, int64_t soff, double *dst, i
     return true;
 }
 
-// Cooperative launch of G blocks (all co-resident): w, then c_i, then r.
+// Cooperative launch of G blocks (all co-resident): w, then c_i, then r.  Nothing where the
+// sort has left a long run out of order (it is done again, and this launch after it): the
+// tables and C_v of disordered states were a third of a preparation that sorts twice.
 __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64_t n, double *w, double *ci,
                                                          double *r, double *dscal, TableCtl *ctl,
-                                                         uint64_t budget_ns) {
+                                                         uint64_t budget_ns, const uint32_t *sort_status) {
+    if (__ldcg(sort_status) & DEV_LONG_RUN) return;  // (the same in every thread: nothing writes it here)
     // positions past the last non-zero state: x_i = 0 and every sum before them
     // is +0, so w_i = c_i = r_i = 0 exactly; the scans start at the last non-zero one
     const int64_t nz = *reinterpret_cast<const long long *>(dscal + 2);
@@ -759,6 +762,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64
 // and max_v lambda_v = c / min_v C_v (the rounded division is monotone).
 __global__ void k_cv(const double *xs, const int32_t *perm, const double *w, double *dscal, int64_t n, double *Cv,
                      uint32_t *status) {
+    if (ld_relaxed_u32(status) & DEV_LONG_RUN) return;  // (set before this launch, if at all)
     const double c = dscal[0];
     const double w1 = w[1];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1003,7 +1007,8 @@ static percis_status prep_states_once(percis_ctx *ctx, bool full_sort, bool *aga
     TableCtl *tctl = ctx->table_ctl.as<TableCtl>();
     uint64_t budget = (uint64_t)(ctx->opt.timeout_s * 1e9);
     int64_t nn = n;
-    void *args[] = {&xs, &nn, &w, &ci, &r, &dscal, &tctl, &budget};
+    const uint32_t *sst = st;
+    void *args[] = {&xs, &nn, &w, &ci, &r, &dscal, &tctl, &budget, &sst};
     PERCIS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_tables, dim3(G), dim3(kScanThreads), args, 0,
                                                  ctx->stream));
     ctx->launches++;

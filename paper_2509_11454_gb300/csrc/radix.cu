@@ -305,8 +305,9 @@ __global__ void __launch_bounds__(kTileSort / 2) k_sort_tiles(unsigned long long
 
 // Pairs sorted (stably) by the bits from kFixBits up: the runs that agree there are put
 // in the order of the whole key.  A key smaller than the one before it in its run is a
-// descent; the first of a run lists the run's head (at most n / 2), and if the run is
-// above kFixRun long *over is set instead.  Runs of equal keys have none.
+// descent; the first of a run lists the run's head (at most n / 2), and one that lies
+// more than kFixRun behind the head sets *over instead, where nothing is fixed: all is
+// sorted again.  Runs of equal keys have none.
 constexpr int kFixBits = 24, kFixRun = 64;
 __global__ void k_list_runs(const unsigned long long *keys, int64_t n, long long *heads, unsigned long long *nheads,
                             uint32_t *over) {
@@ -315,22 +316,27 @@ __global__ void k_list_runs(const unsigned long long *keys, int64_t n, long long
         const unsigned long long key = keys[i], top = key >> kFixBits;
         unsigned long long next = keys[i - 1];
         if (next <= key || next >> kFixBits != top) continue;
+        if (ld_relaxed_u32(over) & DEV_LONG_RUN) return;
+        if (i > kFixRun && keys[i - kFixRun - 1] >> kFixBits == top) {
+            atomicOr(over, DEV_LONG_RUN);
+            return;
+        }
         int64_t h = i - 1;
         bool mine = true;  // an earlier descent of the run is another thread's
-        while (h > 0 && mine && i - h <= kFixRun) {
+        while (h > 0 && mine) {
             const unsigned long long k = keys[h - 1];
             if (k >> kFixBits != top) break;
             mine = k <= next;
             next = k;
             --h;
         }
-        if (i - h > kFixRun) atomicOr(over, DEV_LONG_RUN);
-        else if (mine) heads[atomicAdd(nheads, 1ull)] = h;
+        if (mine) heads[atomicAdd(nheads, 1ull)] = h;
     }
 }
 
 __global__ void k_fix_runs(unsigned long long *keys, int32_t *vals, int64_t n, const long long *heads,
                            const unsigned long long *nheads, uint32_t *over) {
+    if (ld_relaxed_u32(over) & DEV_LONG_RUN) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, m = (int64_t)*nheads;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += stride) {
         const int64_t h = heads[r];
@@ -415,7 +421,9 @@ percis_status radix_sort_u64(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uin
 // 28 bits of a double's mantissa tell all but a few states apart), then the runs that
 // agree there; where a long run is out of order (states within 2^-28 of one another
 // by the hundred) DEV_LONG_RUN is set in *status and the caller sorts again with `full`,
-// all eight passes.  1.5M states: 327 us of kernels with eight passes, 218 us.
+// all eight passes.  1.5M states: 327 us of kernels with eight passes, 218 us; their whole
+// preparation 458 us, where a quarter of them (a saturated sigmoid) or all lie within 2^-28
+// of one another 866 and 862 us (eight passes at once: about 570).
 int state_sort_swaps(int64_t n, bool full) {
     if (n > kMergeMaxN) return full ? 8 : (64 - kFixBits) / 8;
     int k = 0;
