@@ -432,6 +432,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const Place at, const 
             ctl->qn[1] = 0;
             ctl->qh[0] = 0;
             ctl->qh[1] = 0;
+            for (int q = 0; q < 2; ++q) ctl->fedges[q] = ctl->uedges[q] = 0ull;  // (a last level leaves its own)
             ctl->push_next = a.policy != 0;
             ctl->t_start = globaltimer_ns();
         }

@@ -451,3 +451,27 @@ def test_phase_after_a_failed_allocation(binding):
         for a, b in zip(phase(), ref):
             assert np.array_equal(a, b), leave
     eng.close()
+
+
+@pytest.mark.parametrize("count", [70, 100, 130, 200])
+def test_batch_direction_from_its_own_work(binding, count):
+    """The work estimates that choose a level's direction are the batch's own: those of the
+    last batch (64 lanes, one after the other) before its first level, none, and before its
+    second, from the neighbours of its sources."""
+    g = synth.barabasi_albert(600, 2, 3)
+    eng = _engine(binding, g, synth.states_uniform(g.n, 3), lanes=64, lane_order=0, instrument=1)
+    s = _np(eng.run_phase(4, 1, count)["s"])
+    rec = binding.percis_last_levels(eng.ctx)
+    eng.close()
+    u = np.unique(s)
+    assert (len(u) > 64) == (count > 70)  # (one batch, or several)
+    last = u[(len(u) - 1) // 64 * 64:]
+    deg = np.diff(g.row_ptr)
+    seen = np.zeros((len(last), g.n), dtype=bool)
+    for lane, v in enumerate(last):
+        seen[lane, g.col[g.row_ptr[v]:g.row_ptr[v + 1]]] = True
+    front = seen.any(axis=0)
+    seen[np.arange(len(last)), last] = True
+    assert len(rec) >= 2
+    assert (rec[0][3], rec[0][1] >> 1) == (0, 0)
+    assert (rec[1][3], rec[1][1] >> 1) == (deg[front].sum(), deg[~seen.all(axis=0)].sum())
