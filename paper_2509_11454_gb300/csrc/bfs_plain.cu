@@ -472,7 +472,8 @@ static percis_status ensure_plain(percis_ctx *ctx) {
     PERCIS_TRY(ensure(ctx, ctx->qb, sizeof(int32_t) * n, "queue"));
     PERCIS_TRY(ensure(ctx, ctx->plain_ctl, 256, "plain ctl"));
     if (fresh || ctx->epoch <= 0 || ctx->epoch > (1 << 30)) {
-        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->stamp.p, 0, sizeof(u64) * n, ctx->stream));
+        // (all of the buffer: a larger graph that still fits it is not fresh)
+        PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->stamp.p, 0, ctx->stamp.bytes, ctx->stream));
         PERCIS_CUDA(ctx, cudaMemsetAsync(ctx->plain_ctl.p, 0, 256, ctx->stream));
         ctx->epoch = 0;
     }

@@ -475,3 +475,25 @@ def test_batch_direction_from_its_own_work(binding, count):
     assert len(rec) >= 2
     assert (rec[0][3], rec[0][1] >> 1) == (0, 0)
     assert (rec[1][3], rec[1][1] >> 1) == (deg[front].sum(), deg[~seen.all(axis=0)].sum())
+
+
+@pytest.mark.parametrize("n", [3000, 30000, 200000])
+def test_plain_bfs_on_a_slightly_larger_graph(binding, n):
+    """A graph 1/32 larger than the one the level stamps were allocated for: every vertex of
+    a binary tree at its level, also past the first graph's last, where the memory held
+    other values before (the states of an engine that has gone)."""
+    def tree(n):
+        v = np.arange(1, n)
+        return synth.csr_from_edges(n, v, (v - 1) // 2, directed=False)
+
+    for _ in range(4):
+        old = [_engine(binding, tree(n), 0.5 + 0.5 * synth.states_uniform(n, 1)) for _ in range(4)]
+        for eng in old:
+            eng.close()
+        eng = binding.PercIS(0)
+        for k in (n, n + n // 32):
+            g = tree(k)
+            eng.load_csr(g.row_ptr, g.col)
+            dist, sigma = (_np(a) for a in eng.bfs(0))
+            assert np.array_equal(dist, np.floor(np.log2(np.arange(k) + 1))) and np.all(sigma == 1), k
+        eng.close()
