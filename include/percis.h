@@ -111,11 +111,14 @@ typedef struct {
                                  (largest) graph at most half full, at most 2^20 entries; k =
                                  at most 2^k.  Samples that would fill more than 3/4 of it, or
                                  pass 4,095 levels on a side, are handed to the heavy pass. */
-    int32_t bi_scratch_gib;   /* direct store: device memory its blocks may use, GiB (0 = 48);
-                                 it holds 56 bytes per vertex and block, so it caps the blocks
-                                 (the heavy pass wants one block per SM: 152 x 56 x n bytes) */
+    int32_t bi_scratch_gib;   /* direct store: device memory its blocks may use, GiB (0 = 48;
+                                 fewer blocks run where less can be had); it holds 56 bytes
+                                 per vertex and block, so it caps the blocks (the heavy pass
+                                 wants one block per SM: 152 x 56 x n bytes) */
     int32_t bi_blocks_per_sm; /* bidirectional first pass: resident blocks per SM, 0 (default) = as
-                                 many as fit (4); fewer leave more memory bandwidth to each */
+                                 many as fit (4 of 256 threads, or 8 of 128 on graphs of up to
+                                 2^15 vertices); fewer leave more memory bandwidth to each, and
+                                 any other value keeps 256 threads */
     int32_t tune_form;        /* 1: percis_autotune may also switch between the batched and the
                                  bidirectional form (results then change with the form: both
                                  draw a uniform shortest path, by different procedures) */
@@ -176,7 +179,8 @@ typedef struct {
 percis_status percis_create(percis_ctx **out, int device, void *stream);
 /* Free every buffer the context owns.  NULL is ignored. */
 void percis_destroy(percis_ctx *ctx);
-/* Switch the stream later calls are ordered on (not owned). */
+/* Switch the stream later calls are ordered on (not owned); the graphs of a
+ * many-graph context follow. */
 percis_status percis_set_stream(percis_ctx *ctx, void *stream);
 /* Last error message of this context ("" when none).  Owned by the context. */
 const char *percis_last_error(const percis_ctx *ctx);

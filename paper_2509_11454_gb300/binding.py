@@ -344,9 +344,6 @@ class PercIS:
         self.options = o
         return {name: getattr(o, name) for name, _ in o._fields_}
 
-    def _sync_stream(self):
-        percis_set_stream(self.ctx, self.torch.cuda.current_stream(self.device).cuda_stream)
-
     def load_csr(self, row_ptr, col, directed: bool = False):
         t = self.torch
         rp = row_ptr if isinstance(row_ptr, np.ndarray) else row_ptr.to(t.int64).contiguous()

@@ -1,6 +1,7 @@
 // Plain form of RandomSP (Section III-B): for every sampled pair one
 // cooperative launch runs a level-synchronous sigma-counting BFS from s over
-// the whole GPU (frontier queues, warp per frontier vertex), truncated once
+// the whole GPU (frontier queues; a warp takes eight rows, all of it a long one,
+// and 32 warps a hub's; block 0 alone the small levels), truncated once
 // t's level is discovered, then one single-warp launch backtracks a uniform
 // shortest path.  This is the baseline the batched form is measured against.
 // It also serves VertexDiamUB and the single-source BFS inspection call.
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(kPlainBlock, 1) k_plain_bfs(PlainArgs a) {
     __shared__ double s_red[kPlainWarps];
     __shared__ int32_t s_buf[kPlainWarps][kClaimBuf];  // claimed vertices on their way to the frontier
     PlainCtl *ctl = a.ctl;
-    GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
+    GridBarrier *bar = &ctl->bar;
     uint32_t *status = &ctl->status;
     const u64 ep = (u64)(uint32_t)a.epoch << 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "internal.h"
+
 namespace percis {
 
 // Status bits written by kernels into a device word (atomicOr).
@@ -111,12 +113,6 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
     return t;
 }
 
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -127,10 +123,6 @@ __device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t *p) {
     uint64_t v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
-}
-
-__device__ __forceinline__ int64_t ld_relaxed_s64(const int64_t *p) {
-    return (int64_t)ld_relaxed_u64((const uint64_t *)p);
 }
 
 // ------------------------------------------------------------ grid barrier
@@ -146,18 +138,13 @@ __device__ __forceinline__ int64_t ld_relaxed_s64(const int64_t *p) {
 // budget_ns the waiting block sets DEV_TIMEOUT and the word's top bit, which every
 // poll and later arrival sees, so that each barrier from there on returns false; a
 // kernel that sees `false` must exit.
-struct alignas(8) GridBarrier {
-    uint32_t count;  // low and high half of the arrivals
-    uint32_t gen;
-};
-
 __device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, uint64_t budget_ns,
                                           uint32_t blocks) {
     __shared__ int s_ok;
     constexpr uint64_t kOver = 1ull << 63;
     __syncthreads();
     if (threadIdx.x == 0) {
-        uint64_t *word = reinterpret_cast<uint64_t *>(bar);
+        unsigned long long *word = &bar->arrivals;
         uint64_t a;
         // release: the block's writes (ordered before by the block barrier); acquire: for the last to arrive
         asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(a) : "l"(word), "l"(1ull) : "memory");
@@ -178,7 +165,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *status, ui
                     if (c >= target) break;
                     if (globaltimer_ns() - t0 > budget_ns) {
                         atomicOr(status, DEV_TIMEOUT);
-                        atomicOr(reinterpret_cast<unsigned long long *>(word), (unsigned long long)kOver);
+                        atomicOr(word, (unsigned long long)kOver);
                         ok = 0;
                         break;
                     }
@@ -205,12 +192,6 @@ __device__ __forceinline__ double warp_inclusive_scan(double v) {
         if (lane >= off) v = __dadd_rn(v, o);
     }
     return v;
-}
-
-__device__ __forceinline__ uint64_t warp_or64(uint64_t v) {
-    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
-    const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
-    return ((uint64_t)hi << 32) | lo;
 }
 
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {

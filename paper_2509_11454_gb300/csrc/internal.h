@@ -24,9 +24,14 @@ struct DevBuf {
     }
 };
 
-// Control block of the persistent kernels (device memory, zeroed per launch).
+// Arrivals at a grid barrier since the word was zeroed (grid_sync).
+struct GridBarrier {
+    unsigned long long arrivals;
+};
+
+// Control block of a batch of the batched form (device memory, zeroed per launch).
 struct alignas(16) MsCtl {
-    uint32_t bar_count, bar_gen;  // GridBarrier
+    GridBarrier bar;
     uint32_t status;
     uint32_t ticket;
     int32_t level;                // last level reached
@@ -51,7 +56,7 @@ struct PairTables {
 };
 
 struct PlainCtl {
-    uint32_t bar_count, bar_gen;
+    GridBarrier bar;
     uint32_t status;
     int32_t qsize[3];  // queue sizes, level L in slot L % 3: rows of ordinary length,
     int32_t hsize[3];  // long rows, and the level's vertices of long in-rows
@@ -88,7 +93,7 @@ struct percis_ctx {
     bool have_states = false;
     percis::DevBuf x, xs, perm, w, ci, r, Cv, grp_lo, grp_hi;
     double c_host = 0.0, dhat_host = 0.0;
-    percis::DevBuf dscal;  // device scalars: [0] = c, [1] = dhat
+    percis::DevBuf dscal;  // device scalars: [0] = c, [1] = smallest C_v, [2] = number of non-zero states (int64)
 
     // plain BFS state
     percis::DevBuf stamp, plain_hub, sigma1, qa, qb, plain_ctl;
@@ -234,8 +239,8 @@ percis_status transpose_finish(percis_ctx *ctx);  // in-adjacency: offsets (vali
 percis_status prep_graph(percis_ctx *ctx);  // transpose (directed), validation, VertexDiamUB
 percis_status prep_states(percis_ctx *ctx);  // sort, tables, C_v, lambda, d^
 percis_status prep_lambda(percis_ctx *ctx, double *lam);  // lambda_v of every vertex (device)
-percis_status prep_groups(percis_ctx *ctx);
-percis_status wait_graph(percis_ctx *ctx);  // the context stream waits for the in-adjacency  // tie groups of the sorted states (backward, on first use)
+percis_status prep_groups(percis_ctx *ctx);  // tie groups of the sorted states (backward, on first use)
+percis_status wait_graph(percis_ctx *ctx);   // the context stream waits for the in-adjacency
 percis_status prep_vorder(percis_ctx *ctx);  // lane order of the batched form (on first use)
 
 // sampler.cu

@@ -1,8 +1,9 @@
 // Batched form of RandomSP: up to W = 64*K distinct sources ("lanes") share
 // one persistent cooperative launch.  Per vertex the launch keeps K 64-bit
 // words of visited bits and, for every level L, K words of frontier bits
-// F_L(v) (bit j set iff v is at distance L from lane j's source).  A level is
-// one pull pass over all vertices:
+// F_L(v) (bit j set iff v is at distance L from lane j's source).  A level finds
+// its vertices by a pull over all that some lane has not visited, or by a push
+// over the frontier's out-edges, whichever is estimated to be less work:
 //     c = active & ~visited(v),  F_{L+1}(v) = OR_{u in in(v)} F_L(u) & c,
 //     sigma_j(v) = sum over u in in(v) with bit j of F_L(u) & c of sigma_j(u)
 // (the sigma recurrence of the oracle, summed in any order: the values are
@@ -389,7 +390,7 @@ __device__ __forceinline__ bool ms_batch(const MsArgs &a, const Place at, const 
     bool ovf = false;
     unsigned long long n_s[2] = {0, 0}, n_uv = 0, n_ue = 0;  // sigma reads and writes; frontier vertices, edges
     MsCtl *ctl = a.ctl;
-    GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
+    GridBarrier *bar = &ctl->bar;
     uint32_t *status = a.status;
     const int lane = threadIdx.x & 31;
     const int warp_in_block = threadIdx.x >> 5;
@@ -1048,7 +1049,7 @@ __global__ void __launch_bounds__(kMsBlock, 4) k_msbfs(const __grid_constant__ M
     const int32_t grp = (int32_t)blockIdx.x % l.groups;
     const Place at{(int32_t)blockIdx.x / l.groups, (int32_t)gridDim.x / l.groups};
     const MsArgs &a = l.g[grp];
-    GridBarrier *bar = reinterpret_cast<GridBarrier *>(a.ctl);
+    GridBarrier *bar = &a.ctl->bar;
     uint32_t *status = a.status;
     int64_t B = 1;
     long long U = 0;
@@ -1407,8 +1408,8 @@ percis_status batched_phase(percis_ctx *ctx, uint64_t seed, uint32_t tag_path, i
         Lcap = (int)std::max<int64_t>(Lcap, std::min<int64_t>(ctx->vertex_diam + 3, std::min<int64_t>(lmem, 1 << 20)));
     }
     const int64_t B = ctx->multi ? (int64_t)plan.size() : (n_sources + W - 1) / W;
-    // batches side by side, while their state stays within 24 GiB (the work counters and
-    // the level records are those of one batch at a time)
+    // batches side by side, while their state stays within 24 GiB (fewer where that cannot be
+    // had: ms_give_back; the work counters and the level records are those of one at a time)
     int G = 1;
     if (!ctx->opt.instrument) {
         const MsSizes z = ms_sizes(W, Lcap, nr_max);

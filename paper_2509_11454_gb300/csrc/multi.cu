@@ -1,9 +1,10 @@
 // Many independent graphs in one context.  Each graph is its own instance of
 // the problem of Section II (own C, lambda, d^, vertex-diameter bound, l1 and
-// l), kept in a sub-context that does its own state preprocessing, pair
-// sampling, bounds, finalisation and backward pass with the single-graph
-// kernels.  The union context holds the block-diagonal CSR and runs the
-// sigma-counting BFS of all graphs together: the sampled sources of every
+// l), kept in a sub-context that does its own state preprocessing, bounds and
+// the vertices' part of the backward pass with the single-graph kernels.  The
+// union context holds the block-diagonal CSR and draws the pairs, finalises, adds
+// the samples' part of the backward pass and runs the sigma-counting BFS of all
+// graphs together.  In the batched form the sampled sources of every
 // graph are grouped into lanes, and consecutive lanes share one batched
 // launch over the vertex range of their graphs.
 //
@@ -36,8 +37,8 @@ struct MultiGraph {
     std::vector<PairTables> tabs_host;
     DevBuf tabs;                        // every graph's sampling tables
     DevBuf soff_dev, ell_dev, c_dev, stats, pmax;  // c_dev: C of every graph
-    // recorded per-graph sampling launches of each phase (pair tag 0 / 1), the
-    // counts they were recorded for, and the device word they read the seed from
+    // the recorded sampling launch of each phase (pair tag 0 / 1), the counts and
+    // buffers it was recorded for, and the device word it reads the seed from
     cudaGraphExec_t samp_exec[2] = {nullptr, nullptr};
     std::vector<int64_t> samp_key[2];
     DevBuf seed_dev;
@@ -89,8 +90,7 @@ __global__ void k_pmax_multi(const double *Cv, const double *C, const unsigned l
 __global__ void k_finalize_multi(const double *Cv, const double *C, const unsigned long long *cnt, const double *acc,
                                  const int32_t *gid, const double *ell, int64_t n, double *pc) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-{
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const double k = acc ? acc[v] : (double)cnt[v];
         pc[v] = k == 0.0 ? 0.0 : C[gid[v]] / Cv[v] * k / ell[gid[v]];
     }

@@ -33,7 +33,7 @@ constexpr int kBlock = 256;
 constexpr double kDefaultBudgetS = 10.0;
 
 struct NoAllocCtl {
-    uint32_t bar_count, bar_gen;  // GridBarrier
+    GridBarrier bar;
     uint32_t status;
     int32_t qsize[2];
     int32_t found;
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kBlock) k_bfs_noalloc(int64_t n, const int64_t
     NoAllocCtl *ctl = reinterpret_cast<NoAllocCtl *>(scratch);
     int32_t *qa = reinterpret_cast<int32_t *>(scratch + kCtlBytes);
     int32_t *qb = qa + kNoAllocMaxN;
-    GridBarrier *bar = reinterpret_cast<GridBarrier *>(ctl);
+    GridBarrier *bar = &ctl->bar;
     uint32_t *status = &ctl->status;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;

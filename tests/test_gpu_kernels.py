@@ -497,3 +497,24 @@ def test_plain_bfs_on_a_slightly_larger_graph(binding, n):
             dist, sigma = (_np(a) for a in eng.bfs(0))
             assert np.array_equal(dist, np.floor(np.log2(np.arange(k) + 1))) and np.all(sigma == 1), k
         eng.close()
+
+
+@pytest.mark.parametrize("n,diamond", [(600, False), (200, True)])
+@pytest.mark.parametrize("lanes", [64, 512])
+def test_batched_needed_counts_past_their_list(binding, n, diamond, lanes):
+    """Needed (vertex, level) pairs past the room of their list (2 n; a directed cycle's
+    lanes need every vertex at nearly every level, and its walks are too few for the
+    counts of all vertices): the counts are then listed level by level; the oracle's."""
+    src, dst = np.arange(n), (np.arange(n) + 1) % n
+    if diamond:  # 0 -> n -> 2 beside 0 -> 1 -> 2
+        src, dst, n = np.append(src, [0, n]), np.append(dst, [n, 2]), n + 1
+    g = synth.csr_from_edges(n, src, dst, directed=True)
+    x = synth.states_uniform(n, 2)
+    eng = _engine(binding, g, x, lanes=lanes)
+    ph = eng.run_phase(7, 1, 1500)
+    nodes = _np(eng.get_paths(1500)[1])
+    ref = oracle.run_samples(oracle.from_synth(g), oracle.prepare(x), 7, 1, 3, 0, 1500, keep_paths=True)
+    for k in ("s", "t", "kind", "ilen", "cnt"):
+        assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
+    assert np.array_equal(nodes, ref.path_nodes) and ref.ilen.sum() > 100 * n
+    eng.close()
