@@ -258,7 +258,8 @@ percis_status percis_get_prep(percis_ctx *ctx, int32_t *perm, double *xs, double
                               double *lambda, double *c, double *dhat, int64_t *vertex_diam);
 
 /* Algorithm 2 sampling of pairs i0 .. i0+count-1 with Philox tag `tag`
- * (0 = phase 1, 1 = phase 2).  Device outputs s, t: int32[count] node ids. */
+ * (0 = phase 1, 1 = phase 2).  Device outputs s, t: int32[count] node ids.
+ * INVALID on many graphs (percis_run_phase draws theirs). */
 percis_status percis_sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag, int64_t i0, int64_t count, int32_t *s,
                                   int32_t *t);
 
@@ -282,7 +283,8 @@ percis_status percis_msbfs(percis_ctx *ctx, int32_t nsrc, const int32_t *sources
  * (any may be NULL): s, t int32[count]; kind int32[count] (0 = path sampled,
  * 1 = R(x_s - x_t) = 0, 2 = t unreachable); ilen int32[count] = |I(tau)|;
  * cnt int64[n] = number of sampled paths with v internal.  The paths stay
- * in the context for percis_get_paths / percis_backward. */
+ * in the context for percis_get_paths / percis_backward.  Of many graphs (G of
+ * them), graph g takes samples floor(count g / G) to floor(count (g + 1) / G) - 1. */
 percis_status percis_run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count, int32_t *s, int32_t *t,
                                int32_t *kind, int32_t *ilen, int64_t *cnt);
 
@@ -323,7 +325,7 @@ percis_status percis_estimate_graphs(percis_ctx *ctx, double eps, double delta, 
 /* Autotuner (speed options only; not in the paper, whose results these options
  * do not change).  Coordinate descent, each candidate timed (CUDA events, best
  * of two) on probe phases of probe_samples pairs drawn with `seed` from the
- * loaded graph and states:
+ * loaded graph (or graphs, as percis_run_phase shares it out) and states:
  *  - batched form: lane order {0, 1}, then lanes {64, 128, 256, 512}, then
  *    direction {pull, push, work estimate with push_alpha 0.25, 0.5, 1, 2};
  *  - bidirectional form: bi_heavy_edges {2048, 4096, 8192, 16384, 65536,

@@ -183,6 +183,11 @@ percis_status need_states(percis_ctx *ctx) {
     return PERCIS_OK;
 }
 
+// a phase of `count` samples in all (of many graphs: each its share)
+percis_status phase_of(percis_ctx *ctx, uint64_t seed, int phase, int64_t count, PhaseOut *po) {
+    return ctx->multi ? multi_run_phase(ctx, seed, phase, count, po) : run_phase(ctx, seed, phase, count, po);
+}
+
 // (plain: the plain form's word too)
 uint32_t read_status(percis_ctx *ctx, bool plain = true) {
     char *hm = host_mirror(ctx);
@@ -679,6 +684,7 @@ percis_status percis_get_prep(percis_ctx *ctx, int32_t *perm, double *xs, double
 percis_status percis_sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag, int64_t i0, int64_t count, int32_t *s,
                                   int32_t *t) {
     PERCIS_TRY(need_states(ctx));
+    if (ctx->multi) return set_err(ctx, PERCIS_E_INVALID, "the pairs of many graphs are drawn by their phases");
     if (count < 0 || i0 < 0 || (count > 0 && (!s || !t))) return set_err(ctx, PERCIS_E_INVALID, "bad arguments");
     DeviceGuard g(ctx->device);
     PERCIS_TRY(sample_pairs(ctx, seed, tag, i0, count, s, t, nullptr));
@@ -731,7 +737,7 @@ percis_status percis_run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_
     if ((phase != 0 && phase != 1) || count < 1) return set_err(ctx, PERCIS_E_INVALID, "phase 0/1, count >= 1");
     DeviceGuard g(ctx->device);
     PhaseOut po;
-    PERCIS_TRY(run_phase(ctx, seed, phase, count, &po));
+    PERCIS_TRY(phase_of(ctx, seed, phase, count, &po));
     ctx->last_ell = count;
     auto cp = [&](void *dst, const DevBuf &b, size_t bytes) -> percis_status {
         if (!dst) return PERCIS_OK;
@@ -775,7 +781,7 @@ percis_status percis_autotune(percis_ctx *ctx, int64_t probe_samples, uint64_t s
         for (int rep = 0; rep < 2; ++rep) {
             PhaseOut po;
             PERCIS_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
-            PERCIS_TRY(run_phase(ctx, seed + (uint64_t)rep, 0, probe_samples, &po));
+            PERCIS_TRY(phase_of(ctx, seed + (uint64_t)rep, 0, probe_samples, &po));
             PERCIS_CUDA(ctx, cudaEventRecord(e1, ctx->stream));
             PERCIS_CUDA(ctx, cudaEventSynchronize(e1));
             float t = 0.f;

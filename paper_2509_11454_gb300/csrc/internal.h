@@ -313,6 +313,8 @@ struct LaneBatch {
     int32_t lane_base, nlanes, vlo;
     int64_t nr;
 };
+// one phase of `count` samples spread evenly over the graphs
+percis_status multi_run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count, PhaseOut *po);
 percis_status multi_plan_batches(percis_ctx *ctx, int64_t n_sources, int W, std::vector<LaneBatch> *out);
 percis_status multi_lambda(percis_ctx *ctx, double *lam);  // lambda_v of every graph's vertices
 int64_t multi_range(percis_ctx *ctx);  // vertex range of the batch buffers

@@ -282,6 +282,19 @@ percis_status multi_phase(percis_ctx *ctx, uint64_t seed, int phase, const std::
 
 }  // namespace
 
+percis_status percis::multi_run_phase(percis_ctx *ctx, uint64_t seed, int phase, int64_t count, PhaseOut *po) {
+    MultiGraph *m = ctx->multi;
+    std::vector<int64_t> counts((size_t)m->G);
+    for (int32_t g = 0; g < m->G; ++g)
+        counts[g] = count / m->G * (g + 1) + count % m->G * (g + 1) / m->G - (count / m->G * g + count % m->G * g / m->G);
+    PERCIS_TRY(multi_phase(ctx, seed, phase, counts, po));
+    // (a backward pass divides each graph's samples by their number)
+    const std::vector<double> ell(counts.begin(), counts.end());
+    PERCIS_TRY(ensure(ctx, m->ell_dev, sizeof(double) * m->G, "graph l"));
+    PERCIS_CUDA(ctx, cudaMemcpyAsync(m->ell_dev.p, ell.data(), sizeof(double) * m->G, cudaMemcpyHostToDevice, ctx->stream));
+    return PERCIS_OK;
+}
+
 extern "C" percis_status percis_load_graphs(percis_ctx *ctx, int32_t num_graphs, const int64_t *graph_vptr, int64_t n,
                                             int64_t nnz, const int64_t *row_ptr, const int32_t *col, int directed) {
     if (!ctx) return PERCIS_E_INVALID;

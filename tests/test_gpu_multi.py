@@ -262,3 +262,41 @@ def test_stream_switch(binding, form, own):
         lo, hi = vptr[g], vptr[g + 1]
         lam = oracle.prepare(x[lo:hi], cv_method="sorted").lam
         assert np.max(np.abs(switched[1][lo:hi] - lam) / lam) <= 1e-12
+
+
+@pytest.mark.parametrize("form", ["batched", "bidir"])
+@pytest.mark.parametrize("count", [2, 400, 4001])
+def test_phases_without_an_estimate(binding, form, count):
+    """A phase of many graphs before any estimate, with more samples than any phase before
+    it, and with fewer than there are graphs: each graph's share, with the oracle's pairs,
+    lengths, counts and gradients; the autotuner's probes; no pairs outside a phase."""
+    graphs = synth.graph_batch([300, 90, 160], 3)
+    vptr, rp, col = synth.union_csr(graphs)
+    x = synth.states_uniform(int(vptr[-1]), 1)
+    eng = binding.PercIS(0)
+    eng.set_options(form=form)
+    eng.load_graphs(vptr, rp, col)
+    eng.set_states(x)
+    eng.autotune(probe_samples=count, seed=1)
+    eng.set_options(form=form)
+    eng.run_phase(6, 1, 3)
+    ph = {k: v.cpu().numpy() for k, v in eng.run_phase(6, 1, count).items()}
+    gvec = np.random.default_rng(3).standard_normal(int(vptr[-1]))
+    gx = eng.backward(torch.as_tensor(gvec, device="cuda")).cpu().numpy()
+    with pytest.raises(RuntimeError, match="INVALID"):
+        eng.sample_pairs(1, 0, 0, 10)
+    eng.close()
+    for g, graph in enumerate(graphs):
+        lo, hi = vptr[g], vptr[g + 1]
+        a, b = count * g // 3, count * (g + 1) // 3
+        prep = oracle.prepare(x[lo:hi], cv_method="sorted")
+        ref = oracle.run_samples(oracle.from_synth(graph), prep, 6, 1, 3, a, b - a, keep_paths=True,
+                                 bidir=form == "bidir")
+        for k in ("s", "t"):
+            assert np.array_equal(ph[k][a:b] - lo, getattr(ref, k)), (g, k)
+        for k in ("kind", "ilen"):
+            assert np.array_equal(ph[k][a:b], getattr(ref, k)), (g, k)
+        assert np.array_equal(ph["cnt"][lo:hi], ref.cnt), g
+        if b > a:
+            want = oracle.vjp_fixed(prep, b - a, ref, prep.lam * ref.cnt / (b - a), gvec[lo:hi])
+            assert np.linalg.norm(gx[lo:hi] - want) <= 1e-10 * max(np.linalg.norm(want), 1e-300), g
