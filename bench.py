@@ -66,9 +66,9 @@ DEFAULT_WORKLOAD = "rmat22_beta"
 # DRAM traffic per launch of the dominant kernel from an ncu capture, valid only
 # for the kernel source it was taken on (sha256 of the .cu file) and the workload.
 NCU_TRAFFIC = {
-    # one phase-2 pass (first pass + heavy pass) of a warm-up estimate: 1.022 GB read + 0.254 GB written
-    ("rmat22_beta", "bibfs.cu"): {"sha256": "f0b7f101d1fd218f480f96be6b1301e4e79c9c902a692ce54032a0b89f61ebd2",
-                                  "bytes_per_unit": 1.276e9},
+    # one phase-2 pass (first pass + heavy pass) of a warm-up estimate: 1.050 GB read + 0.318 GB written
+    ("rmat22_beta", "bibfs.cu"): {"sha256": "5523f662ddd8b8af12af36a81205b948da3246eb6b3e826932b168f1aa2135b9",
+                                  "bytes_per_unit": 1.368e9},
 }
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 L2_FLUSH_BYTES = 256 << 20
