@@ -175,7 +175,8 @@ typedef struct {
 /* ------------------------------------------------------------ lifecycle */
 
 /* Create a context on `device`.  `stream` is a cudaStream_t (NULL = a new
- * non-blocking stream owned by the context). */
+ * stream owned by the context, ordered with the legacy default stream, where
+ * such a caller's work is). */
 percis_status percis_create(percis_ctx **out, int device, void *stream);
 /* Free every buffer the context owns.  NULL is ignored. */
 void percis_destroy(percis_ctx *ctx);

@@ -301,7 +301,8 @@ def percis_last_levels(ctx, cap: int = 32) -> list[tuple[int, ...]]:
 # ------------------------------------------------------ torch-facing engine
 
 class PercIS:
-    """One library context bound to a CUDA device and torch's current stream."""
+    """One library context bound to a CUDA device and torch's current stream (on torch's
+    default stream, which has no handle: to a stream of its own that waits for it)."""
 
     def __init__(self, device: int = 0, **options):
         import torch

@@ -401,7 +401,9 @@ percis_status percis_create(percis_ctx **out, int device, void *stream) {
     if (stream) {
         ctx->stream = (cudaStream_t)stream;
     } else {
-        e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
+        // (one that waits for the legacy default stream: a caller there has no handle to give,
+        // and its inputs may still be in the making)
+        e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamDefault);
         if (e != cudaSuccess) {
             delete ctx;
             return PERCIS_E_CUDA;

@@ -236,6 +236,7 @@ percis_status transpose_sort(percis_ctx *ctx);    // in-adjacency: edges sorted 
 percis_status transpose_finish(percis_ctx *ctx);  // in-adjacency: offsets (valid columns)
 
 // prep.cu
+percis_status ensure_aux(percis_ctx *ctx);  // the second stream and its events
 percis_status prep_graph(percis_ctx *ctx);  // transpose (directed), validation, VertexDiamUB
 percis_status prep_states(percis_ctx *ctx);  // sort, tables, C_v, lambda, d^
 percis_status prep_lambda(percis_ctx *ctx, double *lam);  // lambda_v of every vertex (device)

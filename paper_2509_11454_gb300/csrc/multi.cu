@@ -161,10 +161,17 @@ percis_status multi_sample_pairs(percis_ctx *ctx, uint64_t seed, uint32_t tag) {
     key.push_back((int64_t)(uintptr_t)m->soff_dev.p);
     if (!m->samp_exec[k] || m->samp_key[k] != key) {
         drop_graph(m, k);
+        // on the second stream: the context's own may wait for the legacy default stream, whose
+        // use by another thread would then break the capture
+        PERCIS_TRY(ensure_aux(ctx));
         cudaGraph_t graph = nullptr;
-        PERCIS_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-        const percis_status st = issue(m->seed_dev.as<uint64_t>());
-        const cudaError_t ec = cudaStreamEndCapture(ctx->stream, &graph);
+        PERCIS_CUDA(ctx, cudaStreamBeginCapture(ctx->aux, cudaStreamCaptureModeThreadLocal));
+        percis_status st;
+        {
+            AuxScope scope(ctx);
+            st = issue(m->seed_dev.as<uint64_t>());
+        }
+        const cudaError_t ec = cudaStreamEndCapture(ctx->aux, &graph);
         if (st != PERCIS_OK) {
             if (graph) cudaGraphDestroy(graph);
             return st;

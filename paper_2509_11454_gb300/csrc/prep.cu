@@ -883,6 +883,13 @@ percis_status prep_vorder(percis_ctx *ctx) {
     return PERCIS_OK;
 }
 
+percis_status ensure_aux(percis_ctx *ctx) {
+    if (!ctx->aux_go) PERCIS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->aux_go, cudaEventDisableTiming));
+    if (!ctx->graph_ready) PERCIS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->graph_ready, cudaEventDisableTiming));
+    if (!ctx->aux) PERCIS_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking));
+    return PERCIS_OK;
+}
+
 percis_status prep_graph(percis_ctx *ctx) {
     const int64_t n = ctx->n, nnz = ctx->nnz;
     PERCIS_TRY(ensure(ctx, ctx->status, 64, "status"));
@@ -908,11 +915,7 @@ percis_status prep_graph(percis_ctx *ctx) {
         // here; the sort's digits are masked, so it reads and writes in bounds whatever
         // the columns hold.  Its last step (the offsets, indexed by column) waits for the
         // check.  The states can be prepared on this stream meanwhile.
-        if (!ctx->aux) {
-            PERCIS_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking));
-            PERCIS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->aux_go, cudaEventDisableTiming));
-            PERCIS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->graph_ready, cudaEventDisableTiming));
-        }
+        PERCIS_TRY(ensure_aux(ctx));
         PERCIS_CUDA(ctx, cudaEventRecord(ctx->aux_go, ctx->stream));
         PERCIS_CUDA(ctx, cudaStreamWaitEvent(ctx->aux, ctx->aux_go, 0));
     }

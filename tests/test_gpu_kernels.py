@@ -518,3 +518,30 @@ def test_batched_needed_counts_past_their_list(binding, n, diamond, lanes):
         assert np.array_equal(_np(ph[k]), getattr(ref, k)), k
     assert np.array_equal(nodes, ref.path_nodes) and ref.ilen.sum() > 100 * n
     eng.close()
+
+
+def test_work_queued_by_torch_is_waited_for(binding):
+    """On torch's default stream, beside which the context has a stream of its own: states
+    and gradients that are still being made, and an output buffer still being written, are
+    waited for (each behind about 10 ms of other work)."""
+    g = synth.barabasi_albert(500, 3, 1)
+    x = torch.as_tensor(synth.states_uniform(g.n, 1), device="cuda")
+    grad = torch.as_tensor(np.random.default_rng(2).standard_normal(g.n), device="cuda")
+    eng = _engine(binding, g, x)
+    pc = eng.estimate(0.1, 0.1, 3)[0].clone()
+    gx = eng.backward(grad).clone()
+    torch.cuda.synchronize()
+
+    def late(value):
+        buf = torch.full_like(value, 0.25)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(20_000_000)
+        return buf.copy_(value)
+
+    eng.set_states(late(x))
+    assert torch.equal(eng.prep()["xs"], torch.sort(x, descending=True).values)
+    out = late(x)
+    assert torch.equal(eng.estimate(0.1, 0.1, 3, out=out)[0], pc)
+    got = eng.backward(late(grad))
+    assert torch.linalg.norm(got - gx) <= 1e-10 * torch.linalg.norm(gx)
+    eng.close()

@@ -300,3 +300,38 @@ def test_phases_without_an_estimate(binding, form, count):
         if b > a:
             want = oracle.vjp_fixed(prep, b - a, ref, prep.lam * ref.cnt / (b - a), gvec[lo:hi])
             assert np.linalg.norm(gx[lo:hi] - want) <= 1e-10 * max(np.linalg.norm(want), 1e-300), g
+
+
+def test_sampling_recorded_beside_the_default_stream(binding):
+    """The sampling launch is recorded while another thread keeps the default stream busy,
+    which the context's own stream waits for: the same estimates as without recording."""
+    import threading
+
+    graphs = synth.graph_batch([60, 90, 40], 3)
+    vptr, rp, col = synth.union_csr(graphs)
+    x = synth.states_uniform(int(vptr[-1]), 1)
+    stop = threading.Event()
+
+    def work():
+        a = torch.zeros(1 << 16, device="cuda")
+        while not stop.is_set():
+            a.add_(1.0)
+
+    thread = threading.Thread(target=work)
+    thread.start()
+    try:
+        pcs = []
+        for graphs_on in (0, 1):
+            eng = binding.PercIS(0)
+            eng.set_options(form="bidir", cuda_graphs=graphs_on)
+            eng.load_graphs(vptr, rp, col)
+            eng.set_states(x)
+            for ell in (100, 120, 140, 160):  # (a new recording each)
+                eng.set_options(ell1=ell, ell=ell)
+                pcs.append(eng.estimate_graphs(0.1, 0.1, seed=5)[0].cpu().numpy())
+            eng.close()
+    finally:
+        stop.set()
+        thread.join()
+    for a, b in zip(pcs[:4], pcs[4:]):
+        assert np.array_equal(a, b)
