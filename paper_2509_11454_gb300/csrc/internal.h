@@ -230,6 +230,7 @@ percis_status radix_sort_u64(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uin
 // the states' sort (see radix.cu): it changes buffers state_sort_swaps times (an odd number
 // leaves the result in tk / tv); *status and *nheads are zeroed device words
 int state_sort_swaps(int64_t n, bool full);
+bool state_sort_may_repeat(int64_t n, bool full);  // (may set DEV_LONG_RUN)
 percis_status sort_states(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uint64_t *tk, int32_t *tv, int64_t n,
                           bool full, uint32_t *status, uint64_t *nheads);
 percis_status transpose_sort(percis_ctx *ctx);    // in-adjacency: edges sorted by target (valid row_ptr)

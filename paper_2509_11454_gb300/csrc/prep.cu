@@ -734,7 +734,8 @@ __device__ bool grid_running_sum(const double *src, int64_t soff, double *dst, i
 __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64_t n, double *w, double *ci,
                                                          double *r, double *dscal, TableCtl *ctl,
                                                          uint64_t budget_ns, const uint32_t *sort_status) {
-    if (__ldcg(sort_status) & DEV_LONG_RUN) return;  // (the same in every thread: nothing writes it here)
+    // (null where the sort cannot leave one; the same in every thread: nothing writes it here)
+    if (sort_status && (__ldcg(sort_status) & DEV_LONG_RUN)) return;
     // positions past the last non-zero state: x_i = 0 and every sum before them
     // is +0, so w_i = c_i = r_i = 0 exactly; the scans start at the last non-zero one
     const int64_t nz = *reinterpret_cast<const long long *>(dscal + 2);
@@ -761,8 +762,8 @@ __global__ void __launch_bounds__(kScanThreads) k_tables(const double *xs, int64
 // a phase counted): a division for every vertex was most of this kernel's FP64 work,
 // and max_v lambda_v = c / min_v C_v (the rounded division is monotone).
 __global__ void k_cv(const double *xs, const int32_t *perm, const double *w, double *dscal, int64_t n, double *Cv,
-                     uint32_t *status) {
-    if (ld_relaxed_u32(status) & DEV_LONG_RUN) return;  // (set before this launch, if at all)
+                     uint32_t *status, const uint32_t *sort_status) {
+    if (sort_status && (ld_relaxed_u32(sort_status) & DEV_LONG_RUN)) return;  // (set before this launch, if at all)
     const double c = dscal[0];
     const double w1 = w[1];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1010,12 +1011,12 @@ static percis_status prep_states_once(percis_ctx *ctx, bool full_sort, bool *aga
     TableCtl *tctl = ctx->table_ctl.as<TableCtl>();
     uint64_t budget = (uint64_t)(ctx->opt.timeout_s * 1e9);
     int64_t nn = n;
-    const uint32_t *sst = st;
+    const uint32_t *sst = state_sort_may_repeat(n, full_sort) ? st : nullptr;
     void *args[] = {&xs, &nn, &w, &ci, &r, &dscal, &tctl, &budget, &sst};
     PERCIS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_tables, dim3(G), dim3(kScanThreads), args, 0,
                                                  ctx->stream));
     ctx->launches++;
-    k_cv<<<g, 256, 0, ctx->stream>>>(xs, perm, w, dscal, n, ctx->Cv.as<double>(), st);
+    k_cv<<<g, 256, 0, ctx->stream>>>(xs, perm, w, dscal, n, ctx->Cv.as<double>(), st, sst);
     PERCIS_CHECK_LAUNCH(ctx, "C_v");
     ctx->groups_ready = false;  // built by the first backward pass that needs them
     struct Back {

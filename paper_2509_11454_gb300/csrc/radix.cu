@@ -424,6 +424,8 @@ percis_status radix_sort_u64(percis_ctx *ctx, uint64_t *keys, int32_t *vals, uin
 // all eight passes.  1.5M states: 327 us of kernels with eight passes, 218 us; their whole
 // preparation 458 us, where a quarter of them (a saturated sigmoid) or all lie within 2^-28
 // of one another 866 and 862 us.
+bool state_sort_may_repeat(int64_t n, bool full) { return n > kMergeMaxN && !full; }
+
 int state_sort_swaps(int64_t n, bool full) {
     if (n > kMergeMaxN) return full ? 8 : (64 - kFixBits) / 8;
     int k = 0;
